@@ -24,6 +24,14 @@
 #define JK_BOYS_TMAX 36.0
 #define JK_BOYS_NPTS (36 * 32 + 2)
 #define JK_BOYS_MCOL (JK_MAXLQ + 8)
+// Taylor rows of the FP64 seeds (md.cuh, boys_attenuated_tab): JK_TROW doubles
+// per point u_k = k / JK_BOYS_INV_STEP, the first eight the Taylor
+// coefficients, the ninth e^{-u_k}.  Slices 0 .. JK_MAXLQ hold F_L, slice
+// JK_MAXLQ + 1 holds H_0(u) = int_1^inf e^{-u t^2} dt; every slice has
+// JK_TPTS points (u up to JK_TMAX, H and e^{-u} are negligible above).
+#define JK_TROW 10
+#define JK_TMAX 64.0
+#define JK_TPTS (64 * 32 + 2)
 
 struct ShellRec {
     double c[3];
@@ -92,6 +100,7 @@ struct PlanDev {
     const int *spi_order;        // spi indices grouped by shell pair (for the reciprocal build)
     const double *boys;          // [JK_BOYS_NPTS][JK_BOYS_MCOL]
     const float *boys_f;
+    const double *boys_t;        // [JK_MAXLQ + 2][JK_TPTS][JK_TROW] Taylor rows of F_L and H_0
     const PpiF *ppf;
     const float *ppB;            // B = |K| p^{-5/4} of each primitive pair (descending inside an image)
     float mag_thr;               // B_i B_j below this: the primitive quartet is below the real-space threshold

@@ -69,13 +69,12 @@ struct Acc<float> {
 };
 
 // Attenuated seeds s_m = (-2 alpha)^m F_m(alpha X^2) - c_w (-2 alpha_w)^m F_m(alpha_w X^2)
-// = (-2 alpha)^m G_m(alpha X^2, c_w)  (see boys_attenuated).
+// = (-2 alpha)^m G_m(alpha X^2, c_w)  (see boys_attenuated_tab, boys_attenuated).
 template <int L>
 __device__ __forceinline__ void seeds(double x2, double alpha, double aw, double cw, const PlanDev &pl, double *s)
 {
-    (void)aw;
     double G[L + 1];
-    boys_attenuated<L, double>(alpha * x2, cw, pl.boys, G);
+    boys_attenuated_tab<L>(alpha * x2, aw * x2, cw, pl.boys_t, G);
     double f = 1.0;
 #pragma unroll
     for (int m = 0; m <= L; ++m) {

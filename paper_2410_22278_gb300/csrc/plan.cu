@@ -272,6 +272,36 @@ void boys_table(int ncol, int npts, double inv_step, std::vector<double> &out)
     }
 }
 
+// Taylor rows of the FP64 seeds (layout: JK_TROW in jk_internal.h): F_{L+j}/j!
+// from the Boys table, and H_j/j! with H_0(u) = (sqrt(pi)/2) erfc(sqrt u) /
+// sqrt u and H_{m+1} = ((2m+1) H_m + e^{-u}) / 2u (all terms positive), in
+// long double.  The tables are the same for every plan and are made once.
+const std::vector<double> &taylor_rows()
+{
+    static const std::vector<double> rows = [] {
+        const int nsl = JK_MAXLQ + 2;
+        std::vector<double> F, out((size_t)nsl * JK_TPTS * JK_TROW, 0.0);
+        boys_table(JK_MAXLQ + 8, JK_TPTS, JK_BOYS_INV_STEP, F);
+        for (int k = 0; k < JK_TPTS; ++k) {
+            const long double u = (long double)k / JK_BOYS_INV_STEP, e = expl(-u);
+            for (int L = 0; L < nsl; ++L) out[((size_t)L * JK_TPTS + k) * JK_TROW + 8] = (double)e;
+            long double fac = 1.0L;
+            long double h = k > 0 ? 0.886226925452758013649083741670573L * erfcl(sqrtl(u)) / sqrtl(u) : 0.0L;
+            for (int j = 0; j < 8; ++j) {
+                if (j > 0) fac *= j;
+                for (int L = 0; L <= JK_MAXLQ; ++L)
+                    out[((size_t)L * JK_TPTS + k) * JK_TROW + j] = (double)((long double)F[(size_t)k * (JK_MAXLQ + 8) + L + j] / fac);
+                if (k > 0) {
+                    out[((size_t)(JK_MAXLQ + 1) * JK_TPTS + k) * JK_TROW + j] = (double)(h / fac);
+                    h = ((2 * j + 1) * h + e) / (2.0L * u);
+                }
+            }
+        }
+        return out;
+    }();
+    return rows;
+}
+
 // Squared real-space radius for one primitive quartet: Eq.
 // pbc_eri_real_cutoff_implementation, widened for the Hermite polynomial
 // growth (2 alpha_w |X|)^L that the s-type derivation leaves out.  Returns
@@ -307,6 +337,7 @@ PlanDev Plan::dev() const
     d.spi_order = d_spi_order;
     d.boys = d_boys;
     d.boys_f = d_boys_f;
+    d.boys_t = d_boys_t;
     d.r1 = d_r1;
     d.ppf = d_ppf;
     d.r1f = d_r1f;
@@ -979,6 +1010,7 @@ int finish_plan_device(Plan *P)
     boys_table(JK_BOYS_MCOL, JK_BOYS_NPTS, JK_BOYS_INV_STEP, tab);
     std::vector<float> tabf(tab.begin(), tab.end());
     if ((rc = upload(tab, &P->d_boys, b)) || (rc = upload(tabf, &P->d_boys_f, b))) return rc;
+    if ((rc = upload(taylor_rows(), &P->d_boys_t, b))) return rc;
     std::vector<double> g0 = {0.0, 0.0, 0.0, 1.0};
     if ((rc = upload(g0, &P->d_g0, b))) return rc;
     {
@@ -1073,7 +1105,7 @@ void destroy_plan(Plan *P)
     if (!P) return;
     cudaSetDevice(P->device);
     release_cache(P);
-    void *ptrs[] = {P->d_shells, P->d_spi, P->d_ppi, P->d_ppf, P->d_ppB, P->d_r1f, P->d_spair, P->d_spi_order, P->d_boys, P->d_boys_f, P->d_r1, P->d_gvec,
+    void *ptrs[] = {P->d_shells, P->d_spi, P->d_ppi, P->d_ppf, P->d_ppB, P->d_r1f, P->d_spair, P->d_spi_order, P->d_boys, P->d_boys_f, P->d_boys_t, P->d_r1, P->d_gvec,
                     P->d_g0, P->d_compf, P->d_ppi_ab, P->d_kblk, P->d_kblk2, P->d_pvals, P->d_gtab0, P->d_ppi_pidx, P->d_phase, P->d_ppdf, P->d_gdf, P->d_phasef, P->ws.gtab, P->ws.gtab2, P->d_S, P->ws.Dp, P->ws.X, P->ws.Y, P->ws.JLR, P->ws.KLR, P->ws.T1, P->ws.T2,
                     P->ws.M, P->ws.Z, P->ws.rho, P->ws.rho_part, P->ws.DhD, P->ws.JH, P->ws.DhF, P->ws.dmax, P->ws.scal, P->ws.err, P->ws.cnt, P->ws.big, P->ws.nbig,
                     P->ws.Ms, P->ws.Zs, P->ws.Ds, P->ws.Mex, P->ws.Zex, P->ws.Dex, P->ws.Dpf, P->ws.dmaxf, P->ws.Cs, P->ws.Cex, P->ws.Kpart,

@@ -150,6 +150,7 @@ struct Plan {
     int *d_spi_order = nullptr;
     double *d_boys = nullptr;
     float *d_boys_f = nullptr;
+    double *d_boys_t = nullptr;  // Taylor rows of the FP64 seeds
     double *d_r1 = nullptr;
     double *d_gvec = nullptr;
     double *d_g0 = nullptr;  // one G = 0 entry with unit weight (overlap)
@@ -201,6 +202,7 @@ int energy_noalloc(const Plan *P, const double *D, const double *J, const double
 
 // host helpers shared by plan.cu and api.cu
 void boys_table(int ncol, int npts, double inv_step, std::vector<double> &out);
+const std::vector<double> &taylor_rows();
 double ewald_point_charges_host(const double *lat, int n, const double *q, const double *xyz, double omega, double delta);
 
 }  // namespace jk

@@ -86,11 +86,52 @@ __device__ __forceinline__ bool prim_reaches(const PlanDev &pl, const PpiF &bf, 
     return false;
 }
 
-// One primitive quartet (bra pair xb, ket pair xk): screening radius of Eq.
-// pbc_eri_real_cutoff_implementation (single precision), minimum image,
-// the R1 images inside the sphere, seeds and the Hermite R table, then the
-// contraction with both E tables into the Cartesian block V; the events go
-// to the lane's tally (flops.h).
+// Exact screening radius of one primitive quartet (Eq.
+// pbc_eri_real_cutoff_implementation, single precision); false when the
+// quartet has no term above the threshold.
+template <int L>
+__device__ __forceinline__ bool prim_radius(const PlanDev &pl, const PpiF &bf, const PpiF &kf, float &r)
+{
+    const float ipf = bf.pad, iqf = kf.pad;
+    const float awf = frcp_fast(ipf + iqf + pl.inv_omega2f);
+    const float cwf = fsqrt_fast(awf * (ipf + iqf));
+    const float preff = 34.986836655249725f * bf.K * kf.K * ipf * iqf * rsqrtf(bf.p + kf.p);
+    const float lg = __logf(fabsf(preff) * (1.0f - cwf)) - pl.log_ewald_R;
+    if (!(lg > 0.0f)) return false;
+    r = fsqrt_fast(fdiv_fast(lg, awf));
+    if (L > 0) {
+        r = fsqrt_fast(fdiv_fast(lg + L * __logf(1.0f + 2.0f * awf * r), awf));
+        r = fsqrt_fast(fdiv_fast(lg + L * __logf(1.0f + 2.0f * awf * r), awf));
+        r += 0.5f + 0.25f * L;  // the Gaussian bound is derived for s functions; widen for L > 0
+    }
+    return true;
+}
+
+// alpha = 1/(1/p + 1/q), alpha_w = 1/(1/p + 1/q + 1/w^2), c_w = sqrt(alpha_w / alpha).
+// FP64: one reciprocal square root instead of two divisions and a square
+// root (about 12 FP64 instructions against 30; within 3 ulp).
+__device__ __forceinline__ void alphas(double ipq, double iw2, double &alpha, double &aw, double &cw)
+{
+    const double b = ipq + iw2, y = rsqrt(ipq * b), t = y * y;
+    alpha = t * b;
+    aw = t * ipq;
+    cw = ipq * y;
+}
+__device__ __forceinline__ void alphas(float ipq, float iw2, float &alpha, float &aw, float &cw)
+{
+    aw = 1.0f / (ipq + iw2);
+    alpha = 1.0f / ipq;
+    cw = sqrtf(aw * ipq);
+}
+
+// One primitive quartet (bra pair b, ket pair k): screening radius, minimum
+// image, the R1 images inside the sphere, seeds and the Hermite R table, then
+// the contraction with both E tables into the Cartesian block V; the events
+// go to the lane's tally (flops.h).  The image search runs in single
+// precision (it only decides which terms are formed) and each lane walks on
+// to its next image inside the sphere before the terms are formed, so the
+// lanes of a warp form them together; with the test and the term in one loop
+// body the lanes whose candidate failed waited for the others.
 template <int LA, int LB, int LC, int LD, typename T>
 __device__ __forceinline__ void prim_term(const PlanDev &pl, const PrimE<LA, LB, T> &b, const PpiF &bf, const PrimE<LC, LD, T> &k,
                                           const PpiF &kf, T *V, Tally &tl)
@@ -98,49 +139,50 @@ __device__ __forceinline__ void prim_term(const PlanDev &pl, const PrimE<LA, LB,
     constexpr int NA = ncart(LA), NB = ncart(LB), NC = ncart(LC), ND = ncart(LD);
     constexpr int L = LA + LB + LC + LD, LAB = LA + LB, LCD = LC + LD;
     constexpr int NTA = LAB + 1, NTC = LCD + 1, D = L + 1;
-    const float iw2 = pl.inv_omega2f;
-    const float ipf = bf.pad, iqf = kf.pad;
-    const float awf = frcp_fast(ipf + iqf + iw2);
-    const float cwf = fsqrt_fast(awf * (ipf + iqf));
-    const float preff = 34.986836655249725f * bf.K * kf.K * ipf * iqf * rsqrtf(bf.p + kf.p);
     ++tl.screen;
-    const float lg = __logf(fabsf(preff) * (1.0f - cwf)) - pl.log_ewald_R;
-    if (!(lg > 0.0f)) return;
-    float r = fsqrt_fast(fdiv_fast(lg, awf));
-    if (L > 0) {
-        r = fsqrt_fast(fdiv_fast(lg + L * __logf(1.0f + 2.0f * awf * r), awf));
-        r = fsqrt_fast(fdiv_fast(lg + L * __logf(1.0f + 2.0f * awf * r), awf));
-        r += 0.5f + 0.25f * L;  // the Gaussian bound is derived for s functions; widen for L > 0
-    }
+    float r;
+    if (!prim_radius<L>(pl, bf, kf, r)) return;
+    ++tl.radius;
     const float r2 = r * r;
     const PairT<T> &x = b.x, &y = k.x;
+    float F0[3] = {bf.P[0] - kf.P[0], bf.P[1] - kf.P[1], bf.P[2] - kf.P[2]}, f[3];
     T X0[3] = {x.P[0] - y.P[0], x.P[1] - y.P[1], x.P[2] - y.P[2]};
-    {
-        T f[3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a)
-            f[a] = rint(latc(pl.Finv, pl.Finvf, 3 * a, T(0)) * X0[0] + latc(pl.Finv, pl.Finvf, 3 * a + 1, T(0)) * X0[1] +
-                        latc(pl.Finv, pl.Finvf, 3 * a + 2, T(0)) * X0[2]);
+    for (int a = 0; a < 3; ++a) f[a] = rintf(pl.Finvf[3 * a] * F0[0] + pl.Finvf[3 * a + 1] * F0[1] + pl.Finvf[3 * a + 2] * F0[2]);
+    if (f[0] != 0.0f || f[1] != 0.0f || f[2] != 0.0f) {
 #pragma unroll
-        for (int a = 0; a < 3; ++a)
-            X0[a] -= f[0] * latc(pl.L, pl.Lf, a, T(0)) + f[1] * latc(pl.L, pl.Lf, 3 + a, T(0)) + f[2] * latc(pl.L, pl.Lf, 6 + a, T(0));
+        for (int a = 0; a < 3; ++a) {
+            F0[a] -= f[0] * pl.Lf[a] + f[1] * pl.Lf[3 + a] + f[2] * pl.Lf[6 + a];
+            X0[a] -= T(f[0]) * latc(pl.L, pl.Lf, a, T(0)) + T(f[1]) * latc(pl.L, pl.Lf, 3 + a, T(0)) + T(f[2]) * latc(pl.L, pl.Lf, 6 + a, T(0));
+        }
     }
-    ++tl.radius;
-    const float x0n = fsqrt_fast((float)(X0[0] * X0[0] + X0[1] * X0[1] + X0[2] * X0[2]));
+    const float x0n = fsqrt_fast(F0[0] * F0[0] + F0[1] * F0[1] + F0[2] * F0[2]);
     T Rs[D * D * D];
 #pragma unroll
     for (int q = 0; q < D * D * D; ++q) Rs[q] = T(0);
     bool any = false;
     const T ip = x.ip, iq = y.ip;
-    const T aw = T(1) / (ip + iq + latc(&pl.inv_omega2, &pl.inv_omega2f, 0, T(0)));
-    const T alpha = T(1) / (ip + iq);
-    const T cw = sqrt(aw * (ip + iq));
-    for (int c = 0; c < pl.nr1; ++c) {
-        if (pl.r1f[4 * c + 3] - x0n >= r) break;
+    T alpha, aw, cw;
+    alphas(ip + iq, latc(&pl.inv_omega2, &pl.inv_omega2f, 0, T(0)), alpha, aw, cw);
+    const float4 *lat = reinterpret_cast<const float4 *>(pl.r1f);
+    int c = 0;
+    while (true) {
+        bool hit = false;
+        while (c < pl.nr1) {
+            const float4 R = __ldg(lat + c);
+            if (R.w - x0n >= r) break;
+            ++tl.cand;
+            const float fx = F0[0] - R.x, fy = F0[1] - R.y, fz = F0[2] - R.z;
+            if (fx * fx + fy * fy + fz * fz < r2) {
+                hit = true;
+                break;
+            }
+            ++c;
+        }
+        if (!hit) break;
         const T Xx = X0[0] - lat_at(pl, 4 * c, T(0)), Xy = X0[1] - lat_at(pl, 4 * c + 1, T(0)), Xz = X0[2] - lat_at(pl, 4 * c + 2, T(0));
         const T x2 = Xx * Xx + Xy * Xy + Xz * Xz;
-        ++tl.cand;
-        if ((float)x2 >= r2) continue;
+        ++c;
         any = true;
         ++tl.img;
         T s[L + 1];
