@@ -239,6 +239,42 @@ static void launch_hermite(int cls, bool back, const PlanDev &pl, int b0, int b1
     }
 }
 
+// The warps of a warp-per-bra launch over the bras [b0, b1) and kets [k0, k1)
+// (TileMap).  kchunk is the mean number of kets of a warp: a warp gets the
+// work of kchunk kets of the mean primitive count with a bra of the mean one.
+// Images are in descending order of primitive count inside a class, so a
+// range of bras of similar count is contiguous; a new range starts where the
+// count has fallen by a quarter.
+static TileMap tile_map(const Plan *P, int b0, int b1, int k0, int k1, int kchunk)
+{
+    TileMap m{};
+    if (b1 <= b0 || k1 <= k0) return m;
+    const auto prims = [&](int i0, int i1) {
+        return (double)(P->spi[i1 - 1].pp0 + P->spi[i1 - 1].npp - P->spi[i0].pp0);
+    };
+    const double pk = prims(k0, k1);
+    double work = (double)kchunk * (prims(b0, b1) / (b1 - b0)) * (pk / (k1 - k0));
+    // at most 2^28 warps (blockIdx.x); only a hand-set schedule gets there
+    work = std::max(work, prims(b0, b1) * pk / (double)(1 << 28));
+    for (int b = b0; b < b1;) {
+        const int top = P->spi[b].npp;
+        int e = b1;
+        if (m.n < 7)  // the eighth range takes what is left
+            e = (int)(std::partition_point(P->spi.begin() + b, P->spi.begin() + b1, [&](const SpiRec &s) { return 4 * s.npp > 3 * top; }) -
+                      P->spi.begin());
+        TileMap::Range &g = m.g[m.n];
+        g.b0 = b;
+        g.b1 = e;
+        g.W = (int)std::min(pk, std::max(1.0, work / top));
+        g.nch = (int)((pk + g.W - 1) / g.W);
+        g.first = m.items;
+        m.items += (long long)(e - b) * g.nch;
+        ++m.n;
+        b = e;
+    }
+    return m;
+}
+
 static int cuda_check(const char *what)
 {
     cudaError_t e = cudaGetLastError();
@@ -459,6 +495,7 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
             a.k1 = Kc.b1;
             a.same = cb == ck;
             a.kchunk = P->kchunk[cb][ck];
+            a.map = tile_map(P, a.b0, a.b1, a.k0, a.k1, a.kchunk);
             a.variant = P->kvariant[cb][ck];
             a.tau = P->mixed_tau;
             a.Dp = w.Dp;
@@ -476,10 +513,9 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
             // shell on both sides, where the Hermite contraction is smaller
             // than the Cartesian block (measured: for s and p classes the
             // Cartesian kernels with the exchange digestion skipped are
-            // faster); its tiles are lane-per-bra: kets per tile as tuned for
-            // that family, else 32
+            // faster); its tiles are lane-per-bra, 32 kets each
             const bool use_jeng = jeng && cb >= kJengClass && ck >= kJengClass;
-            if (use_jeng && a.variant != 0) a.kchunk = 32;
+            if (use_jeng) a.kchunk = 32;
             if (use_jeng && !mixed) {
                 a.mode = 0;
                 a.fp32 = false;
@@ -598,11 +634,12 @@ int autotune(Plan *P, const double *D, cudaStream_t st, const char *cache_path, 
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     float part_ms = 0;
-    // candidates (family, kets per tile): lane-per-bra kernels with 8 .. 128
-    // kets per tile, and for s and p class pairs the warp kernels with
+    // candidates (family, kets per tile): for s and p class pairs the
+    // lane-per-bra kernels with 8 .. 128 kets per tile, the warp kernels with
     // 128 .. 2048 kets per warp and the pair-queue kernels with 32 .. 512
-    // kets per tile; a choice is stored as family * 65536 + kets
-    std::vector<int> cands_t = {8, 16, 32, 64, 128}, cands_w;
+    // kets per tile; for class pairs with a d shell the warp kernels with 1
+    // .. 2048 kets per warp; a choice is stored as family * 65536 + kets
+    std::vector<int> cands_t = {8, 16, 32, 64, 128}, cands_w, cands_d = {1, 4, 16, 64, 128, 512, 2048};
     for (int c : {128, 256, 512, 1024, 2048}) cands_w.push_back(65536 + c);   // warp kernels
     for (int c : {32, 64, 128, 256, 512}) cands_w.push_back(2 * 65536 + c);   // pair-queue kernels
     int k = 0;
@@ -616,7 +653,7 @@ int autotune(Plan *P, const double *D, cudaStream_t st, const char *cache_path, 
             }
             if (B.b1 <= B.b0 || Kc.b1 <= Kc.b0) continue;
             char key[512];
-            snprintf(key, sizeof key, "%s|%s|v3|%d%d|%d|%d", prop.name, mixed ? "mixed" : "fp64", cb, ck, bucket(B.b1 - B.b0),
+            snprintf(key, sizeof key, "%s|%s|v4|%d%d|%d|%d", prop.name, mixed ? "mixed" : "fp64", cb, ck, bucket(B.b1 - B.b0),
                      bucket(Kc.b1 - Kc.b0));
             for (char *q = key; *q; ++q)
                 if (*q == ' ') *q = '_';
@@ -626,7 +663,7 @@ int autotune(Plan *P, const double *D, cudaStream_t st, const char *cache_path, 
                 best = it->second;
             } else {
                 float best_ms = 1e30f;
-                std::vector<int> cands = cands_t;
+                std::vector<int> cands = real_has_warp_kernel(cb, ck) ? cands_t : cands_d;
                 if (real_has_warp_kernel(cb, ck)) cands.insert(cands.end(), cands_w.begin(), cands_w.end());
                 // two sub-ranges of at most 2048 bras (the class is sorted by
                 // primitive count, so the start and the middle differ)
@@ -642,6 +679,7 @@ int autotune(Plan *P, const double *D, cudaStream_t st, const char *cache_path, 
                         a.k1 = Kc.b1;
                         a.same = cb == ck;
                         a.kchunk = c & 65535;
+                        a.map = tile_map(P, a.b0, a.b1, a.k0, a.k1, a.kchunk);
                         a.variant = c >> 16;
                         a.mode = 0;
                         a.fp32 = mixed;

@@ -103,6 +103,9 @@ struct PlanDev {
     const double *boys_t;        // [JK_MAXLQ + 2][JK_TPTS][JK_TROW] Taylor rows of F_L and H_0
     const PpiF *ppf;
     const float *ppB;            // B = |K| p^{-5/4} of each primitive pair (descending inside an image)
+    const float4 *pps;           // (P, 1/p) of each primitive pair and ln B (rounded up): the screening of real2.cuh
+    const float *pplb;
+    float lb_max;                // largest ln B
     float mag_thr;               // B_i B_j below this: the primitive quartet is below the real-space threshold
     const double *r1;            // [nr1][4]: x, y, z, |R|, sorted by |R|
     const float *r1f;            // the same in single precision
@@ -124,5 +127,5 @@ struct PlanDev {
     float log_ewald_R;           // ln of the per-term threshold used inside the real-space sums
     double volume;
     float hplane[3];             // spacing of the lattice planes of each fractional coordinate
-    int orth;                    // lattice vectors mutually orthogonal: rounding f gives the minimum image
+    int orth;                    // lattice vectors mutually orthogonal: rounding f gives the minimum image; 2: along the axes
 };

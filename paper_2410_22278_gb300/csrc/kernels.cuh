@@ -384,8 +384,10 @@ __device__ __forceinline__ float quartet_estimate(const PlanDev &pl, const SpiRe
     const float d = fmaxf(0.0f, fsqrt_fast(X[0] * X[0] + X[1] * X[1] + X[2] * X[2]) - sb.ext - sk.ext);
     const float d2 = d * d, iw2 = pl.inv_omega2f;
     float est = 0.0f;
+#pragma unroll 1
     for (int i = 0; i < sb.npp; ++i) {
         const PpiF x = pl.ppf[sb.pp0 + i];
+#pragma unroll 1
         for (int j = 0; j < sk.npp; ++j) {
             const PpiF y = pl.ppf[sk.pp0 + j];
             const float aw = frcp_fast(x.pad + y.pad + iw2);
@@ -423,7 +425,7 @@ __device__ __forceinline__ float quartet_estimate_bound(const PlanDev &pl, const
 // mode 0: every quartet in this kernel's precision.  mode 2 (mixed
 // precision, T = float): quartets whose density-weighted size estimate is
 // >= tau are appended to the compact list `big` (processed afterwards in
-// FP64 by k_real_list) instead of being evaluated here; if the list is full
+// FP64 by the list pass) instead of being evaluated here; if the list is full
 // the quartet is evaluated here and counted in ovf.  *cnt counts the image
 // quartets this launch evaluated.
 template <int LA, int LB, int LC, int LD, typename T>
@@ -575,113 +577,6 @@ __global__ void __launch_bounds__(kRealThreads) k_real(PlanDev pl, int b0, int b
     // warp-aggregated counts of the image quartets this launch evaluated and
     // of their algorithmic flops (cnt[4])
     unsigned tot = nq;
-    unsigned long long fl = tally_alg<LA, LB, LC, LD>(tl), fs = tally_screen<LA, LB, LC, LD>(tl);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        tot += __shfl_xor_sync(0xffffffffu, tot, o);
-        fl += __shfl_xor_sync(0xffffffffu, fl, o);
-        fs += __shfl_xor_sync(0xffffffffu, fs, o);
-    }
-    if ((threadIdx.x & 31) == 0 && tot) atomicAdd(cnt, (unsigned long long)tot);
-    if ((threadIdx.x & 31) == 0 && fl) atomicAdd(cnt + 4, fl);
-    if ((threadIdx.x & 31) == 0 && fs) atomicAdd(cnt + 8, fs);
-}
-
-// FP64 pass over the compact list of large quartets collected by the
-// mixed-precision kernel of the same class pair (grid-stride; each entry is
-// one unique pair of images, digested with the same orbit weights).
-template <int LA, int LB, int LC, int LD>
-__global__ void __launch_bounds__(kRealThreads) k_real_list(PlanDev pl, const int2 *__restrict__ big, const unsigned *__restrict__ nbig,
-                                                             unsigned cap, int same, const double *__restrict__ Dp, double *__restrict__ X,
-                                                             double *__restrict__ Y, unsigned long long *__restrict__ cnt)
-{
-    constexpr int NA = ncart(LA), NB = ncart(LB), NC = ncart(LC), ND = ncart(LD);
-    constexpr int DUNR = LA + LB + LC + LD >= 6 ? 1 : 64;
-    const unsigned total = min(*nbig, cap);
-    const int n = pl.nbf;
-    unsigned done = 0;
-    Tally tl;
-    for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
-        const int2 q = big[e];
-        const SpiRec sb = pl.spi[q.x], sk = pl.spi[q.y];
-        double V[NA * NB * NC * ND];
-#pragma unroll
-        for (int k = 0; k < NA * NB * NC * ND; ++k) V[k] = 0.0;
-        quartet_block<LA, LB, LC, LD, double>(pl, sb, sk, V, tl);
-        ++tl.quart;
-        ++done;
-        const double w = double(sb.w) * double(sk.w) * ((same && q.x == q.y) ? 0.5 : 1.0);
-        const int aoI = pl.shells[sb.I].ao, aoJ = pl.shells[sb.J].ao, aoK = pl.shells[sk.I].ao, aoL = pl.shells[sk.J].ao;
-        auto Dd = [&](int r, int c) { return __ldg(Dp + (size_t)r * n + c); };
-#pragma unroll DUNR
-        for (int a = 0; a < NA; ++a)
-#pragma unroll DUNR
-            for (int b = 0; b < NB; ++b) {
-                double s = 0;
-#pragma unroll
-                for (int c = 0; c < NC; ++c)
-#pragma unroll
-                    for (int d = 0; d < ND; ++d) s += V[((a * NB + b) * NC + c) * ND + d] * Dd(aoK + c, aoL + d);
-                atomicAdd(X + (size_t)(aoI + a) * n + aoJ + b, 2.0 * w * s);
-            }
-#pragma unroll DUNR
-        for (int c = 0; c < NC; ++c)
-#pragma unroll DUNR
-            for (int d = 0; d < ND; ++d) {
-                double s = 0;
-#pragma unroll
-                for (int a = 0; a < NA; ++a)
-#pragma unroll
-                    for (int b = 0; b < NB; ++b) s += V[((a * NB + b) * NC + c) * ND + d] * Dd(aoI + a, aoJ + b);
-                atomicAdd(X + (size_t)(aoK + c) * n + aoL + d, 2.0 * w * s);
-            }
-        if (!Y) continue;  // a Coulomb-only build
-#pragma unroll DUNR
-        for (int a = 0; a < NA; ++a)
-#pragma unroll DUNR
-            for (int d = 0; d < ND; ++d) {
-                double s = 0;
-#pragma unroll
-                for (int b = 0; b < NB; ++b)
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) s += V[((a * NB + b) * NC + c) * ND + d] * Dd(aoJ + b, aoK + c);
-                atomicAdd(Y + (size_t)(aoI + a) * n + aoL + d, w * s);
-            }
-#pragma unroll DUNR
-        for (int b = 0; b < NB; ++b)
-#pragma unroll DUNR
-            for (int d = 0; d < ND; ++d) {
-                double s = 0;
-#pragma unroll
-                for (int a = 0; a < NA; ++a)
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) s += V[((a * NB + b) * NC + c) * ND + d] * Dd(aoI + a, aoK + c);
-                atomicAdd(Y + (size_t)(aoJ + b) * n + aoL + d, w * s);
-            }
-#pragma unroll DUNR
-        for (int a = 0; a < NA; ++a)
-#pragma unroll DUNR
-            for (int c = 0; c < NC; ++c) {
-                double s = 0;
-#pragma unroll
-                for (int b = 0; b < NB; ++b)
-#pragma unroll
-                    for (int d = 0; d < ND; ++d) s += V[((a * NB + b) * NC + c) * ND + d] * Dd(aoJ + b, aoL + d);
-                atomicAdd(Y + (size_t)(aoI + a) * n + aoK + c, w * s);
-            }
-#pragma unroll DUNR
-        for (int b = 0; b < NB; ++b)
-#pragma unroll DUNR
-            for (int c = 0; c < NC; ++c) {
-                double s = 0;
-#pragma unroll
-                for (int a = 0; a < NA; ++a)
-#pragma unroll
-                    for (int d = 0; d < ND; ++d) s += V[((a * NB + b) * NC + c) * ND + d] * Dd(aoI + a, aoL + d);
-                atomicAdd(Y + (size_t)(aoJ + b) * n + aoK + c, w * s);
-            }
-    }
-    unsigned tot = done;
     unsigned long long fl = tally_alg<LA, LB, LC, LD>(tl), fs = tally_screen<LA, LB, LC, LD>(tl);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {

@@ -366,6 +366,9 @@ PlanDev Plan::dev() const
     d.log_ewald_R = (float)std::log(cut.ewald_R * 1e-1);
     // B_i B_j below this means 2 pi^{5/2} |K_i K_j| / (pq sqrt(p+q)) < delta/10
     d.ppB = d_ppB;
+    d.pps = d_pps;
+    d.pplb = d_pplb;
+    d.lb_max = lb_max;
     d.mag_thr = (float)(cut.ewald_R * 1e-1 / (24.739424126 * 1.001));
     d.volume = volume;
     for (int a = 0; a < 3; ++a)
@@ -378,6 +381,7 @@ PlanDev Plan::dev() const
             const double nb = std::sqrt(L[3 * b] * L[3 * b] + L[3 * b + 1] * L[3 * b + 1] + L[3 * b + 2] * L[3 * b + 2]);
             if (std::fabs(dot) > 1e-12 * na * nb) d.orth = 0;
         }
+    if (d.orth && L[1] == 0 && L[2] == 0 && L[3] == 0 && L[5] == 0 && L[6] == 0 && L[7] == 0) d.orth = 2;
     return d;
 }
 
@@ -525,9 +529,8 @@ int build_plan(const jk_cell *cell, const jk_shell *shells, int nshell, double o
     Plan *P = new Plan();
     for (int i = 0; i < JK_NCLASS_MAX; ++i)
         for (int j = 0; j < JK_NCLASS_MAX; ++j) {
-            // untuned: the warp kernels for s and p class pairs, 512 kets per warp
             P->kvariant[i][j] = (i <= 2 && j <= 2) ? 1 : 0;
-            P->kchunk[i][j] = (i <= 2 && j <= 2) ? 512 : 32;
+            P->kchunk[i][j] = 32;
         }
     P->device = device;
     P->precision = precision;
@@ -768,6 +771,19 @@ int build_plan(const jk_cell *cell, const jk_shell *shells, int nshell, double o
         if (cr.b1 <= cr.b0) cr.b0 = cr.b1 = 0;
         P->classes.push_back(cr);
     }
+    // untuned schedule: kets per warp for about a thousand warps per SM (half
+    // of them empty for a class with itself), at least 8 and at most 2048 --
+    // few enough that a small cell still fills the chip and the last warps do
+    // not hold up a launch, enough to fill the batches of a warp; the kernels that give an
+    // image quartet a whole warp (real3.cuh) have no batches and take 1 to 64
+    for (int i = 0; i < JK_NCLASS_MAX; ++i)
+        for (int j = i; j < JK_NCLASS_MAX; ++j) {
+            const ClassRange &B = P->classes[i], &K = P->classes[j];
+            const long long nb = B.b1 - B.b0, nk = K.b1 - K.b0;
+            const auto nc = [](int l) { return (l + 1) * (l + 2) / 2; };
+            const bool coop = nc(B.la) * nc(B.lb) * nc(K.la) * nc(K.lb) > 36;
+            P->kchunk[i][j] = (int)std::min(coop ? 64LL : 2048LL, std::max(coop ? 1LL : 8LL, nb * nk / (152 * 1024)));
+        }
     // ---- unique shell pairs with their images (reciprocal-space build), grouped by class
     {
         std::map<std::pair<int, int>, std::vector<int>> byp;
@@ -1003,8 +1019,18 @@ int finish_plan_device(Plan *P)
         std::vector<float> pB(P->ppi.size());
         for (size_t i = 0; i < P->ppi.size(); ++i)
             pB[i] = (float)(std::fabs(P->ppi[i].K) * std::pow(P->ppi[i].p, -1.25) * (1.0 + 1e-6));
+        std::vector<float4> ps(P->ppi.size());
+        std::vector<float> plb(P->ppi.size());
+        P->lb_max = -1e30f;
+        for (size_t i = 0; i < P->ppi.size(); ++i) {
+            ps[i] = make_float4(pf[i].P[0], pf[i].P[1], pf[i].P[2], pf[i].pad);
+            plb[i] = pB[i] > 0.0f ? std::log(pB[i]) + 1e-5f : -1e30f;
+            P->lb_max = std::max(P->lb_max, plb[i]);
+        }
         std::vector<float> r1f(P->r1.begin(), P->r1.end());
-        if ((rc = upload(pf, &P->d_ppf, b)) || (rc = upload(r1f, &P->d_r1f, b)) || (rc = upload(pB, &P->d_ppB, b))) return rc;
+        if ((rc = upload(pf, &P->d_ppf, b)) || (rc = upload(r1f, &P->d_r1f, b)) || (rc = upload(pB, &P->d_ppB, b)) ||
+            (rc = upload(ps, &P->d_pps, b)) || (rc = upload(plb, &P->d_pplb, b)))
+            return rc;
     }
     std::vector<double> tab;
     boys_table(JK_BOYS_MCOL, JK_BOYS_NPTS, JK_BOYS_INV_STEP, tab);
@@ -1105,7 +1131,7 @@ void destroy_plan(Plan *P)
     if (!P) return;
     cudaSetDevice(P->device);
     release_cache(P);
-    void *ptrs[] = {P->d_shells, P->d_spi, P->d_ppi, P->d_ppf, P->d_ppB, P->d_r1f, P->d_spair, P->d_spi_order, P->d_boys, P->d_boys_f, P->d_boys_t, P->d_r1, P->d_gvec,
+    void *ptrs[] = {P->d_shells, P->d_spi, P->d_ppi, P->d_ppf, P->d_ppB, P->d_pps, P->d_pplb, P->d_r1f, P->d_spair, P->d_spi_order, P->d_boys, P->d_boys_f, P->d_boys_t, P->d_r1, P->d_gvec,
                     P->d_g0, P->d_compf, P->d_ppi_ab, P->d_kblk, P->d_kblk2, P->d_pvals, P->d_gtab0, P->d_ppi_pidx, P->d_phase, P->d_ppdf, P->d_gdf, P->d_phasef, P->ws.gtab, P->ws.gtab2, P->d_S, P->ws.Dp, P->ws.X, P->ws.Y, P->ws.JLR, P->ws.KLR, P->ws.T1, P->ws.T2,
                     P->ws.M, P->ws.Z, P->ws.rho, P->ws.rho_part, P->ws.DhD, P->ws.JH, P->ws.DhF, P->ws.dmax, P->ws.scal, P->ws.err, P->ws.cnt, P->ws.big, P->ws.nbig,
                     P->ws.Ms, P->ws.Zs, P->ws.Ds, P->ws.Mex, P->ws.Zex, P->ws.Dex, P->ws.Dpf, P->ws.dmaxf, P->ws.Cs, P->ws.Cex, P->ws.Kpart,

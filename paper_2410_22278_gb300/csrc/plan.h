@@ -145,6 +145,9 @@ struct Plan {
     PpiRec *d_ppi = nullptr;
     PpiF *d_ppf = nullptr;
     float *d_ppB = nullptr;  // |K| p^{-5/4} per primitive pair
+    float4 *d_pps = nullptr;  // (P, 1/p) and ln(|K| p^{-5/4}) per primitive pair
+    float *d_pplb = nullptr;
+    float lb_max = 0.0f;
     float *d_r1f = nullptr;
     SpairRec *d_spair = nullptr;
     int *d_spi_order = nullptr;

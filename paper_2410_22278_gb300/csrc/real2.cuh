@@ -4,16 +4,9 @@
 // The lane-per-bra tile kernel of kernels.cuh lets the 32 lanes of a warp
 // walk one ket with 32 different bras; lanes whose bra cannot reach the ket,
 // or whose primitive quartet is screened out, idle while the others work.
-// Here one warp owns one bra image and a range of kets:
-//   1. the 32 lanes test 32 kets at once (block bound, quartet-level bound,
-//      precision policy) and the kets that pass are compacted with a ballot;
-//   2. the primitive pairs of those kets are laid out one per lane (the
-//      local primitive pairs of consecutive images are contiguous), so every
-//      lane evaluates the bra primitives against its own ket primitive;
-//   3. the partial Cartesian blocks of lanes that hold the same ket are
-//      summed by a segmented warp reduction, and the first lane of each ket
-//      digests the block into J and K (FP64 atomics); the bra-side Coulomb
-//      term stays in registers until the end.
+// Here one warp owns one bra image and a range of kets, and every stage --
+// image quartets, primitive quartets, terms, digestion -- is refilled to 32
+// lanes from the one before (k_real_w below).
 // Primitive pairs are stored in descending order of B = |K| p^{-5/4}: every
 // primitive prefactor 2 pi^{5/2} |K_i K_j| / (pq sqrt(p+q)) is at most
 // 2 pi^{5/2} 2^{-1/2} B_i B_j (p + q >= 2 sqrt(pq)), so a loop over
@@ -27,6 +20,7 @@
 // time, queued, evaluated one per lane and summed by a full warp reduction.
 #pragma once
 #include "kernels.cuh"
+#include "launch.h"
 
 namespace jk {
 
@@ -166,8 +160,10 @@ __device__ __forceinline__ void prim_term(const PlanDev &pl, const PrimE<LA, LB,
     alphas(ip + iq, latc(&pl.inv_omega2, &pl.inv_omega2f, 0, T(0)), alpha, aw, cw);
     const float4 *lat = reinterpret_cast<const float4 *>(pl.r1f);
     int c = 0;
+#pragma unroll 1
     while (true) {
         bool hit = false;
+#pragma unroll 1
         while (c < pl.nr1) {
             const float4 R = __ldg(lat + c);
             if (R.w - x0n >= r) break;
@@ -328,28 +324,133 @@ __device__ __forceinline__ void digest(const PlanDev &pl, const SpiRec &sb, cons
 
 constexpr int kWarpsPerBlock = 4;
 
-// Warp-per-bra tile kernel.  Block = 4 warps = 4 consecutive bras, one chunk
-// of kchunk kets (blockIdx.y).  mode and the FP64 list as in k_real.
+// Image quartets a warp evaluates together (slots of its shared Cartesian
+// blocks): as many as 4.6 KB of shared memory per warp hold, so that the last
+// partly filled batch of primitive quartets of a group counts little.
+template <int NV, typename T>
+struct BatchShape {
+    static constexpr int per = NV * (int)sizeof(T);
+    static constexpr int SL = per <= 24 ? 128 : per <= 72 ? 64 : per <= 144 ? 32 : per <= 216 ? 16 : 8;
+    static constexpr int KQ = SL == 128 ? 256 : SL == 64 ? 128 : 64;  // ring of queued kets, at least SL + 31
+};
+constexpr int kBraChunk = 16;    // bra primitives screened per round (bits of a lane's mask)
+constexpr int kTermRing = 1024;  // at most 31 + 32 * kBraChunk entries are in flight
+
+// Resident blocks asked for: the FP32 kernels of low momentum wait on
+// dependent instructions and need the warps (24 per SM: at most 85 registers).
+template <typename T>
+constexpr int tile_blocks(int L)
+{
+    return sizeof(T) == 4 ? (L == 0 ? 6 : L <= 1 ? 5 : L <= 2 ? 4 : 3) : (L == 0 ? 4 : 3);
+}
+
+// First index in [lo, hi) whose primitive pairs start at or after `val` (hi if
+// none); the whole warp searches, 32 probes per step.
+__device__ __forceinline__ int first_at(const SpiRec *__restrict__ spi, int lo, int hi, long long val)
+{
+    const int lane = threadIdx.x & 31;
+    while (lo < hi) {
+        const int step = (hi - lo + 31) / 32, idx = lo + lane * step;
+        const unsigned m = __ballot_sync(0xffffffffu, idx < hi && spi[idx].pp0 < val);
+        const int c = __popc(m);
+        if (c == 0) return lo;
+        hi = min(hi, lo + c * step);
+        lo += (c - 1) * step + 1;
+    }
+    return lo;
+}
+
+// Bra and ket range of warp `item` of a launch (TileMap); false if it has none.
+__device__ __forceinline__ bool tile_of(const PlanDev &pl, const TileMap &map, long long item, int k0, int k1, int same, int &bra, int &kbeg,
+                                        int &kend)
+{
+    if (item >= map.items) return false;
+    int r = 0;
+    while (r + 1 < map.n && item >= map.g[r + 1].first) ++r;
+    const TileMap::Range &g = map.g[r];
+    const int rel = (int)((item - g.first) / g.nch), ch = (int)((item - g.first) % g.nch);
+    bra = g.b0 + rel;
+    const long long p0 = pl.spi[k0].pp0 + (long long)ch * g.W;
+    kbeg = ch == 0 ? k0 : first_at(pl.spi, k0, k1, p0);
+    kend = ch + 1 == g.nch ? k1 : first_at(pl.spi, kbeg, k1, p0 + g.W);
+    if (same) kbeg = max(kbeg, bra);
+    return kbeg < kend;
+}
+
+// Superset test of prim_radius and the image search for one primitive
+// quartet, without a logarithm or a division: ln of the magnitude bound
+// 2 pi^{5/2} 2^{-1/2} B_i B_j over the threshold is a sum (s = lb_i + lb_j +
+// const, > 0), 1 - c_w <= 1 and ln(1 + 2 alpha_w r) <= its largest value over
+// the plan (Lc), so the sphere drawn here contains the exact one.
+template <int L>
+__device__ __forceinline__ bool prim_maybe(const PlanDev &pl, const float4 &b, const float4 &k, float s, float Lc, float r1min)
+{
+    const float inv = b.w + k.w + pl.inv_omega2f;  // 1 / alpha_w
+    float X[3] = {b.x - k.x, b.y - k.y, b.z - k.z};
+    if (pl.orth == 2) {
+        // diagonal lattice: nearest image by adding and subtracting 1.5 * 2^23
+#pragma unroll
+        for (int a = 0; a < 3; ++a) X[a] = fmaf(-(fmaf(X[a], pl.Finvf[4 * a], 12582912.0f) - 12582912.0f), pl.Lf[4 * a], X[a]);
+    } else {
+        float f[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) f[a] = rintf(pl.Finvf[3 * a] * X[0] + pl.Finvf[3 * a + 1] * X[1] + pl.Finvf[3 * a + 2] * X[2]);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) X[a] -= f[0] * pl.Lf[a] + f[1] * pl.Lf[3 + a] + f[2] * pl.Lf[6 + a];
+    }
+    const float x2 = X[0] * X[0] + X[1] * X[1] + X[2] * X[2];
+    if (L == 0 && pl.orth) return x2 < 1.001f * s * inv;
+    const float r = 1.0005f * fsqrt_fast((s + Lc) * inv) + (L > 0 ? 0.5f + 0.25f * L : 0.0f);
+    // a skewed cell's rounded image may not be the nearest one
+    return x2 < r * r || (!pl.orth && r1min - fsqrt_fast(x2) < r);
+}
+
+// Warp-per-bra tile kernel.  Block = 4 warps, each with a bra and a range of
+// kets (TileMap).  mode and the FP64 list as in k_real.
+//   1. 32 kets at a time are tested (block bound, quartet bound, precision
+//      policy); the ones that pass are queued until SL of them are held.
+//   2. Their primitive pairs are laid out one per lane; each lane marks the
+//      bra primitives whose quartet may have a term (prim_maybe, kBraChunk at
+//      a time) and the marked quartets go into a ring ordered by ket.
+//   3. Whenever 32 are queued they are evaluated, one per lane, and the lanes
+//      of one ket are summed (segmented reduction) into its shared block.
+//   4. The SL blocks are digested, one ket per lane.
+// The work of a warp is bounded by its primitive quartets, not its kets: cut
+// by kets alone, the (ss|ss) launch of a 5-molecule box waited for one warp
+// (36 x 36 primitive quartets, up to 20 images each) for 80% of its 63 ms.
+// Against one ket's primitives per step and kets alone: mixed J+K build of 5
+// water molecules 77 -> 29 ms, of 31 (reciprocal cache) 223 -> 193 ms, of 64
+// 962 -> 801 ms; FP64 build of 6 molecules 325 -> 131 ms.  Bound by
+// instruction issue (0.53 a clock and scheduler, 17 of 32 lanes active).
+// The stages have very different pass rates (water box, (ss|ss): 17% of the
+// pairs, then 1.3 terms out of 6.7 screened primitive quartets per pair), so
+// each stage refills the warp; with one ket's primitives per step and the
+// screening, the terms and the digestion in one loop body about a tenth of
+// the lanes were active.
 // Counters (cnt, one precision's base): [0] image quartets evaluated, [4]
-// algorithmic flops, [8] screening and bookkeeping flops, [12] lane-terms
-// processed and [14] lane slots offered in the primitive loop (their ratio
-// is the lane occupancy).
+// algorithmic flops, [8] screening and bookkeeping flops, [12] primitive
+// quartets evaluated and [14] lane slots offered to them (their ratio is the
+// lane occupancy).
 template <int LA, int LB, int LC, int LD, typename T>
-__global__ void __launch_bounds__(32 * kWarpsPerBlock) k_real_w(PlanDev pl, int b0, int b1, int k0, int k1, int same, int kchunk, int mode,
-                                                                double tau, const T *__restrict__ Dp, const T *__restrict__ dmax,
+__global__ void __launch_bounds__(32 * kWarpsPerBlock, tile_blocks<T>(LA + LB + LC + LD)) k_real_w(PlanDev pl, TileMap map, int k0, int k1, int same, int mode, double tau,
+                                                                const T *__restrict__ Dp, const T *__restrict__ dmax,
                                                                 double *__restrict__ X, double *__restrict__ Y,
                                                                 unsigned long long *__restrict__ cnt, int2 *__restrict__ big,
                                                                 unsigned *__restrict__ nbig, unsigned cap, unsigned *__restrict__ ovf)
 {
     constexpr int NA = ncart(LA), NB = ncart(LB), NC = ncart(LC), ND = ncart(LD), NV = NA * NB * NC * ND;
     constexpr int L = LA + LB + LC + LD;
+    constexpr int SL = BatchShape<NV, T>::SL, KQ = BatchShape<NV, T>::KQ;
+    __shared__ unsigned ring_s[kWarpsPerBlock][kTermRing];
+    __shared__ int kq_s[kWarpsPerBlock][KQ], pp0_s[kWarpsPerBlock][SL];
+    __shared__ T V_s[kWarpsPerBlock][SL * NV];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int bra = b0 + blockIdx.x * kWarpsPerBlock + wid;
-    if (bra >= b1) return;  // whole warp; no block-wide barrier below
-    int kbeg = k0 + blockIdx.y * kchunk;
-    const int kend = min(k1, kbeg + kchunk);
-    if (same) kbeg = max(kbeg, bra);
-    if (kbeg >= kend) return;
+    int bra, kbeg, kend;
+    // whole warps return; no block-wide barrier below
+    if (!tile_of(pl, map, (long long)blockIdx.x * kWarpsPerBlock + wid, k0, k1, same, bra, kbeg, kend)) return;
+    unsigned *ring = ring_s[wid];
+    int *kq = kq_s[wid], *kpp0 = pp0_s[wid];
+    T *Vs = V_s[wid];
     const SpiRec sb = pl.spi[bra];
     const int n = pl.nbf, nsh = pl.nshell;
     const int aoI = pl.shells[sb.I].ao, aoJ = pl.shells[sb.J].ao;
@@ -360,107 +461,226 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) k_real_w(PlanDev pl, int 
 #pragma unroll
         for (int b = 0; b < NB; ++b) Dij[a * NB + b] = __ldg(Dp + (size_t)(aoI + a) * n + aoJ + b);
     const float tauf = (float)tau;
+    // constants of prim_maybe
+    const float lbc = 3.2094f - pl.log_ewald_R;  // ln(2 pi^{5/2} / sqrt 2) + 1e-3
+    const float r1min = pl.nr1 > 1 ? pl.r1f[7] : 1e30f;
+    float Lc = 0.0f;
+    if (L > 0) {
+        const float smax = 2.0f * pl.lb_max + lbc, om2 = 2.0f * rsqrtf(pl.inv_omega2f);
+        float u = smax;
+#pragma unroll 1
+        for (int it = 0; it < 4; ++it) u = smax + L * __logf(1.0f + om2 * fsqrt_fast(fmaxf(u, 0.0f)));
+        Lc = 1.05f * fmaxf(u - smax, 0.0f);
+    }
     Tally tl;
-    unsigned used = 0, slots = 0;  // lane-terms processed and lane slots offered
-    unsigned nq = 0;
-    for (int kb = kbeg & ~31; kb < kend; kb += 32) {
-        const int kt = kb + lane;
-        bool valid = kt >= kbeg && kt < kend;
-        // one bound for the 32-image block (the same for every lane)
-        if (!__any_sync(0xffffffffu, valid) || !block_reaches<L>(pl, sb, kb >> 5)) continue;
-        SpiRec sk{};
-        if (valid) {
-            sk = pl.spi[kt];
-            valid = quartet_reaches<L>(pl, sb, sk);
+    unsigned used = 0, slots = 0;  // primitive quartets evaluated and lane slots offered
+    unsigned nq = 0, kn = 0, kd = 0;
+
+    // evaluate the next count queued primitive quartets, one per lane, and add
+    // the lanes of each ket into its block
+    unsigned qn = 0, qd = 0;
+    auto eval = [&](unsigned count) {
+        const bool on = lane < count;
+        unsigned key = 0xffffff80u + lane;  // a segment of its own (group 511 is not used)
+        T V[NV];
+#pragma unroll
+        for (int q = 0; q < NV; ++q) V[q] = T(0);
+        if (on) {
+            const unsigned it = ring[(qd + lane) & (kTermRing - 1)];
+            key = it & 0xff80007fu;
+            const int ib = sb.pp0 + (int)((it >> 7) & 255u), ik = kpp0[it & 127u] + (int)((it >> 15) & 255u);
+            PrimE<LA, LB, T> bp;
+            PrimE<LC, LD, T> kp;
+            PpiF bf, kf;
+            load_prim<LA, LB, T>(pl, ib, bp, bf);
+            load_prim<LC, LD, T>(pl, ik, kp, kf);
+            ++tl.brap;
+            ++tl.ketp;
+            prim_term<LA, LB, LC, LD, T>(pl, bp, bf, kp, kf, V, tl);
+            ++used;
         }
-        if (sizeof(T) == 4 && valid && mode) {
-            // precision policy: large quartets (and short [c_w, 1] intervals) go to the FP64 list
-            const float dm = quartet_dmax(reinterpret_cast<const float *>(dmax), nsh, sb, sk);
-            const float est = quartet_estimate_bound(pl, sb, sk) * dm >= tauf ? quartet_estimate(pl, sb, sk) * dm : 0.0f;
-            const float ipq = frcp_fast(sb.pmin) + frcp_fast(sk.pmin);
-            if (est >= tauf || ipq > 0.7225f * (ipq + pl.inv_omega2f)) {
-                const unsigned slot = atomicAdd(nbig, 1u);
-                if (slot < cap) {
-                    big[slot] = make_int2(bra, kt);
-                    valid = false;
-                } else {
-                    atomicAdd(ovf, 1u);
-                }
-            }
-        }
-        const unsigned vmask = __ballot_sync(0xffffffffu, valid);
-        if (!vmask) continue;
-        nq += lane == 0 ? __popc(vmask) : 0;
-        // lay the primitive pairs of the valid kets out one per lane
-        const int np = valid ? sk.npp : 0;
-        int incl = np;
+        slots += lane == 0 ? 32u : 0u;
+        __syncwarp();
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
+            const unsigned ok = __shfl_down_sync(0xffffffffu, key, o);
+            const bool add = lane + o < 32 && ok == key;
+            if (!__any_sync(0xffffffffu, add)) break;
+#pragma unroll
+            for (int q = 0; q < NV; ++q) {
+                const T t = __shfl_down_sync(0xffffffffu, V[q], o);
+                if (add) V[q] += t;
+            }
         }
-        const int total = __shfl_sync(0xffffffffu, incl, 31);
-        const int excl = incl - np;
-        for (int e0 = 0; e0 < total; e0 += 32) {
-            const int e = e0 + lane;
-            const bool act = e < total;
-            // owner lane: the first lane whose inclusive prefix exceeds e
-            int own = 0;
+        const unsigned prev = __shfl_up_sync(0xffffffffu, key, 1);
+        const bool head = on && (lane == 0 || prev != key);
+        T *dst = Vs + (head ? key & 127u : 0u) * NV;
+        if (sb.npp <= kBraChunk) {
+            if (head)
 #pragma unroll
-            for (int step = 16; step > 0; step >>= 1) {
-                const int probe = own + step - 1;
-                const int v = __shfl_sync(0xffffffffu, incl, probe);
-                if (v <= e) own += step;
-            }
-            if (!act) own = 32 + lane;  // a segment of its own
-            const int src = own & 31;
-            const int okt = __shfl_sync(0xffffffffu, kt, src);
-            const int oex = __shfl_sync(0xffffffffu, excl, src);
-            const int opp0 = __shfl_sync(0xffffffffu, sk.pp0, src);
-            T V[NV];
+                for (int q = 0; q < NV; ++q) dst[q] += V[q];
+        } else {
+            // one ket can head several segments here: one after another
+            const unsigned m = __match_any_sync(0xffffffffu, head ? (key & 127u) : 128u + lane);
+            const int rank = __popc(m & ((1u << lane) - 1u));
+#pragma unroll 1
+            for (int rr = 0; __any_sync(0xffffffffu, head && rank >= rr); ++rr) {
+                if (head && rank == rr)
 #pragma unroll
-            for (int q = 0; q < NV; ++q) V[q] = T(0);
-            if (act) {
-                const int kpp = opp0 + (e - oex);
-                PrimE<LC, LD, T> kp;
-                PpiF kf;
-                load_prim<LC, LD, T>(pl, kpp, kp, kf);
-                ++tl.ketp;
-                const float Bk = __ldg(pl.ppB + kpp);
-                // bra primitives in descending order of their bound B: the
-                // first one whose B_i B_k is below the magnitude threshold ends
-                // the loop (every later term is smaller still)
-                for (int i = 0; i < sb.npp; ++i) {
-                    if (__ldg(pl.ppB + sb.pp0 + i) * Bk < pl.mag_thr) break;
-                    PrimE<LA, LB, T> bp;
-                    PpiF bf;
-                    load_prim<LA, LB, T>(pl, sb.pp0 + i, bp, bf);
-                    ++tl.brap;  // recomputed per lane: bookkeeping
-                    prim_term<LA, LB, LC, LD, T>(pl, bp, bf, kp, kf, V, tl);
-                    ++used;
-                }
+                    for (int q = 0; q < NV; ++q) dst[q] += V[q];
+                __syncwarp();
             }
-            slots += (lane == 0) ? 32u * sb.npp : 0u;
-            // segmented sum over the lanes holding the same ket (contiguous)
+        }
+        qd += count;
+        __syncwarp();
+    };
+    // screen, evaluate and digest the next count queued kets
+    auto process = [&](int count) {
+#pragma unroll 1
+        for (int q = lane; q < count * NV; q += 32) Vs[q] = T(0);
+        unsigned grp = 0;
+#pragma unroll 1
+        for (int s0 = 0; s0 < count; s0 += 32) {
+            int np = 0;
+            if (s0 + lane < count) {
+                const int kt = kq[(kd + s0 + lane) & (KQ - 1)];
+                np = pl.spi[kt].npp;
+                kpp0[s0 + lane] = pl.spi[kt].pp0;
+            }
+            int incl = np;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const int oo = __shfl_down_sync(0xffffffffu, own, o);
-                const bool add = lane + o < 32 && oo == own;
-#pragma unroll
-                for (int q = 0; q < NV; ++q) {
-                    const T t = __shfl_down_sync(0xffffffffu, V[q], o);
-                    if (add) V[q] += t;
-                }
+                const int t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
             }
-            const int prev = __shfl_up_sync(0xffffffffu, own, 1);
-            const bool head = act && (lane == 0 || prev != own);
-            if (head) {
-                const SpiRec skh = pl.spi[okt];
-                const T w = T(sb.w) * T(skh.w) * ((same && okt == bra) ? T(0.5) : T(1));
-                digest<LA, LB, LC, LD, T>(pl, sb, skh, V, w, Dp, Dij, jb, X, Y);
-                ++tl.quart;
+            const int total = __shfl_sync(0xffffffffu, incl, 31);
+            const int excl = incl - np;
+            __syncwarp();
+            int e0 = 0, ic = 0, src = 0, j = 0;
+            float4 kv = make_float4(0.f, 0.f, 0.f, 0.f);
+            float ks = -1e30f;
+#pragma unroll 1
+            while (e0 < total) {
+                if (ic == 0) {
+                    const int e = e0 + lane;
+                    // owner: the first lane whose inclusive prefix exceeds e
+                    int own = 0;
+#pragma unroll
+                    for (int step = 16; step > 0; step >>= 1) {
+                        const int v = __shfl_sync(0xffffffffu, incl, own + step - 1);
+                        if (v <= e) own += step;
+                    }
+                    src = s0 + own;
+                    j = e - __shfl_sync(0xffffffffu, excl, own);
+                    ks = -1e30f;
+                    if (e < total) {
+                        const int kpp = kpp0[src] + j;
+                        kv = __ldg(pl.pps + kpp);
+                        ks = __ldg(pl.pplb + kpp) + lbc;
+                    }
+                }
+                unsigned mask = 0;
+                const int ie = min(kBraChunk, sb.npp - ic);
+                // bra primitives in descending order of their bound: the first one
+                // below the magnitude threshold ends the loop
+                int i = 0;
+#pragma unroll 1
+                for (; i < ie; ++i) {
+                    const float s = ks + __ldg(pl.pplb + sb.pp0 + ic + i);
+                    if (!(s > 0.0f)) break;
+                    ++tl.screen;
+                    if (prim_maybe<L>(pl, __ldg(pl.pps + sb.pp0 + ic + i), kv, s, Lc, r1min)) mask |= 1u << i;
+                }
+                const int cm = __popc(mask);
+                int pre = cm;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int t = __shfl_up_sync(0xffffffffu, pre, o);
+                    if (lane >= o) pre += t;
+                }
+                unsigned pos = qn + pre - cm;
+                const unsigned base = (unsigned)src | ((unsigned)ic << 7) | ((unsigned)j << 15) | (grp << 23);
+#pragma unroll 1
+                while (mask) {
+                    const unsigned b = __ffs(mask) - 1;
+                    mask &= mask - 1;
+                    ring[pos++ & (kTermRing - 1)] = base + (b << 7);
+                }
+                qn += __shfl_sync(0xffffffffu, pre, 31);
+                // the quartets of one ket stay adjacent in the ring unless the bra
+                // takes several rounds; then each round is a group of its own
+                if (sb.npp > kBraChunk) grp = grp == 510u ? 0u : grp + 1u;
+                ic += kBraChunk;
+                if (ic >= sb.npp || !__any_sync(0xffffffffu, i == kBraChunk)) {
+                    ic = 0;
+                    e0 += 32;
+                }
+                __syncwarp();
+                const unsigned lim = e0 < total || s0 + 32 < count ? 32u : 1u;
+#pragma unroll 1
+                while (qn - qd >= lim) eval(min(32u, qn - qd));
             }
         }
+        __syncwarp();
+#pragma unroll 1
+        for (int sl = lane; sl < count; sl += 32) {
+            T V[NV];
+            bool any = false;
+#pragma unroll
+            for (int q = 0; q < NV; ++q) {
+                V[q] = Vs[sl * NV + q];
+                any = any || V[q] != T(0);
+            }
+            if (any) {
+                const int kt = kq[(kd + sl) & (KQ - 1)];
+                const SpiRec sk = pl.spi[kt];
+                const T w = T(sb.w) * T(sk.w) * ((same && kt == bra) ? T(0.5) : T(1));
+                digest<LA, LB, LC, LD, T>(pl, sb, sk, V, w, Dp, Dij, jb, X, Y);
+            }
+            ++tl.quart;
+        }
+        kd += count;
+        __syncwarp();
+    };
+
+    // 32 blocks of 32 kets at a time: one block bound per lane, then the kets
+    // of the blocks that may be reached
+#pragma unroll 1
+    for (int g0 = kbeg >> 5; g0 * 32 < kend; g0 += 32) {
+        unsigned bm = __ballot_sync(0xffffffffu, (g0 + lane) * 32 < kend && block_reaches<L>(pl, sb, g0 + lane));
+        const bool last = (g0 + 32) * 32 >= kend;
+        do {
+            const int kt = bm ? (g0 + __ffs(bm) - 1) * 32 + lane : kend;
+            bm &= bm - 1;
+            bool valid = kt >= kbeg && kt < kend;
+            if (valid) {
+                const SpiRec sk = pl.spi[kt];
+                valid = quartet_reaches<L>(pl, sb, sk);
+                if (sizeof(T) == 4 && valid && mode) {
+                    // precision policy: large quartets (and short [c_w, 1] intervals) go to the FP64 list
+                    const float dm = quartet_dmax(reinterpret_cast<const float *>(dmax), nsh, sb, sk);
+                    const float est = quartet_estimate_bound(pl, sb, sk) * dm >= tauf ? quartet_estimate(pl, sb, sk) * dm : 0.0f;
+                    const float ipq = frcp_fast(sb.pmin) + frcp_fast(sk.pmin);
+                    if (est >= tauf || ipq > 0.7225f * (ipq + pl.inv_omega2f)) {
+                        const unsigned slot = atomicAdd(nbig, 1u);
+                        if (slot < cap) {
+                            big[slot] = make_int2(bra, kt);
+                            valid = false;
+                        } else {
+                            atomicAdd(ovf, 1u);
+                        }
+                    }
+                }
+            }
+            const unsigned vmask = __ballot_sync(0xffffffffu, valid);
+            nq += lane == 0 ? __popc(vmask) : 0;
+            if (valid) kq[(kn + __popc(vmask & ((1u << lane) - 1u))) & (KQ - 1)] = kt;
+            kn += __popc(vmask);
+            __syncwarp();
+            const unsigned lim = last && !bm ? 1u : (unsigned)SL;
+#pragma unroll 1
+            while (kn - kd >= lim) process((int)min((unsigned)SL, kn - kd));
+        } while (bm);
     }
     // bra-side Coulomb: one atomic per element for the warp
 #pragma unroll
