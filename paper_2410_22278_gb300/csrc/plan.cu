@@ -1050,6 +1050,11 @@ int finish_plan_device(Plan *P)
         }
         P->ppi_pidx.resize(P->ppi.size());
         for (size_t i = 0; i < P->ppi.size(); ++i) P->ppi_pidx[i] = pid[P->ppi[i].p];
+        P->pval_kmax.assign(P->pvals.size(), 0.0);
+        for (size_t i = 0; i < P->ppi.size(); ++i) {
+            double &k = P->pval_kmax[P->ppi_pidx[i]];
+            k = std::max(k, std::fabs(P->ppi[i].K));
+        }
         std::vector<double> gt0(P->pvals.size());
         for (size_t i = 0; i < gt0.size(); ++i) gt0[i] = std::pow(kPi / P->pvals[i], 1.5);
         // phase table, rounded from extended precision
@@ -1081,6 +1086,7 @@ int finish_plan_device(Plan *P)
                 const double v = (P->L[3 * k] * G[0] + P->L[3 * k + 1] * G[1] + P->L[3 * k + 2] * G[2]) / (2.0 * kPi);
                 const double r = std::rint(v);
                 if (std::fabs(v - r) > 1e-6 || std::fabs(r) > 64) ok = false;
+                P->g_nmax = std::max(P->g_nmax, std::fabs(v - r) > 1e-6 ? 1 << 20 : (int)std::min(std::fabs(r), 1e6));
                 nk[k] = (float)r;
             }
             const dfl gx = dfl_split(G[0]), gy = dfl_split(G[1]), gz = dfl_split(G[2]);

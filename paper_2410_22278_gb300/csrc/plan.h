@@ -160,6 +160,8 @@ struct Plan {
     // structure-factor tables: distinct pair exponents, the exponent index of
     // each primitive pair, (cos, sin)(2 pi k / 1024), and (pi/p)^{3/2} (G = 0)
     std::vector<double> pvals;
+    std::vector<double> pval_kmax;  // largest |K| of each distinct exponent
+    int g_nmax = 0;                 // largest |n_k| of the reciprocal vectors in the reciprocal basis
     std::vector<int> ppi_pidx;
     std::vector<double2> ppi_ab;  // exponents (a, b) of each primitive pair (one-electron operators)
     double2 *d_ppi_ab = nullptr;
