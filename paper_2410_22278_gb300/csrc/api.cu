@@ -235,25 +235,15 @@ int jk_build_host(jk_plan *plan, const double *Dh, double *Jh, double *Kh, void 
     return rc;
 }
 
-__global__ void jk_energy_kernel(size_t n2, const double *D, const double *J, const double *K, double *out);
-
 int jk_energy(const jk_plan *plan, const double *D, const double *J, const double *K, double *e_coul, double *e_exch, void *cuda_stream)
 {
     if (!plan || !D || !e_coul || !e_exch) return fail(JK_ERR_INVALID, "NULL argument");
-    cudaStream_t st = (cudaStream_t)cuda_stream;
-    if (cudaSetDevice(plan->p->device) != cudaSuccess) return fail(JK_ERR_CUDA, "cudaSetDevice failed");
-    const size_t n2 = (size_t)plan->p->nbf * plan->p->nbf;
-    double *dev = nullptr;
-    if (cudaMallocAsync((void **)&dev, 2 * sizeof(double), st) != cudaSuccess) return fail(JK_ERR_OOM, "energy scratch");
-    cudaMemsetAsync(dev, 0, 2 * sizeof(double), st);
-    jk_energy_kernel<<<(unsigned)std::min<size_t>((n2 + 255) / 256, 2432), 256, 0, st>>>(n2, D, J, K, dev);
-    double h[2] = {0, 0};
-    cudaMemcpyAsync(h, dev, 2 * sizeof(double), cudaMemcpyDeviceToHost, st);
-    cudaFreeAsync(dev, st);
-    if (cudaStreamSynchronize(st) != cudaSuccess) return fail(JK_ERR_CUDA, "energy reduction failed");
-    *e_coul = 0.5 * h[0];
-    *e_exch = -0.25 * h[1];
-    return JK_OK;
+    try {
+        if (cudaSetDevice(plan->p->device) != cudaSuccess) return fail(JK_ERR_CUDA, "cudaSetDevice failed");
+        return jk::energy(plan->p, D, J, K, e_coul, e_exch, (cudaStream_t)cuda_stream);
+    } catch (...) {
+        return fail(JK_ERR_INVALID, "unexpected host exception");
+    }
 }
 
 int jk_energy_noalloc(const jk_plan *plan, const double *D, const double *J, const double *K, double *e_coul, double *e_exch,
@@ -300,34 +290,6 @@ int jk_ewald_point_charges(const jk_cell *cell, int n, const double *q, const do
 }
 
 }  // extern "C"
-
-__global__ void jk_energy_kernel(size_t n2, const double *D, const double *J, const double *K, double *out)
-{
-    double s0 = 0, s1 = 0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n2; i += (size_t)gridDim.x * blockDim.x) {
-        if (J) s0 += D[i] * J[i];
-        if (K) s1 += D[i] * K[i];
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-    }
-    __shared__ double sh[2][32];
-    if ((threadIdx.x & 31) == 0) {
-        sh[0][threadIdx.x >> 5] = s0;
-        sh[1][threadIdx.x >> 5] = s1;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double a = 0, b = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            a += sh[0][w];
-            b += sh[1][w];
-        }
-        atomicAdd(out, a);
-        atomicAdd(out + 1, b);
-    }
-}
 
 __global__ void jk_scale_kernel(int n, const double *f, const double *A, double *B)
 {

@@ -1127,6 +1127,7 @@ int finish_plan_device(Plan *P)
     std::vector<double> zeros((size_t)P->nbf * P->nbf, 0.0);
     if ((rc = upload(zeros, &P->d_S, b))) return rc;
     if ((rc = alloc_ws(P))) return rc;
+    if ((rc = energy_reserve(P))) return rc;
     if ((rc = compute_overlap_raw(P, 0))) return rc;
     if (cudaDeviceSynchronize() != cudaSuccess) return fail(JK_ERR_CUDA, "plan setup kernels failed");
     return JK_OK;
@@ -1137,6 +1138,7 @@ void destroy_plan(Plan *P)
     if (!P) return;
     cudaSetDevice(P->device);
     release_cache(P);
+    energy_release(P);
     void *ptrs[] = {P->d_shells, P->d_spi, P->d_ppi, P->d_ppf, P->d_ppB, P->d_pps, P->d_pplb, P->d_r1f, P->d_spair, P->d_spi_order, P->d_boys, P->d_boys_f, P->d_boys_t, P->d_r1, P->d_gvec,
                     P->d_g0, P->d_compf, P->d_ppi_ab, P->d_kblk, P->d_kblk2, P->d_pvals, P->d_gtab0, P->d_ppi_pidx, P->d_phase, P->d_ppdf, P->d_gdf, P->d_phasef, P->ws.gtab, P->ws.gtab2, P->d_S, P->ws.Dp, P->ws.X, P->ws.Y, P->ws.JLR, P->ws.KLR, P->ws.T1, P->ws.T2,
                     P->ws.M, P->ws.Z, P->ws.rho, P->ws.rho_part, P->ws.DhD, P->ws.JH, P->ws.DhF, P->ws.dmax, P->ws.scal, P->ws.err, P->ws.cnt, P->ws.big, P->ws.nbig,

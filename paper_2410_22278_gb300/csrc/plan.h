@@ -112,6 +112,14 @@ struct RecipCache {
     CUtensorMap tm_Ms;
 };
 
+// Scratch of one jk_energy call: block partials and a block counter on the
+// device, the two sums in pinned host memory.  A plan keeps one per call that
+// was ever in flight on it at once.
+struct EnergySlot {
+    double *part = nullptr;
+    double *host = nullptr;
+};
+
 struct Plan {
     int device = 0;
     jk_precision precision = JK_FP64;
@@ -180,6 +188,8 @@ struct Plan {
     RecipCache cache;
     PhaseTimer timer;
     std::mutex build_mu;
+    std::mutex energy_mu;
+    std::vector<EnergySlot> energy_free;  // not in use by a call
     PlanDev dev() const;
 };
 
@@ -202,6 +212,9 @@ int ozaki_finish(Plan *P, cudaStream_t st);
 struct Plan;
 void launch_gauss_table(const Plan *P, int g0, int gcur, double *tab, cudaStream_t st);
 int one_electron(Plan *P, int natom, const double *Z, const double *xyz, double *T, double *V, cudaStream_t st);
+int energy(Plan *P, const double *D, const double *J, const double *K, double *e_coul, double *e_exch, cudaStream_t st);
+int energy_reserve(Plan *P);
+void energy_release(Plan *P);
 int energy_noalloc(const Plan *P, const double *D, const double *J, const double *K, double *e_coul, double *e_exch,
                    cudaStream_t st);
 
