@@ -390,8 +390,8 @@ static int reciprocal_phase(Plan *P, double *J, double *K, cudaStream_t st)
                 slab_gemv_t(Mc, npk, m2, w.T1, w.rho_part, w.rho, st);
                 slab_gemv_n(Mc, npk, m2, w.rho, 1.0, w.T2, st);
             } else {
-                slab_gemv_t(Mc, (long long)n2, m2, w.Dp, w.rho_part, w.rho, st);
-                slab_gemv_n(Mc, (long long)n2, m2, w.rho, 1.0, w.JLR, st);
+                slab_sym_t(Mc, n, m2, w.Dp, w.T1, w.rho_part, w.rho, g0 == 0, st);
+                slab_sym_n(Mc, n, m2, w.rho, w.JLR, st);
             }
             tm.stop(3, ev, 3);
         }

@@ -71,17 +71,160 @@ __global__ void k_slab_dot_final(int m2, int splits, const double *__restrict__ 
     rho[b] = t;
 }
 
+static int slab_dot_splits(long long n2, int m2)
+{
+    // about eight blocks per SM in total (a chunk of one G vector has only two
+    // slabs), at least 4096 elements per block
+    const long long want = std::max(1LL, (152LL * 8 + m2 - 1) / std::max(1, m2));
+    return (int)std::max(1LL, std::min({want, (n2 + 4095) / 4096, (long long)kSlabSplitsMax}));
+}
+
+// Triangle of an n x n matrix in rows of constant length: row pair r (r <
+// (n + 1) / 2) is row r from its diagonal on followed by row n - 1 - r from
+// its diagonal on, n + 1 elements; the middle pair of an odd n has only the
+// first half.  Position e of pair r; false if it has no element.
+__device__ __forceinline__ bool tri_pair(int n, int r, int e, int &i, int &j)
+{
+    if (e < n - r) {
+        i = r;
+        j = r + e;
+        return true;
+    }
+    i = n - 1 - r;
+    j = i + e - (n - r);
+    return i != r;
+}
+
+// Ds = D + D^T off the diagonal, D on it
+__global__ void k_sym_full(int n, const double *__restrict__ D, double *__restrict__ Ds)
+{
+    const size_t n2 = (size_t)n * n;
+    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < n2; x += (size_t)gridDim.x * blockDim.x) {
+        const size_t i = x / n, j = x - i * n;
+        Ds[x] = i == j ? D[x] : D[x] + D[j * n + i];
+    }
+}
+
+// k_slab_dot over one triangle of symmetric n x n slabs.  One FP64 FMA per
+// element is all the arithmetic there is, and at 2 per clock and SM that is
+// what bounds the pass (832 functions, 94 GB of slabs: 22 ms for the full
+// matrices, 20.3 ms of it FP64 issue; the copy rate would allow 14): half the
+// elements, half the time.
+__global__ void __launch_bounds__(256) k_slab_dot_sym(const double *__restrict__ M, int n, const double *__restrict__ Ds, int splits,
+                                                      double *__restrict__ part)
+{
+    __shared__ double sh[8];
+    const int b = blockIdx.y, sidx = blockIdx.x;
+    const long long tot = (long long)((n + 1) / 2) * (n + 1), per = (tot + splits - 1) / splits;
+    const long long i0 = sidx * per, i1 = min(tot, i0 + per);
+    const double *Mb = M + (size_t)b * n * n;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    long long x = i0 + threadIdx.x;
+    int r = (int)(x / (n + 1)), e = (int)(x - (long long)r * (n + 1));
+    for (; x < i1; x += 4 * 256) {
+        size_t o[4];
+        bool v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            int i = 0, j = 0;
+            v[u] = x + 256 * u < i1 && tri_pair(n, r, e, i, j);
+            o[u] = v[u] ? (size_t)i * n + j : 0;
+            e += 256;
+            while (e > n) {
+                e -= n + 1;
+                ++r;
+            }
+        }
+        double m[4], dd[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            m[u] = v[u] ? __ldg(Mb + o[u]) : 0.0;
+            dd[u] = v[u] ? __ldg(Ds + o[u]) : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[u] = fma(m[u], dd[u], acc[u]);
+    }
+    double s = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += sh[w];
+        part[(size_t)b * splits + sidx] = t;
+    }
+}
+
+// k_slab_axpy over one triangle: y gets both triangles.  blockIdx.y splits the
+// slabs (FP64 atomics) when one thread per element leaves the chip idle.
+__global__ void __launch_bounds__(256) k_slab_axpy_sym(const double *__restrict__ M, int n, int m2, const double *__restrict__ rho, int per,
+                                                       double *__restrict__ y)
+{
+    __shared__ double r[1024];
+    const long long tot = (long long)((n + 1) / 2) * (n + 1), x = (long long)blockIdx.x * 256 + threadIdx.x;
+    int i = 0, j = 0;
+    const bool v = x < tot && tri_pair(n, (int)(x / (n + 1)), (int)(x % (n + 1)), i, j);
+    const size_t n2 = (size_t)n * n;
+    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    const int bb = blockIdx.y * per, be = min(m2, bb + per);
+    for (int b0 = bb; b0 < be; b0 += 1024) {
+        const int nb = min(1024, be - b0);
+        __syncthreads();
+        for (int k = threadIdx.x; k < nb; k += 256) r[k] = rho[b0 + k];
+        __syncthreads();
+        if (v) {
+            const double *col = M + (size_t)b0 * n2 + (size_t)i * n + j;
+            int k = 0;
+            for (; k + 7 < nb; k += 8) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) acc[u] = fma(__ldg(col + (size_t)(k + u) * n2), r[k + u], acc[u]);
+            }
+            for (; k < nb; ++k) acc[0] = fma(__ldg(col + (size_t)k * n2), r[k], acc[0]);
+        }
+    }
+    if (!v) return;
+    const double s = ((acc[0] + acc[1]) + (acc[2] + acc[3])) + ((acc[4] + acc[5]) + (acc[6] + acc[7]));
+    if (gridDim.y > 1) {
+        atomicAdd(y + (size_t)i * n + j, s);
+        if (i != j) atomicAdd(y + (size_t)j * n + i, s);
+    } else {
+        y[(size_t)i * n + j] += s;
+        if (i != j) y[(size_t)j * n + i] += s;
+    }
+}
+
+void slab_sym_t(const double *M, int n, int m2, const double *D, double *Ds, double *part, double *rho, bool first, cudaStream_t st)
+{
+    if (m2 <= 0) return;
+    if (first) k_sym_full<<<(unsigned)std::min<long long>(((long long)n * n + 255) / 256, 152 * 16), 256, 0, st>>>(n, D, Ds);
+    const int splits = slab_dot_splits((long long)n * (n + 1) / 2, m2);
+    k_slab_dot_sym<<<dim3(splits, m2), 256, 0, st>>>(M, n, Ds, splits, part);
+    k_slab_dot_final<<<(m2 + 127) / 128, 128, 0, st>>>(m2, splits, part, rho);
+}
+
+void slab_sym_n(const double *M, int n, int m2, const double *rho, double *y, cudaStream_t st)
+{
+    if (m2 <= 0 || n <= 0) return;
+    const int nx = (int)(((long long)((n + 1) / 2) * (n + 1) + 255) / 256);
+    // about eight blocks per SM, at least 64 slabs each
+    const int ns = std::max(1, std::min((152 * 8 + nx - 1) / nx, m2 / 64)), per = (m2 + ns - 1) / ns;
+    k_slab_axpy_sym<<<dim3(nx, (m2 + per - 1) / per), 256, 0, st>>>(M, n, m2, rho, per, y);
+}
+
 // y[i] += alpha sum_b M[b][i] rho[b]; threads over i (coalesced per b),
 // eight independent accumulators (eight loads in flight per thread), rho
-// staged through shared memory.
+// staged through shared memory; blockIdx.y splits the slabs (FP64 atomics)
+// when one thread per element leaves the chip idle.
 __global__ void __launch_bounds__(256) k_slab_axpy(const double *__restrict__ M, long long n2, int m2, const double *__restrict__ rho,
-                                                   double alpha, double *__restrict__ y)
+                                                   double alpha, int per, double *__restrict__ y)
 {
     __shared__ double r[1024];
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int b0 = 0; b0 < m2; b0 += 1024) {
-        const int nb = min(1024, m2 - b0);
+    const int bb = blockIdx.y * per, be = min(m2, bb + per);
+    for (int b0 = bb; b0 < be; b0 += 1024) {
+        const int nb = min(1024, be - b0);
         __syncthreads();
         for (int k = threadIdx.x; k < nb; k += blockDim.x) r[k] = rho[b0 + k];
         __syncthreads();
@@ -95,15 +238,10 @@ __global__ void __launch_bounds__(256) k_slab_axpy(const double *__restrict__ M,
             for (; k < nb; ++k) acc[0] = fma(__ldg(col + (size_t)k * n2), r[k], acc[0]);
         }
     }
-    if (i < n2) y[i] += alpha * (((acc[0] + acc[1]) + (acc[2] + acc[3])) + ((acc[4] + acc[5]) + (acc[6] + acc[7])));
-}
-
-int slab_dot_splits(long long n2, int m2)
-{
-    // about eight blocks per SM in total (a chunk of one G vector has only two
-    // slabs), at least 4096 elements per block
-    const long long want = std::max(1LL, (152LL * 8 + m2 - 1) / std::max(1, m2));
-    return (int)std::max(1LL, std::min({want, (n2 + 4095) / 4096, (long long)kSlabSplitsMax}));
+    if (i >= n2) return;
+    const double s = alpha * (((acc[0] + acc[1]) + (acc[2] + acc[3])) + ((acc[4] + acc[5]) + (acc[6] + acc[7])));
+    if (gridDim.y > 1) atomicAdd(y + i, s);
+    else y[i] += s;
 }
 
 void slab_gemv_t(const double *M, long long n2, int m2, const double *x, double *part, double *rho, cudaStream_t st)
@@ -117,7 +255,9 @@ void slab_gemv_t(const double *M, long long n2, int m2, const double *x, double 
 void slab_gemv_n(const double *M, long long n2, int m2, const double *rho, double alpha, double *y, cudaStream_t st)
 {
     if (m2 <= 0 || n2 <= 0) return;
-    k_slab_axpy<<<(unsigned)((n2 + 255) / 256), 256, 0, st>>>(M, n2, m2, rho, alpha, y);
+    const int nx = (int)((n2 + 255) / 256);
+    const int ns = std::max(1, std::min((152 * 8 + nx - 1) / nx, m2 / 64)), per = (m2 + ns - 1) / ns;
+    k_slab_axpy<<<dim3(nx, (m2 + per - 1) / per), 256, 0, st>>>(M, n2, m2, rho, alpha, per, y);
 }
 
 // ---------------------------------------------------------------------------

@@ -24,6 +24,11 @@ constexpr int kSlabSplitsMax = 1024;
 void slab_gemv_t(const double *M, long long n2, int m2, const double *x, double *part, double *rho, cudaStream_t st);
 // y[i] += alpha sum_b M[b][i] rho[b].
 void slab_gemv_n(const double *M, long long n2, int m2, const double *rho, double alpha, double *y, cudaStream_t st);
+// The same two passes over full n x n slabs of symmetric matrices, reading one
+// triangle: rho[b] = sum_ij M[b][ij] D[ij] (Ds, n x n scratch, receives the
+// symmetrised D) and y[ij] += sum_b M[b][ij] rho[b].
+void slab_sym_t(const double *M, int n, int m2, const double *D, double *Ds, double *part, double *rho, bool first, cudaStream_t st);
+void slab_sym_n(const double *M, int n, int m2, const double *rho, double *y, cudaStream_t st);
 // Row-major batched FP64 GEMM; sc = 0 reduces every batch into one C (atomics).
 void dgemm_batched(int m, int n, int k, const double *A, long long lda, long long sa, const double *B, long long ldb, long long sb,
                    double *C, long long ldc, long long sc, int nbatch, double alpha, double beta, bool upper, cudaStream_t st);
