@@ -38,7 +38,9 @@ __global__ void k_to_float(size_t n, const double *__restrict__ a, float *__rest
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) b[i] = (float)a[i];
 }
 
-__global__ void k_dmax(PlanDev pl, const double *__restrict__ Dp, double *__restrict__ dmax)
+// max |D'| per shell block, its single-precision copy and the largest of all
+// (dmaxf[nshell^2], zeroed before the launch)
+__global__ void k_dmax(PlanDev pl, const double *__restrict__ Dp, double *__restrict__ dmax, float *__restrict__ dmaxf)
 {
     const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const int nsh = pl.nshell;
@@ -49,6 +51,8 @@ __global__ void k_dmax(PlanDev pl, const double *__restrict__ Dp, double *__rest
     for (int i = 0; i < ncart(a.l); ++i)
         for (int j = 0; j < ncart(b.l); ++j) m = fmax(m, fabs(Dp[(size_t)(a.ao + i) * pl.nbf + b.ao + j]));
     dmax[idx] = m;
+    dmaxf[idx] = (float)m;
+    atomicMax(reinterpret_cast<int *>(dmaxf + (size_t)nsh * nsh), __float_as_int((float)m));  // m >= 0: ordered as integers
 }
 
 // out[k] += sum_i A_k[i] * B[i] for k = 0, 1 (two traces in one pass)
@@ -445,9 +449,9 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
     k_scale<<<grid_for(n2), 256, 0, st>>>(n, P->d_compf, D, w.Dp);
     if (mixed) {
         const long long ns2 = (long long)P->nshell * P->nshell;
-        k_dmax<<<(unsigned)((ns2 + 255) / 256), 256, 0, st>>>(pl, w.Dp, w.dmax);
+        cudaMemsetAsync(w.dmaxf + ns2, 0, sizeof(float), st);
+        k_dmax<<<(unsigned)((ns2 + 255) / 256), 256, 0, st>>>(pl, w.Dp, w.dmax, w.dmaxf);
         k_to_float<<<grid_for(n2), 256, 0, st>>>(n2, w.Dp, w.Dpf);
-        k_to_float<<<grid_for((size_t)ns2), 256, 0, st>>>((size_t)ns2, w.dmax, w.dmaxf);
     }
     cudaMemsetAsync(w.X, 0, n2 * sizeof(double), st);
     cudaMemsetAsync(w.Y, 0, n2 * sizeof(double), st);
@@ -461,7 +465,7 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
     // mixed precision: slices of D' and its low-rank factorisation for the
     // exchange contraction (decided on the device; nothing waits for it)
     if (mixed && K && (rc = ozaki_begin(P, st))) return rc;
-    tm.stop(0, ev, mixed ? (K ? 8 : 4) : 1);
+    tm.stop(0, ev, mixed ? (K ? 7 : 3) : 1);
 
     // Coulomb-only build: the J-engine (Hermite densities in, Hermite J out)
     // (only the classes with a d shell, l_I = 2, take part: kJengClass)

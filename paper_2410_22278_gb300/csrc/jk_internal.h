@@ -95,6 +95,9 @@ struct PlanDev {
     const SpiRec *spi;
     const float4 *kblk;          // images 32k .. 32k+31: bounding sphere (centre, radius including extents)
     const float2 *kblk2;         // the same images: largest S, smallest pair exponent
+    const float4 *spq;           // per image: centre and extent
+    const float4 *spr;           // per image, and one past the last: S, ln S (both rounded up), 1 / pmin, first primitive pair (int bits)
+    const int4 *spd;             // per image: first basis functions of its shells, orbit weight (float bits)
     const PpiRec *ppi;
     const SpairRec *spair;
     const int *spi_order;        // spi indices grouped by shell pair (for the reciprocal build)
@@ -105,7 +108,7 @@ struct PlanDev {
     const float *ppB;            // B = |K| p^{-5/4} of each primitive pair (descending inside an image)
     const float4 *pps;           // (P, 1/p) of each primitive pair and ln B (rounded up): the screening of real2.cuh
     const float *pplb;
-    float lb_max;                // largest ln B
+    float lb_max, ls_max;        // largest ln B and ln S
     float mag_thr;               // B_i B_j below this: the primitive quartet is below the real-space threshold
     const double *r1;            // [nr1][4]: x, y, z, |R|, sorted by |R|
     const float *r1f;            // the same in single precision

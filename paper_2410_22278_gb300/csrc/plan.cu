@@ -330,6 +330,9 @@ PlanDev Plan::dev() const
     d.nspair = (int)spair.size();
     d.shells = d_shells;
     d.spi = d_spi;
+    d.spq = d_spq;
+    d.spr = d_spr;
+    d.spd = d_spd;
     d.kblk = d_kblk;
     d.kblk2 = d_kblk2;
     d.ppi = d_ppi;
@@ -369,6 +372,7 @@ PlanDev Plan::dev() const
     d.pps = d_pps;
     d.pplb = d_pplb;
     d.lb_max = lb_max;
+    d.ls_max = ls_max;
     d.mag_thr = (float)(cut.ewald_R * 1e-1 / (24.739424126 * 1.001));
     d.volume = volume;
     for (int a = 0; a < 3; ++a)
@@ -444,7 +448,7 @@ static int alloc_ws(Plan *P)
     bool ok = al(&w.gtab, std::max<size_t>(1, P->pvals.size()) * (size_t)gc) && al(&w.Dp, n2) && al(&w.X, n2) && al(&w.Y, n2) && al(&w.JLR, n2) && al(&w.KLR, n2) && al(&w.T1, n2) &&
               al(&w.T2, n2) && al(&w.M, 2 * (size_t)gc * n2) && al(&w.Z, 2 * (size_t)gc * n2) && al(&w.rho, 2 * (size_t)gc) && al(&w.rho_part, 2 * (size_t)gc * kSlabSplitsMax) &&
               al(&w.dmax, (size_t)P->nshell * P->nshell) && al(&w.scal, 16) && (!mixed || al((double **)&w.Dpf, (n2 + 1) / 2)) &&
-              (!mixed || al((double **)&w.dmaxf, ((size_t)P->nshell * P->nshell + 1) / 2));
+              (!mixed || al((double **)&w.dmaxf, ((size_t)P->nshell * P->nshell + 2) / 2));
     {
         // J-engine arrays: stride N_H(2 lmax)
         int lmax = 0;
@@ -997,6 +1001,28 @@ int finish_plan_device(Plan *P)
         }
         if ((rc = upload(kb, &P->d_kblk, b)) || (rc = upload(kb2, &P->d_kblk2, b))) return rc;
     }
+    {
+        const size_t ns = P->spi.size();
+        std::vector<float4> sq(ns), sr(ns + 1);
+        std::vector<int4> sd(ns);
+        P->ls_max = -1e30f;
+        const auto bits = [](int v) {
+            float f;
+            memcpy(&f, &v, sizeof f);
+            return f;
+        };
+        for (size_t i = 0; i < ns; ++i) {
+            const SpiRec &x = P->spi[i];
+            sq[i] = make_float4(x.Pc[0], x.Pc[1], x.Pc[2], x.ext);
+            sr[i] = make_float4(x.S, x.S > 0.0f ? std::log(x.S) + 1e-5f : -1e30f, (float)(1.0 / (double)x.pmin * (1.0 + 1e-6)), bits(x.pp0));
+            P->ls_max = std::max(P->ls_max, sr[i].y);
+            int w;
+            memcpy(&w, &x.w, sizeof w);
+            sd[i] = make_int4(P->shells[x.I].ao, P->shells[x.J].ao, w, 0);
+        }
+        sr[ns] = make_float4(0.0f, -1e30f, 0.0f, bits((int)P->ppi.size()));
+        if ((rc = upload(sq, &P->d_spq, b)) || (rc = upload(sr, &P->d_spr, b)) || (rc = upload(sd, &P->d_spd, b))) return rc;
+    }
     if ((rc = upload(P->shells, &P->d_shells, b)) || (rc = upload(P->spi, &P->d_spi, b)) || (rc = upload(P->ppi, &P->d_ppi, b)) ||
         (rc = upload(P->spair, &P->d_spair, b)) || (rc = upload(P->spi_order, &P->d_spi_order, b)) ||
         (rc = upload(P->r1, &P->d_r1, b)) || (rc = upload(P->gvec, &P->d_gvec, b)) || (rc = upload(P->compf, &P->d_compf, b)))
@@ -1140,7 +1166,7 @@ void destroy_plan(Plan *P)
     release_cache(P);
     energy_release(P);
     void *ptrs[] = {P->d_shells, P->d_spi, P->d_ppi, P->d_ppf, P->d_ppB, P->d_pps, P->d_pplb, P->d_r1f, P->d_spair, P->d_spi_order, P->d_boys, P->d_boys_f, P->d_boys_t, P->d_r1, P->d_gvec,
-                    P->d_g0, P->d_compf, P->d_ppi_ab, P->d_kblk, P->d_kblk2, P->d_pvals, P->d_gtab0, P->d_ppi_pidx, P->d_phase, P->d_ppdf, P->d_gdf, P->d_phasef, P->ws.gtab, P->ws.gtab2, P->d_S, P->ws.Dp, P->ws.X, P->ws.Y, P->ws.JLR, P->ws.KLR, P->ws.T1, P->ws.T2,
+                    P->d_g0, P->d_compf, P->d_ppi_ab, P->d_kblk, P->d_kblk2, P->d_spq, P->d_spr, P->d_spd, P->d_pvals, P->d_gtab0, P->d_ppi_pidx, P->d_phase, P->d_ppdf, P->d_gdf, P->d_phasef, P->ws.gtab, P->ws.gtab2, P->d_S, P->ws.Dp, P->ws.X, P->ws.Y, P->ws.JLR, P->ws.KLR, P->ws.T1, P->ws.T2,
                     P->ws.M, P->ws.Z, P->ws.rho, P->ws.rho_part, P->ws.DhD, P->ws.JH, P->ws.DhF, P->ws.dmax, P->ws.scal, P->ws.err, P->ws.cnt, P->ws.big, P->ws.nbig,
                     P->ws.Ms, P->ws.Zs, P->ws.Ds, P->ws.Mex, P->ws.Zex, P->ws.Dex, P->ws.Dpf, P->ws.dmaxf, P->ws.Cs, P->ws.Cex, P->ws.Kpart,
                     P->ws.lr.Vt, P->ws.lr.diag, P->ws.lr.done_row, P->ws.lr.sgn, P->ws.lr.rowmap, P->ws.lr.dyn, P->ws.lr.bar, P->ws.lr.Ct};

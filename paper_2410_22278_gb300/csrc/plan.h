@@ -43,7 +43,7 @@ struct Workspace {
     double *rho_part = nullptr;  // [2*gc][kSlabSplitsMax] their partial sums
     double *dmax = nullptr;   // [nshell*nshell] max |D'| per shell block
     float *Dpf = nullptr;     // single-precision copies for the FP32 kernels (mixed precision)
-    float *dmaxf = nullptr;
+    float *dmaxf = nullptr;   // [nshell*nshell + 1] of dmax, then its largest value
     double *scal = nullptr;   // small scalars (traces, energies)
     // Coulomb-only builds (J-engine): per local primitive pair, hs Hermite
     // density values (FP64 and FP32) and hs Hermite J accumulators
@@ -148,6 +148,8 @@ struct Plan {
     // device arrays
     ShellRec *d_shells = nullptr;
     SpiRec *d_spi = nullptr;
+    float4 *d_spq = nullptr, *d_spr = nullptr;  // what the screening of image quartets reads, packed (jk_internal.h)
+    int4 *d_spd = nullptr;                      // what the digestion reads
     float4 *d_kblk = nullptr;  // per 32 consecutive images: bounding-sphere centre and radius (incl. extents)
     float2 *d_kblk2 = nullptr; // per 32 consecutive images: largest S, smallest pair exponent
     PpiRec *d_ppi = nullptr;
@@ -155,7 +157,7 @@ struct Plan {
     float *d_ppB = nullptr;  // |K| p^{-5/4} per primitive pair
     float4 *d_pps = nullptr;  // (P, 1/p) and ln(|K| p^{-5/4}) per primitive pair
     float *d_pplb = nullptr;
-    float lb_max = 0.0f;
+    float lb_max = 0.0f, ls_max = 0.0f;
     float *d_r1f = nullptr;
     SpairRec *d_spair = nullptr;
     int *d_spi_order = nullptr;

@@ -245,17 +245,15 @@ __device__ __forceinline__ void prim_term(const PlanDev &pl, const PrimE<LA, LB,
         }
 }
 
-// Digest the block V of the image quartet (bra sb, ket sk) with orbit weight
-// w: ket-side Coulomb X_kl += 2w sum_ij V D_ij (atomics), exchange in its
+// Digest the block V of an image quartet (first basis functions aoI .. aoL of
+// its shells, n in all) with orbit weight w: ket-side Coulomb X_kl += 2w sum_ij V D_ij (atomics), exchange in its
 // four index assignments (the other four of the orbit are transposes, added
 // at assembly), and the bra-side Coulomb term into the lane's jb.
 template <int LA, int LB, int LC, int LD, typename T>
-__device__ __forceinline__ void digest(const PlanDev &pl, const SpiRec &sb, const SpiRec &sk, const T *V, T w, const T *__restrict__ Dp,
-                                       const T *Dij, Acc<T> *jb, double *__restrict__ X, double *__restrict__ Y)
+__device__ __forceinline__ void digest(int n, int aoI, int aoJ, int aoK, int aoL, const T *V, T w, const T *__restrict__ Dp, const T *Dij,
+                                       Acc<T> *jb, double *__restrict__ X, double *__restrict__ Y)
 {
     constexpr int NA = ncart(LA), NB = ncart(LB), NC = ncart(LC), ND = ncart(LD);
-    const int n = pl.nbf;
-    const int aoI = pl.shells[sb.I].ao, aoJ = pl.shells[sb.J].ao, aoK = pl.shells[sk.I].ao, aoL = pl.shells[sk.J].ao;
     auto Dd = [&](int r, int c) { return __ldg(Dp + (size_t)r * n + c); };
 #pragma unroll
     for (int ab = 0; ab < NA * NB; ++ab) {
@@ -342,6 +340,86 @@ template <typename T>
 constexpr int tile_blocks(int L)
 {
     return sizeof(T) == 4 ? (L == 0 ? 6 : L <= 1 ? 5 : L <= 2 ? 4 : 3) : (L == 0 ? 4 : 3);
+}
+
+// Quartet-level screening of one image quartet from the packed records (spq,
+// spr): quartet_reaches of kernels.cuh with ln S instead of a logarithm per
+// pair and, for L > 0, one logarithm instead of two (Lc bounds the correction
+// inside it, so the sphere contains the former one).  big_bound receives
+// quartet_estimate_bound, brief whether [c_w, 1] is short (the two reasons to
+// look at the FP64 list).  All pairs of a launch come through here (7.2e9 for
+// (ss|ss) of the 64-water box, of which 17% pass); read from the 72-byte image
+// records with the density maxima of every passing pair it was 37% of the
+// kernel's time.
+template <int L>
+__device__ __forceinline__ bool pair_reaches(const PlanDev &pl, const float4 &bq, const float4 &br, const float4 &kq, const float4 &kr,
+                                             float Lc, float &big_bound, bool &brief)
+{
+    const float s = br.y + kr.y + (3.2094f - pl.log_ewald_R);  // ln(2 pi^{5/2} / sqrt 2) + 1e-3
+    if (!(s > 0.0f)) return false;
+    const float ipq = br.z + kr.z, inv = ipq + pl.inv_omega2f, aw = frcp_fast(inv);
+    float u = s;
+    if (L > 0) u += L * __logf(1.0f + 2.0f * fsqrt_fast(aw * (s + Lc)));
+    const float ext = bq.w + kq.w;
+    const float r = 1.0002f * fsqrt_fast(u * inv) + (L > 0 ? 0.5f + 0.25f * L : 0.0f) + ext + 1e-3f;
+    float X[3] = {bq.x - kq.x, bq.y - kq.y, bq.z - kq.z}, d2, e2;
+    if (pl.orth == 2) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) X[a] = fmaf(-(fmaf(X[a], pl.Finvf[4 * a], 12582912.0f) - 12582912.0f), pl.Lf[4 * a], X[a]);
+        d2 = e2 = X[0] * X[0] + X[1] * X[1] + X[2] * X[2];
+    } else {
+        float f[3], Y[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            f[a] = pl.Finvf[3 * a] * X[0] + pl.Finvf[3 * a + 1] * X[1] + pl.Finvf[3 * a + 2] * X[2];
+            f[a] -= rintf(f[a]);
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) Y[a] = f[0] * pl.Lf[a] + f[1] * pl.Lf[3 + a] + f[2] * pl.Lf[6 + a];
+        d2 = e2 = Y[0] * Y[0] + Y[1] * Y[1] + Y[2] * Y[2];
+        if (!pl.orth) {
+            // skewed: the rounded image need not be the nearest; plane spacings bound the distance
+            const float dp = fmaxf(fmaxf(pl.hplane[0] * fabsf(f[0]), pl.hplane[1] * fabsf(f[1])), pl.hplane[2] * fabsf(f[2]));
+            d2 = dp * dp;
+        }
+    }
+    const float dd = fmaxf(0.0f, fsqrt_fast(e2) - ext);
+    big_bound = 24.7394241f * 1.002f * br.x * kr.x * __expf(-0.9999f * aw * dd * dd);
+    brief = ipq > 0.7224f * (ipq + pl.inv_omega2f);
+    return d2 < r * r;
+}
+
+// Mixed precision: true if the image quartet (bra, kt) goes to the FP64 list,
+// decided as in k_real; called for the few that may (pair_reaches).
+template <typename T>
+__device__ __noinline__ bool list_quartet(const PlanDev &pl, int bra, int kt, float tauf, const T *__restrict__ dmax, int2 *__restrict__ big,
+                                          unsigned *__restrict__ nbig, unsigned cap, unsigned *__restrict__ ovf)
+{
+    const SpiRec sb = pl.spi[bra], sk = pl.spi[kt];
+    const float dm = quartet_dmax(reinterpret_cast<const float *>(dmax), pl.nshell, sb, sk);
+    const float est = quartet_estimate_bound(pl, sb, sk) * dm >= tauf ? quartet_estimate(pl, sb, sk) * dm : 0.0f;
+    const float ipq = frcp_fast(sb.pmin) + frcp_fast(sk.pmin);
+    if (!(est >= tauf || ipq > 0.7225f * (ipq + pl.inv_omega2f))) return false;
+    const unsigned slot = atomicAdd(nbig, 1u);
+    if (slot < cap) {
+        big[slot] = make_int2(bra, kt);
+        return true;
+    }
+    atomicAdd(ovf, 1u);
+    return false;
+}
+
+// Largest ln(1 + 2 alpha_w r) correction of a screening radius over the plan
+// (alpha_w r = sqrt(alpha_w u) <= omega sqrt(u), u the exponent at the edge).
+template <int L>
+__device__ __forceinline__ float radius_correction(const PlanDev &pl, float smax)
+{
+    if (L == 0) return 0.0f;
+    const float om2 = 2.0f * rsqrtf(pl.inv_omega2f);
+    float u = smax;
+#pragma unroll 1
+    for (int it = 0; it < 4; ++it) u = smax + L * __logf(1.0f + om2 * fsqrt_fast(fmaxf(u, 0.0f)));
+    return 1.05f * fmaxf(u - smax, 0.0f);
 }
 
 // First index in [lo, hi) whose primitive pairs start at or after `val` (hi if
@@ -452,7 +530,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, tile_blocks<T>(LA + LB + 
     int *kq = kq_s[wid], *kpp0 = pp0_s[wid];
     T *Vs = V_s[wid];
     const SpiRec sb = pl.spi[bra];
-    const int n = pl.nbf, nsh = pl.nshell;
+    const int n = pl.nbf;
     const int aoI = pl.shells[sb.I].ao, aoJ = pl.shells[sb.J].ao;
     T Dij[NA * NB];
     Acc<T> jb[NA * NB];
@@ -464,14 +542,11 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, tile_blocks<T>(LA + LB + 
     // constants of prim_maybe
     const float lbc = 3.2094f - pl.log_ewald_R;  // ln(2 pi^{5/2} / sqrt 2) + 1e-3
     const float r1min = pl.nr1 > 1 ? pl.r1f[7] : 1e30f;
-    float Lc = 0.0f;
-    if (L > 0) {
-        const float smax = 2.0f * pl.lb_max + lbc, om2 = 2.0f * rsqrtf(pl.inv_omega2f);
-        float u = smax;
-#pragma unroll 1
-        for (int it = 0; it < 4; ++it) u = smax + L * __logf(1.0f + om2 * fsqrt_fast(fmaxf(u, 0.0f)));
-        Lc = 1.05f * fmaxf(u - smax, 0.0f);
-    }
+    const float Lc = radius_correction<L>(pl, 2.0f * pl.lb_max + lbc);
+    const float Lq = radius_correction<L>(pl, 2.0f * pl.ls_max + lbc);  // the same for whole images
+    const float4 bq = __ldg(pl.spq + bra), br = __ldg(pl.spr + bra);
+    const bool policy = sizeof(T) == 4 && mode;
+    const float dall = policy ? (float)__ldg(dmax + (size_t)pl.nshell * pl.nshell) : 0.0f;
     Tally tl;
     unsigned used = 0, slots = 0;  // primitive quartets evaluated and lane slots offered
     unsigned nq = 0, kn = 0, kd = 0;
@@ -544,8 +619,9 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, tile_blocks<T>(LA + LB + 
             int np = 0;
             if (s0 + lane < count) {
                 const int kt = kq[(kd + s0 + lane) & (KQ - 1)];
-                np = pl.spi[kt].npp;
-                kpp0[s0 + lane] = pl.spi[kt].pp0;
+                const int first = __float_as_int(__ldg(&pl.spr[kt].w));
+                np = __float_as_int(__ldg(&pl.spr[kt + 1].w)) - first;
+                kpp0[s0 + lane] = first;
             }
             int incl = np;
 #pragma unroll
@@ -584,12 +660,19 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, tile_blocks<T>(LA + LB + 
                 // bra primitives in descending order of their bound: the first one
                 // below the magnitude threshold ends the loop
                 int i = 0;
+                float lb = __ldg(pl.pplb + sb.pp0 + ic);
+                float4 bv = __ldg(pl.pps + sb.pp0 + ic);
 #pragma unroll 1
                 for (; i < ie; ++i) {
-                    const float s = ks + __ldg(pl.pplb + sb.pp0 + ic + i);
+                    const float s = ks + lb;
                     if (!(s > 0.0f)) break;
                     ++tl.screen;
-                    if (prim_maybe<L>(pl, __ldg(pl.pps + sb.pp0 + ic + i), kv, s, Lc, r1min)) mask |= 1u << i;
+                    // the next one is on its way while this one is tested
+                    const float4 cur = bv;
+                    const int nx = sb.pp0 + ic + min(i + 1, ie - 1);
+                    lb = __ldg(pl.pplb + nx);
+                    bv = __ldg(pl.pps + nx);
+                    if (prim_maybe<L>(pl, cur, kv, s, Lc, r1min)) mask |= 1u << i;
                 }
                 const int cm = __popc(mask);
                 int pre = cm;
@@ -633,9 +716,9 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, tile_blocks<T>(LA + LB + 
             }
             if (any) {
                 const int kt = kq[(kd + sl) & (KQ - 1)];
-                const SpiRec sk = pl.spi[kt];
-                const T w = T(sb.w) * T(sk.w) * ((same && kt == bra) ? T(0.5) : T(1));
-                digest<LA, LB, LC, LD, T>(pl, sb, sk, V, w, Dp, Dij, jb, X, Y);
+                const int4 kd4 = __ldg(pl.spd + kt);
+                const T w = T(sb.w) * T(__int_as_float(kd4.z)) * ((same && kt == bra) ? T(0.5) : T(1));
+                digest<LA, LB, LC, LD, T>(n, aoI, aoJ, kd4.x, kd4.y, V, w, Dp, Dij, jb, X, Y);
             }
             ++tl.quart;
         }
@@ -654,23 +737,12 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, tile_blocks<T>(LA + LB + 
             bm &= bm - 1;
             bool valid = kt >= kbeg && kt < kend;
             if (valid) {
-                const SpiRec sk = pl.spi[kt];
-                valid = quartet_reaches<L>(pl, sb, sk);
-                if (sizeof(T) == 4 && valid && mode) {
-                    // precision policy: large quartets (and short [c_w, 1] intervals) go to the FP64 list
-                    const float dm = quartet_dmax(reinterpret_cast<const float *>(dmax), nsh, sb, sk);
-                    const float est = quartet_estimate_bound(pl, sb, sk) * dm >= tauf ? quartet_estimate(pl, sb, sk) * dm : 0.0f;
-                    const float ipq = frcp_fast(sb.pmin) + frcp_fast(sk.pmin);
-                    if (est >= tauf || ipq > 0.7225f * (ipq + pl.inv_omega2f)) {
-                        const unsigned slot = atomicAdd(nbig, 1u);
-                        if (slot < cap) {
-                            big[slot] = make_int2(bra, kt);
-                            valid = false;
-                        } else {
-                            atomicAdd(ovf, 1u);
-                        }
-                    }
-                }
+                float eb;
+                bool brief;
+                valid = pair_reaches<L>(pl, bq, br, __ldg(pl.spq + kt), __ldg(pl.spr + kt), Lq, eb, brief);
+                // large quartets (and short [c_w, 1] intervals) go to the FP64 list
+                if (policy && valid && (eb * dall >= tauf || brief))
+                    valid = !list_quartet(pl, bra, kt, tauf, dmax, big, nbig, cap, ovf);
             }
             const unsigned vmask = __ballot_sync(0xffffffffu, valid);
             nq += lane == 0 ? __popc(vmask) : 0;
@@ -992,7 +1064,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) k_real_list_w(PlanDev pl,
 #pragma unroll
                 for (int b = 0; b < NB; ++b) Dij[a * NB + b] = __ldg(Dp + (size_t)(aoI + a) * n + aoJ + b);
             const double w = double(sb.w) * double(sk.w) * ((same && pr.x == pr.y) ? 0.5 : 1.0);
-            digest<LA, LB, LC, LD, double>(pl, sb, sk, V, w, Dp, Dij, jb, X, Y);
+            digest<LA, LB, LC, LD, double>(n, aoI, aoJ, pl.shells[sk.I].ao, pl.shells[sk.J].ao, V, w, Dp, Dij, jb, X, Y);
             ++tl.quart;
 #pragma unroll
             for (int a = 0; a < NA; ++a)

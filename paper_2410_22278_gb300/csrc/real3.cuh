@@ -353,8 +353,11 @@ __global__ void __launch_bounds__(32) k_real_c(PlanDev pl, TileMap map, int k0, 
     int bra, kbeg, kend;
     if (!tile_of(pl, map, blockIdx.x, k0, k1, same, bra, kbeg, kend)) return;
     const SpiRec sb = pl.spi[bra];
-    const int nsh = pl.nshell;
     const float tauf = (float)tau;
+    const float Lq = radius_correction<L>(pl, 2.0f * pl.ls_max + 3.2094f - pl.log_ewald_R);
+    const float4 bq = __ldg(pl.spq + bra), br = __ldg(pl.spr + bra);
+    const bool policy = sizeof(T) == 4 && mode;
+    const float dall = policy ? (float)__ldg(dmax + (size_t)pl.nshell * pl.nshell) : 0.0f;
     Tally tl;
     unsigned nq = 0;
     bool ready = false;
@@ -362,22 +365,10 @@ __global__ void __launch_bounds__(32) k_real_c(PlanDev pl, TileMap map, int k0, 
         const int kt = kb + lane;
         bool valid = kt >= kbeg && kt < kend && block_reaches<L>(pl, sb, kb >> 5);
         if (valid) {
-            const SpiRec sk = pl.spi[kt];
-            valid = quartet_reaches<L>(pl, sb, sk);
-            if (sizeof(T) == 4 && valid && mode) {
-                const float dm = quartet_dmax(reinterpret_cast<const float *>(dmax), nsh, sb, sk);
-                const float est = quartet_estimate_bound(pl, sb, sk) * dm >= tauf ? quartet_estimate(pl, sb, sk) * dm : 0.0f;
-                const float ipq = frcp_fast(sb.pmin) + frcp_fast(sk.pmin);
-                if (est >= tauf || ipq > 0.7225f * (ipq + pl.inv_omega2f)) {
-                    const unsigned slot = atomicAdd(nbig, 1u);
-                    if (slot < cap) {
-                        big[slot] = make_int2(bra, kt);
-                        valid = false;
-                    } else {
-                        atomicAdd(ovf, 1u);
-                    }
-                }
-            }
+            float eb;
+            bool brief;
+            valid = pair_reaches<L>(pl, bq, br, __ldg(pl.spq + kt), __ldg(pl.spr + kt), Lq, eb, brief);
+            if (policy && valid && (eb * dall >= tauf || brief)) valid = !list_quartet(pl, bra, kt, tauf, dmax, big, nbig, cap, ovf);
         }
         unsigned m = __ballot_sync(0xffffffffu, valid);
         nq += __popc(m);
