@@ -57,14 +57,36 @@ __device__ __forceinline__ void two_sum_add(float &hi, float &lo, float x)
 
 }  // namespace
 
+// The first S digits of two adjacent values, stored as one bf16 pair per slice.
+// With W = V + sum_{s>=1} 128 * 2^{55 - 8s} + 64 the balanced digits are plain bits
+// of W: d_0 = W >> 55 and d_s = ((W >> (55 - 8s)) & 255) - 128 (V = sum_s d_s
+// 2^{55 - 8s} + the low bits - 64, identically), so a digit costs a shift, a mask
+// and one exact float subtraction instead of a 64-bit rounding, shift, multiply
+// and subtraction and an integer conversion (which runs at an eighth of the
+// FP32 rate); the slicing is left to the memory system.
+__device__ __forceinline__ float digit_f(unsigned byte) { return __uint_as_float(0x4b000000u | byte) - 8388736.0f; }  // 2^23 + 128
+__device__ __forceinline__ void store_digits(long long V0, long long V1, int S, __nv_bfloat16 *o, size_t sstride)
+{
+    constexpr long long B = (128LL << 47) + (128LL << 39) + (128LL << 31) + (128LL << 23) + (128LL << 15) + (128LL << 7) + 64;
+    const long long W0 = V0 + B, W1 = V1 + B;
+    const int t0 = (int)(W0 >> 55), t1 = (int)(W1 >> 55);  // in [-128, 128]
+    *reinterpret_cast<__nv_bfloat162 *>(o) =
+        __floats2bfloat162_rn(__int_as_float(0x4b400000 + t0) - 12582912.0f, __int_as_float(0x4b400000 + t1) - 12582912.0f);
+#pragma unroll
+    for (int s = 1; s < 7; ++s)
+        if (s < S)
+            *reinterpret_cast<__nv_bfloat162 *>(o + s * sstride) =
+                __floats2bfloat162_rn(digit_f((unsigned)(W0 >> (55 - 8 * s)) & 255u), digit_f((unsigned)(W1 >> (55 - 8 * s)) & 255u));
+}
+
 // Slices of a batch of rows x cols FP64 matrices (row-major, leading dim ld,
 // batch stride bstride elements): one warp per row.  sigma = E_max - 1022
 // with E_max the largest biased exponent in the row (so |x| < 2^sigma);
 // V = x 2^{62 - sigma} (|V| < 2^62) is formed exactly as a signed 64-bit
-// integer by shifting the 53-bit significand, and the digits are taken from
-// the top by rounding to nearest: d_s = round(V_s / 2^{55 - 8s}),
-// V_{s+1} = V_s - d_s 2^{55 - 8s}, so |V_{s+1}| <= 2^{54 - 8s} and the next
-// digit again lies in [-128, 128].  S <= 7.  Output:
+// integer by shifting the 53-bit significand, and the digits are read off
+// store_digits' shifted form: d_0 in [-128, 128], the others in [-128, 127],
+// and what is left after S of them is at most 0.51 of the last place.  S <= 7.
+// Output:
 // out[((b*S + s)*rows_pad + r)*cols_pad + k] (zero outside rows x cols),
 // ex[b*rows_pad + r].
 __global__ void k_ozaki_slice(const double *__restrict__ X, int rows, int cols, int ld, long long bstride, int rows_pad, int cols_pad,
@@ -98,14 +120,7 @@ __global__ void k_ozaki_slice(const double *__restrict__ X, int rows, int cols, 
     // (cols_pad and the slice stride are even)
     for (int k = 2 * lane; k < cols_pad; k += 64) {
         long long V0 = scaled(k), V1 = scaled(k + 1);
-        for (int s = 0; s < S; ++s) {
-            const int shift = 55 - 8 * s;
-            const long long d0 = (V0 + (1LL << (shift - 1))) >> shift;  // arithmetic shift: floor
-            const long long d1 = (V1 + (1LL << (shift - 1))) >> shift;
-            V0 -= d0 * (1LL << shift);
-            V1 -= d1 * (1LL << shift);
-            *reinterpret_cast<__nv_bfloat162 *>(o + s * sstride + k) = __floats2bfloat162_rn((float)d0, (float)d1);
-        }
+        store_digits(V0, V1, S, o + k, sstride);
     }
 }
 
@@ -501,14 +516,7 @@ __global__ void k_ozaki_slice_pair(const float2 *__restrict__ X, int rows, int c
                 V1 = part(x.x) + part(x.y);
             }
         }
-        for (int s = 0; s < S; ++s) {
-            const int shift = 55 - 8 * s;
-            const long long d0 = (V0 + (1LL << (shift - 1))) >> shift;  // arithmetic shift: floor
-            const long long d1 = (V1 + (1LL << (shift - 1))) >> shift;
-            V0 -= d0 * (1LL << shift);
-            V1 -= d1 * (1LL << shift);
-            *reinterpret_cast<__nv_bfloat162 *>(o + s * sstride + k) = __floats2bfloat162_rn((float)d0, (float)d1);
-        }
+        store_digits(V0, V1, S, o + k, sstride);
     }
 }
 
