@@ -109,6 +109,7 @@ struct PlanDev {
     const float4 *pps;           // (P, 1/p) of each primitive pair and ln B (rounded up): the screening of real2.cuh
     const float *pplb;
     float lb_max, ls_max;        // largest ln B and ln S
+    int img_share;               // share the images of a batch out over the lanes (a small cell, lattice vectors fit 11 bits)
     float mag_thr;               // B_i B_j below this: the primitive quartet is below the real-space threshold
     const double *r1;            // [nr1][4]: x, y, z, |R|, sorted by |R|
     const float *r1f;            // the same in single precision

@@ -94,7 +94,7 @@ __device__ __forceinline__ void seeds(float x2, float alpha, float aw, float cw,
 {
     (void)aw;
     float G[L + 1];
-    boys_attenuated<L, float>(alpha * x2, cw, pl.boys_f, G);
+    boys_attenuated<L>(alpha * x2, cw, pl.boys_f, G);
     float f = 1.0f;
 #pragma unroll
     for (int m = 0; m <= L; ++m) {

@@ -371,6 +371,14 @@ PlanDev Plan::dev() const
     d.ppB = d_ppB;
     d.pps = d_pps;
     d.pplb = d_pplb;
+    // Sharing costs a batch about 150 instructions and saves the rounds beyond
+    // the mean image count: worth it where a sphere of the mean radius holds
+    // more than about two images.  The screening radius of the middle of the
+    // range of magnitudes, r = sqrt(ln(1e13) / 2) / omega, decides.
+    {
+        const double r = 3.87 / omega;
+        d.img_share = 4.19 * r * r * r > 2.0 * volume && r1.size() / 4 <= 2048;
+    }
     d.lb_max = lb_max;
     d.ls_max = ls_max;
     d.mag_thr = (float)(cut.ewald_R * 1e-1 / (24.739424126 * 1.001));

@@ -15,9 +15,8 @@
 // pbc_eri_real_cutoff_implementation fails for it and for every later one.
 // Which kernel family (this one, the lane-per-bra one of kernels.cuh or the
 // pair-queue one below) runs a class pair is chosen by the autotuner.
-// The FP64 pass over the large quartets of the mixed path likewise gives one
-// list entry to a whole warp: its primitive quartets are screened 32 at a
-// time, queued, evaluated one per lane and summed by a full warp reduction.
+// The FP64 pass over the large quartets of the mixed path refills its lanes the
+// same way, from groups of list entries (k_real_list_w).
 #pragma once
 #include "kernels.cuh"
 #include "launch.h"
@@ -113,88 +112,126 @@ __device__ __forceinline__ void alphas(double ipq, double iw2, double &alpha, do
 }
 __device__ __forceinline__ void alphas(float ipq, float iw2, float &alpha, float &aw, float &cw)
 {
-    aw = 1.0f / (ipq + iw2);
-    alpha = 1.0f / ipq;
-    cw = sqrtf(aw * ipq);
+    aw = rcp_nr(ipq + iw2);
+    alpha = rcp_nr(ipq);
+    cw = sqrt_nr(aw * ipq);
+}
+__device__ __forceinline__ double inv_sqrt(double x) { return rsqrt(x); }
+__device__ __forceinline__ float inv_sqrt(float x) { return rsqrt_nr(x); }
+
+// Geometry of one primitive quartet: its screening sphere, the nearest image
+// of P - Q (single precision F0 for the image search, X0 for the terms) and
+// its exponents.
+template <typename T>
+struct PrimGeo {
+    float F0[3], r, x0n;
+    T X0[3], alpha, aw, cw;
+};
+
+template <int L, typename T>
+__device__ __forceinline__ bool prim_geo(const PlanDev &pl, const PairT<T> &x, const PpiF &bf, const PairT<T> &y, const PpiF &kf,
+                                         PrimGeo<T> &g, Tally &tl)
+{
+    ++tl.screen;
+    if (!prim_radius<L>(pl, bf, kf, g.r)) return false;
+    ++tl.radius;
+    float f[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        g.F0[a] = bf.P[a] - kf.P[a];
+        g.X0[a] = x.P[a] - y.P[a];
+    }
+    if (pl.orth == 2) {
+        // diagonal lattice: rounding by adding and subtracting 1.5 * 2^23
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            f[a] = fmaf(g.F0[a], pl.Finvf[4 * a], 12582912.0f) - 12582912.0f;
+            g.F0[a] = fmaf(-f[a], pl.Lf[4 * a], g.F0[a]);
+        }
+        if (sizeof(T) == 4 || f[0] != 0.0f || f[1] != 0.0f || f[2] != 0.0f)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) g.X0[a] -= T(f[a]) * latc(pl.L, pl.Lf, 4 * a, T(0));
+    } else {
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            f[a] = rintf(pl.Finvf[3 * a] * g.F0[0] + pl.Finvf[3 * a + 1] * g.F0[1] + pl.Finvf[3 * a + 2] * g.F0[2]);
+        if (f[0] != 0.0f || f[1] != 0.0f || f[2] != 0.0f) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                g.F0[a] -= f[0] * pl.Lf[a] + f[1] * pl.Lf[3 + a] + f[2] * pl.Lf[6 + a];
+                g.X0[a] -= T(f[0]) * latc(pl.L, pl.Lf, a, T(0)) + T(f[1]) * latc(pl.L, pl.Lf, 3 + a, T(0)) +
+                           T(f[2]) * latc(pl.L, pl.Lf, 6 + a, T(0));
+            }
+        }
+    }
+    g.x0n = fsqrt_fast(g.F0[0] * g.F0[0] + g.F0[1] * g.F0[1] + g.F0[2] * g.F0[2]);
+    alphas(x.ip + y.ip, latc(&pl.inv_omega2, &pl.inv_omega2f, 0, T(0)), g.alpha, g.aw, g.cw);
+    return true;
 }
 
-// One primitive quartet (bra pair b, ket pair k): screening radius, minimum
-// image, the R1 images inside the sphere, seeds and the Hermite R table, then
-// the contraction with both E tables into the Cartesian block V; the events
-// go to the lane's tally (flops.h).  The image search runs in single
-// precision (it only decides which terms are formed) and each lane walks on
-// to its next image inside the sphere before the terms are formed, so the
-// lanes of a warp form them together; with the test and the term in one loop
-// body the lanes whose candidate failed waited for the others.
+// Index of the first lattice vector from c on whose image lies inside the
+// sphere, pl.nr1 if there is none.
+template <typename T>
+__device__ __forceinline__ int next_image(const PlanDev &pl, const PrimGeo<T> &g, int c, Tally &tl)
+{
+    const float4 *lat = reinterpret_cast<const float4 *>(pl.r1f);
+    const float r2 = g.r * g.r;
+#pragma unroll 1
+    for (; c < pl.nr1; ++c) {
+        const float4 R = __ldg(lat + c);
+        if (R.w - g.x0n >= g.r) break;
+        ++tl.cand;
+        const float fx = g.F0[0] - R.x, fy = g.F0[1] - R.y, fz = g.F0[2] - R.z;
+        if (fx * fx + fy * fy + fz * fz < r2) return c;
+    }
+    return pl.nr1;
+}
+
+// Rs += Hermite R table of the image c.
+template <int L, typename T>
+__device__ __forceinline__ void add_image(const PlanDev &pl, const T *X0, T alpha, T aw, T cw, int c, T *Rs)
+{
+    constexpr int D = L + 1;
+    const T Xx = X0[0] - lat_at(pl, 4 * c, T(0)), Xy = X0[1] - lat_at(pl, 4 * c + 1, T(0)), Xz = X0[2] - lat_at(pl, 4 * c + 2, T(0));
+    T s[L + 1];
+    seeds<L>(Xx * Xx + Xy * Xy + Xz * Xz, alpha, aw, cw, pl, s);
+    T Bt[D * D * D];
+    herm_R<L, T>(s, Xx, Xy, Xz, Bt);
+#pragma unroll
+    for (int t = 0; t <= L; ++t)
+#pragma unroll
+        for (int u = 0; u <= L - t; ++u)
+#pragma unroll
+            for (int v = 0; v <= L - t - u; ++v) Rs[(t * D + u) * D + v] += Bt[(t * D + u) * D + v];
+}
+
+// One lane's images one after another; false if there is none.  The image
+// search runs in single precision (it only decides which terms are formed)
+// and each lane walks on to its next image before the terms are formed, so
+// the lanes of a warp form them together.
+template <int L, typename T>
+__device__ __forceinline__ bool all_images(const PlanDev &pl, const PrimGeo<T> &g, T *Rs, Tally &tl)
+{
+    int n = 0;
+#pragma unroll 1
+    for (int c = next_image(pl, g, 0, tl); c < pl.nr1; c = next_image(pl, g, c + 1, tl)) {
+        add_image<L, T>(pl, g.X0, g.alpha, g.aw, g.cw, c, Rs);
+        ++n;
+    }
+    tl.img += n;
+    return n > 0;
+}
+
+// V += contraction of the Hermite table Rs of one primitive quartet with both
+// E tables.
 template <int LA, int LB, int LC, int LD, typename T>
-__device__ __forceinline__ void prim_term(const PlanDev &pl, const PrimE<LA, LB, T> &b, const PpiF &bf, const PrimE<LC, LD, T> &k,
-                                          const PpiF &kf, T *V, Tally &tl)
+__device__ __forceinline__ void contract(const PrimE<LA, LB, T> &b, const PrimE<LC, LD, T> &k, const T *Rs, T *V)
 {
     constexpr int NA = ncart(LA), NB = ncart(LB), NC = ncart(LC), ND = ncart(LD);
     constexpr int L = LA + LB + LC + LD, LAB = LA + LB, LCD = LC + LD;
     constexpr int NTA = LAB + 1, NTC = LCD + 1, D = L + 1;
-    ++tl.screen;
-    float r;
-    if (!prim_radius<L>(pl, bf, kf, r)) return;
-    ++tl.radius;
-    const float r2 = r * r;
     const PairT<T> &x = b.x, &y = k.x;
-    float F0[3] = {bf.P[0] - kf.P[0], bf.P[1] - kf.P[1], bf.P[2] - kf.P[2]}, f[3];
-    T X0[3] = {x.P[0] - y.P[0], x.P[1] - y.P[1], x.P[2] - y.P[2]};
-#pragma unroll
-    for (int a = 0; a < 3; ++a) f[a] = rintf(pl.Finvf[3 * a] * F0[0] + pl.Finvf[3 * a + 1] * F0[1] + pl.Finvf[3 * a + 2] * F0[2]);
-    if (f[0] != 0.0f || f[1] != 0.0f || f[2] != 0.0f) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            F0[a] -= f[0] * pl.Lf[a] + f[1] * pl.Lf[3 + a] + f[2] * pl.Lf[6 + a];
-            X0[a] -= T(f[0]) * latc(pl.L, pl.Lf, a, T(0)) + T(f[1]) * latc(pl.L, pl.Lf, 3 + a, T(0)) + T(f[2]) * latc(pl.L, pl.Lf, 6 + a, T(0));
-        }
-    }
-    const float x0n = fsqrt_fast(F0[0] * F0[0] + F0[1] * F0[1] + F0[2] * F0[2]);
-    T Rs[D * D * D];
-#pragma unroll
-    for (int q = 0; q < D * D * D; ++q) Rs[q] = T(0);
-    bool any = false;
-    const T ip = x.ip, iq = y.ip;
-    T alpha, aw, cw;
-    alphas(ip + iq, latc(&pl.inv_omega2, &pl.inv_omega2f, 0, T(0)), alpha, aw, cw);
-    const float4 *lat = reinterpret_cast<const float4 *>(pl.r1f);
-    int c = 0;
-#pragma unroll 1
-    while (true) {
-        bool hit = false;
-#pragma unroll 1
-        while (c < pl.nr1) {
-            const float4 R = __ldg(lat + c);
-            if (R.w - x0n >= r) break;
-            ++tl.cand;
-            const float fx = F0[0] - R.x, fy = F0[1] - R.y, fz = F0[2] - R.z;
-            if (fx * fx + fy * fy + fz * fz < r2) {
-                hit = true;
-                break;
-            }
-            ++c;
-        }
-        if (!hit) break;
-        const T Xx = X0[0] - lat_at(pl, 4 * c, T(0)), Xy = X0[1] - lat_at(pl, 4 * c + 1, T(0)), Xz = X0[2] - lat_at(pl, 4 * c + 2, T(0));
-        const T x2 = Xx * Xx + Xy * Xy + Xz * Xz;
-        ++c;
-        any = true;
-        ++tl.img;
-        T s[L + 1];
-        seeds<L>(x2, alpha, aw, cw, pl, s);
-        T Bt[D * D * D];
-        herm_R<L, T>(s, Xx, Xy, Xz, Bt);
-#pragma unroll
-        for (int t = 0; t <= L; ++t)
-#pragma unroll
-            for (int u = 0; u <= L - t; ++u)
-#pragma unroll
-                for (int v = 0; v <= L - t - u; ++v) Rs[(t * D + u) * D + v] += Bt[(t * D + u) * D + v];
-    }
-    if (!any) return;
-    ++tl.term;
-    const T tp = T(kTwoPi52) * x.K * y.K * ip * iq / sqrt(x.p + y.p);
+    const T tp = T(kTwoPi52) * x.K * y.K * x.ip * y.ip * inv_sqrt(x.p + y.p);
 #pragma unroll
     for (int c = 0; c < NC; ++c)
 #pragma unroll
@@ -243,6 +280,23 @@ __device__ __forceinline__ void prim_term(const PlanDev &pl, const PrimE<LA, LB,
                     V[((a * NB + bb) * NC + c) * ND + d] += tp * v;
                 }
         }
+}
+
+// One primitive quartet (bra pair b, ket pair k) into the Cartesian block V;
+// the events go to the lane's tally (flops.h).
+template <int LA, int LB, int LC, int LD, typename T>
+__device__ __forceinline__ void prim_term(const PlanDev &pl, const PrimE<LA, LB, T> &b, const PpiF &bf, const PrimE<LC, LD, T> &k,
+                                          const PpiF &kf, T *V, Tally &tl)
+{
+    constexpr int L = LA + LB + LC + LD, D = L + 1;
+    PrimGeo<T> g;
+    if (!prim_geo<L, T>(pl, b.x, bf, k.x, kf, g, tl)) return;
+    T Rs[D * D * D];
+#pragma unroll
+    for (int q = 0; q < D * D * D; ++q) Rs[q] = T(0);
+    if (!all_images<L, T>(pl, g, Rs, tl)) return;
+    ++tl.term;
+    contract<LA, LB, LC, LD, T>(b, k, Rs, V);
 }
 
 // Digest the block V of an image quartet (first basis functions aoI .. aoL of
@@ -328,11 +382,12 @@ constexpr int kWarpsPerBlock = 4;
 template <int NV, typename T>
 struct BatchShape {
     static constexpr int per = NV * (int)sizeof(T);
-    static constexpr int SL = per <= 24 ? 128 : per <= 72 ? 64 : per <= 144 ? 32 : per <= 216 ? 16 : 8;
+    static constexpr int SL = per <= 24 ? 128 : per <= 36 ? 64 : per <= 144 ? 32 : per <= 216 ? 16 : 8;
     static constexpr int KQ = SL == 128 ? 256 : SL == 64 ? 128 : 64;  // ring of queued kets, at least SL + 31
 };
 constexpr int kBraChunk = 16;    // bra primitives screened per round (bits of a lane's mask)
 constexpr int kTermRing = 1024;  // at most 31 + 32 * kBraChunk entries are in flight
+constexpr int kListRing = 64;    // of the list kernel: at most 31 + 32
 
 // Resident blocks asked for: the FP32 kernels of low momentum wait on
 // dependent instructions and need the warps (24 per SM: at most 85 registers).
@@ -422,6 +477,108 @@ __device__ __forceinline__ float radius_correction(const PlanDev &pl, float smax
     return 1.05f * fmaxf(u - smax, 0.0f);
 }
 
+// Images of a batch of primitive quartets shared out evenly over the lanes of
+// a warp (FP64, total momentum up to 2, where the sum of the R table over lanes
+// is cheap).  A small cell has several images per primitive quartet, one to
+// twenty: lane by lane, the batch takes as many rounds as its largest count,
+// three times the mean, and an FP64 instruction costs the same however few
+// lanes take part.  FP64 build of 6 water molecules: (ss|ss) 49.7 -> 25.7 ms,
+// (ss|ps) 49.5 -> 37.2 ms.  In single precision the bookkeeping cost more than
+// it saved ((ss|ss) of 5 molecules 7.0 -> 10.0 ms), and so it did for the
+// listed quartets, which have ten and more images each.
+constexpr int kImgRound = 8;  // images a lane lists per round
+template <int L, typename T>
+struct ImgShare {
+    static constexpr bool on = L <= 2 && sizeof(T) == 8;
+    unsigned short list[on ? 32 * kImgRound : 1];  // owner lane and lattice vector
+    T R[on ? 32 * nherm(L) : 1];                    // sums of the owners' R tables
+};
+
+// Rs = R table of the lane's primitive quartet (g, if act), summed over its
+// images; every lane of the warp calls this.  n and total: images of this lane
+// and of the warp.
+template <int L, typename T>
+__device__ __forceinline__ void shared_images(const PlanDev &pl, const PrimGeo<T> &g, int n, ImgShare<L, T> &sh, T *Rs)
+{
+    constexpr int D = L + 1, NH = nherm(L);
+    const int lane = threadIdx.x & 31;
+    Tally none;
+#pragma unroll
+    for (int h = 0; h < NH; ++h) sh.R[h * 32 + lane] = T(0);
+    int c = -1;
+#pragma unroll 1
+    while (__any_sync(0xffffffffu, n > 0)) {
+        const int now = min(n, kImgRound);
+        int pos = now;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, pos, o);
+            if (lane >= o) pos += t;
+        }
+        const int total = __shfl_sync(0xffffffffu, pos, 31);
+        pos -= now;
+#pragma unroll 1
+        for (int i = 0; i < now; ++i) {
+            c = next_image(pl, g, c + 1, none);
+            sh.list[pos + i] = (unsigned short)(lane << 11 | c);
+        }
+        n -= now;
+        __syncwarp();
+#pragma unroll 1
+        for (int e0 = 0; e0 < total; e0 += 32) {
+            const bool on = e0 + lane < total;
+            const unsigned it = on ? sh.list[e0 + lane] : 0u;
+            const int src = (int)(it >> 11);
+            T X0[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) X0[a] = __shfl_sync(0xffffffffu, g.X0[a], src);
+            const T alpha = __shfl_sync(0xffffffffu, g.alpha, src), aw = __shfl_sync(0xffffffffu, g.aw, src),
+                    cw = __shfl_sync(0xffffffffu, g.cw, src);
+            T Ri[D * D * D];
+#pragma unroll
+            for (int q = 0; q < D * D * D; ++q) Ri[q] = T(0);
+            if (on) add_image<L, T>(pl, X0, alpha, aw, cw, (int)(it & 2047u), Ri);
+            __syncwarp();
+            // sum over the lanes of one owner (adjacent), then its first lane adds
+            const int key = on ? src : 32 + lane;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int ok = __shfl_down_sync(0xffffffffu, key, o);
+                const bool add = lane + o < 32 && ok == key;
+                if (!__any_sync(0xffffffffu, add)) break;
+#pragma unroll
+                for (int t = 0; t <= L; ++t)
+#pragma unroll
+                    for (int u = 0; u <= L - t; ++u)
+#pragma unroll
+                        for (int v = 0; v <= L - t - u; ++v) {
+                            const T y = __shfl_down_sync(0xffffffffu, Ri[(t * D + u) * D + v], o);
+                            if (add) Ri[(t * D + u) * D + v] += y;
+                        }
+            }
+            const int prev = __shfl_up_sync(0xffffffffu, key, 1);
+            if (on && (lane == 0 || prev != key)) {
+                int h = 0;
+#pragma unroll
+                for (int t = 0; t <= L; ++t)
+#pragma unroll
+                    for (int u = 0; u <= L - t; ++u)
+#pragma unroll
+                        for (int v = 0; v <= L - t - u; ++v, ++h) sh.R[h * 32 + src] += Ri[(t * D + u) * D + v];
+            }
+            __syncwarp();
+        }
+    }
+    int h = 0;
+#pragma unroll
+    for (int t = 0; t <= L; ++t)
+#pragma unroll
+        for (int u = 0; u <= L - t; ++u)
+#pragma unroll
+            for (int v = 0; v <= L - t - u; ++v, ++h) Rs[(t * D + u) * D + v] = sh.R[h * 32 + lane];
+    __syncwarp();
+}
+
 // First index in [lo, hi) whose primitive pairs start at or after `val` (hi if
 // none); the whole warp searches, 32 probes per step.
 __device__ __forceinline__ int first_at(const SpiRec *__restrict__ spi, int lo, int hi, long long val)
@@ -483,6 +640,105 @@ __device__ __forceinline__ bool prim_maybe(const PlanDev &pl, const float4 &b, c
     return x2 < r * r || (!pl.orth && r1min - fsqrt_fast(x2) < r);
 }
 
+// Evaluate count (<= 32) queued primitive quartets from ring position qd on,
+// one per lane, and add the lanes of each image quartet into its block Vs[slot].
+// A ring entry holds the slot, the positions i and j of the bra and ket
+// primitive pairs in their images (first ones: bra0(slot), ket0(slot)) and a
+// group: the entries of one slot and group are adjacent.  several: a slot may
+// come with more than one group.
+template <int LA, int LB, int LC, int LD, typename T, int RING, bool SHARE, class BraFn, class KetFn>
+__device__ __forceinline__ void eval_terms(const PlanDev &pl, const unsigned *ring, unsigned qd, unsigned count, BraFn bra0, KetFn ket0,
+                                           bool several, T *Vs, Tally &tl, unsigned &used, bool share = false,
+                                           ImgShare<LA + LB + LC + LD, T> *img = nullptr)
+{
+    constexpr int NV = ncart(LA) * ncart(LB) * ncart(LC) * ncart(LD), L = LA + LB + LC + LD;
+    const int lane = threadIdx.x & 31;
+    const bool on = lane < count;
+    unsigned key = 0xffffff80u + lane;  // a segment of its own (group 511 is not used)
+    T V[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) V[q] = T(0);
+    if constexpr (SHARE) {
+        PrimE<LA, LB, T> bp;
+        PrimE<LC, LD, T> kp;
+        PpiF bf, kf;
+        PrimGeo<T> g;
+        bool act = false;
+        if (on) {
+            const unsigned it = ring[(qd + lane) & (RING - 1)];
+            key = it & 0xff80007fu;
+            load_prim<LA, LB, T>(pl, bra0(it & 127u) + (int)((it >> 7) & 255u), bp, bf);
+            load_prim<LC, LD, T>(pl, ket0(it & 127u) + (int)((it >> 15) & 255u), kp, kf);
+            ++tl.brap;
+            ++tl.ketp;
+            act = prim_geo<L, T>(pl, bp.x, bf, kp.x, kf, g, tl);
+            ++used;
+        }
+        T Rs[(L + 1) * (L + 1) * (L + 1)];
+#pragma unroll
+        for (int q = 0; q < (L + 1) * (L + 1) * (L + 1); ++q) Rs[q] = T(0);
+        if (share) {
+            int n = 0;
+            if (act)
+#pragma unroll 1
+                for (int c = next_image(pl, g, 0, tl); c < pl.nr1; c = next_image(pl, g, c + 1, tl)) ++n;
+            tl.img += n;
+            act = n > 0;
+            shared_images<L, T>(pl, g, n, *img, Rs);
+        } else if (act) {
+            act = all_images<L, T>(pl, g, Rs, tl);
+        }
+        if (act) {
+            ++tl.term;
+            contract<LA, LB, LC, LD, T>(bp, kp, Rs, V);
+        }
+    } else if (on) {
+        const unsigned it = ring[(qd + lane) & (RING - 1)];
+        key = it & 0xff80007fu;
+        PrimE<LA, LB, T> bp;
+        PrimE<LC, LD, T> kp;
+        PpiF bf, kf;
+        load_prim<LA, LB, T>(pl, bra0(it & 127u) + (int)((it >> 7) & 255u), bp, bf);
+        load_prim<LC, LD, T>(pl, ket0(it & 127u) + (int)((it >> 15) & 255u), kp, kf);
+        ++tl.brap;
+        ++tl.ketp;
+        prim_term<LA, LB, LC, LD, T>(pl, bp, bf, kp, kf, V, tl);
+        ++used;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned ok = __shfl_down_sync(0xffffffffu, key, o);
+        const bool add = lane + o < 32 && ok == key;
+        if (!__any_sync(0xffffffffu, add)) break;
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            const T t = __shfl_down_sync(0xffffffffu, V[q], o);
+            if (add) V[q] += t;
+        }
+    }
+    const unsigned prev = __shfl_up_sync(0xffffffffu, key, 1);
+    const bool head = on && (lane == 0 || prev != key);
+    T *dst = Vs + (head ? key & 127u : 0u) * NV;
+    if (!several) {
+        if (head)
+#pragma unroll
+            for (int q = 0; q < NV; ++q) dst[q] += V[q];
+    } else {
+        // one slot can head several segments here: one after another
+        const unsigned m = __match_any_sync(0xffffffffu, head ? (key & 127u) : 128u + lane);
+        const int rank = __popc(m & ((1u << lane) - 1u));
+#pragma unroll 1
+        for (int rr = 0; __any_sync(0xffffffffu, head && rank >= rr); ++rr) {
+            if (head && rank == rr)
+#pragma unroll
+                for (int q = 0; q < NV; ++q) dst[q] += V[q];
+            __syncwarp();
+        }
+    }
+    __syncwarp();
+}
+
 // Warp-per-bra tile kernel.  Block = 4 warps, each with a bra and a range of
 // kets (TileMap).  mode and the FP64 list as in k_real.
 //   1. 32 kets at a time are tested (block bound, quartet bound, precision
@@ -522,6 +778,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, tile_blocks<T>(LA + LB + 
     __shared__ unsigned ring_s[kWarpsPerBlock][kTermRing];
     __shared__ int kq_s[kWarpsPerBlock][KQ], pp0_s[kWarpsPerBlock][SL];
     __shared__ T V_s[kWarpsPerBlock][SL * NV];
+    __shared__ ImgShare<L, T> img_s[kWarpsPerBlock];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int bra, kbeg, kend;
     // whole warps return; no block-wide barrier below
@@ -542,6 +799,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, tile_blocks<T>(LA + LB + 
     // constants of prim_maybe
     const float lbc = 3.2094f - pl.log_ewald_R;  // ln(2 pi^{5/2} / sqrt 2) + 1e-3
     const float r1min = pl.nr1 > 1 ? pl.r1f[7] : 1e30f;
+    const bool share = pl.img_share;  // several images per primitive quartet
     const float Lc = radius_correction<L>(pl, 2.0f * pl.lb_max + lbc);
     const float Lq = radius_correction<L>(pl, 2.0f * pl.ls_max + lbc);  // the same for whole images
     const float4 bq = __ldg(pl.spq + bra), br = __ldg(pl.spr + bra);
@@ -551,63 +809,14 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, tile_blocks<T>(LA + LB + 
     unsigned used = 0, slots = 0;  // primitive quartets evaluated and lane slots offered
     unsigned nq = 0, kn = 0, kd = 0;
 
-    // evaluate the next count queued primitive quartets, one per lane, and add
-    // the lanes of each ket into its block
     unsigned qn = 0, qd = 0;
+    // evaluate the next count queued primitive quartets
     auto eval = [&](unsigned count) {
-        const bool on = lane < count;
-        unsigned key = 0xffffff80u + lane;  // a segment of its own (group 511 is not used)
-        T V[NV];
-#pragma unroll
-        for (int q = 0; q < NV; ++q) V[q] = T(0);
-        if (on) {
-            const unsigned it = ring[(qd + lane) & (kTermRing - 1)];
-            key = it & 0xff80007fu;
-            const int ib = sb.pp0 + (int)((it >> 7) & 255u), ik = kpp0[it & 127u] + (int)((it >> 15) & 255u);
-            PrimE<LA, LB, T> bp;
-            PrimE<LC, LD, T> kp;
-            PpiF bf, kf;
-            load_prim<LA, LB, T>(pl, ib, bp, bf);
-            load_prim<LC, LD, T>(pl, ik, kp, kf);
-            ++tl.brap;
-            ++tl.ketp;
-            prim_term<LA, LB, LC, LD, T>(pl, bp, bf, kp, kf, V, tl);
-            ++used;
-        }
+        eval_terms<LA, LB, LC, LD, T, kTermRing, ImgShare<L, T>::on>(
+            pl, ring, qd, count, [&](unsigned) { return sb.pp0; }, [&](unsigned slot) { return kpp0[slot]; }, sb.npp > kBraChunk, Vs, tl,
+            used, share, &img_s[wid]);
         slots += lane == 0 ? 32u : 0u;
-        __syncwarp();
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned ok = __shfl_down_sync(0xffffffffu, key, o);
-            const bool add = lane + o < 32 && ok == key;
-            if (!__any_sync(0xffffffffu, add)) break;
-#pragma unroll
-            for (int q = 0; q < NV; ++q) {
-                const T t = __shfl_down_sync(0xffffffffu, V[q], o);
-                if (add) V[q] += t;
-            }
-        }
-        const unsigned prev = __shfl_up_sync(0xffffffffu, key, 1);
-        const bool head = on && (lane == 0 || prev != key);
-        T *dst = Vs + (head ? key & 127u : 0u) * NV;
-        if (sb.npp <= kBraChunk) {
-            if (head)
-#pragma unroll
-                for (int q = 0; q < NV; ++q) dst[q] += V[q];
-        } else {
-            // one ket can head several segments here: one after another
-            const unsigned m = __match_any_sync(0xffffffffu, head ? (key & 127u) : 128u + lane);
-            const int rank = __popc(m & ((1u << lane) - 1u));
-#pragma unroll 1
-            for (int rr = 0; __any_sync(0xffffffffu, head && rank >= rr); ++rr) {
-                if (head && rank == rr)
-#pragma unroll
-                    for (int q = 0; q < NV; ++q) dst[q] += V[q];
-                __syncwarp();
-            }
-        }
         qd += count;
-        __syncwarp();
     };
     // screen, evaluate and digest the next count queued kets
     auto process = [&](int count) {
@@ -987,105 +1196,130 @@ __global__ void __launch_bounds__(kRealThreads) k_real_q(PlanDev pl, int b0, int
     }
 }
 
-// FP64 pass over the listed large quartets: one warp per list entry.  The
-// entry's npp_bra x npp_ket primitive quartets are screened 32 at a time in
-// single precision, the ones that pass go into a per-warp queue (shared
-// memory) and are evaluated in FP64 one per lane, 32 at a time, into the
-// lane's block; the block is summed over the warp and digested by lane 0.
+// FP64 pass over the listed large quartets.  A warp takes up to SL entries at
+// a time (fewer when the list is too short for eight such turns per warp: with
+// one turn, its heaviest entries side by side in one warp, a short list took
+// twice as long): their
+// primitive quartets are laid out one per lane and screened, the ones that pass
+// go into the ring of k_real_w and are evaluated 32 at a time into the entries'
+// blocks, which are digested one entry per lane.  With one entry per warp the
+// last batch of an entry was half empty (33 primitive quartets on average for
+// (ss|pp) of the 64-water box: two batches) and one lane digested alone.
 // Counters as k_real_w (cnt points at the FP64 slots).
 template <int LA, int LB, int LC, int LD>
-__global__ void __launch_bounds__(32 * kWarpsPerBlock) k_real_list_w(PlanDev pl, const int2 *__restrict__ big, const unsigned *__restrict__ nbig,
-                                                                     unsigned cap, int same, const double *__restrict__ Dp,
-                                                                     double *__restrict__ X, double *__restrict__ Y,
-                                                                     unsigned long long *__restrict__ cnt)
+__global__ void __launch_bounds__(32 * kWarpsPerBlock, 3) k_real_list_w(PlanDev pl, const int2 *__restrict__ big,
+                                                                        const unsigned *__restrict__ nbig, unsigned cap, int same,
+                                                                        const double *__restrict__ Dp, double *__restrict__ X,
+                                                                        double *__restrict__ Y, unsigned long long *__restrict__ cnt)
 {
     constexpr int NA = ncart(LA), NB = ncart(LB), NC = ncart(LC), ND = ncart(LD), NV = NA * NB * NC * ND;
     constexpr int L = LA + LB + LC + LD;
-    __shared__ int qall[kWarpsPerBlock][64];
-    const int lane = threadIdx.x & 31;
-    int *qbuf = qall[threadIdx.x >> 5];
-    const unsigned total = min(*nbig, cap);
+    constexpr int SL = NV * 8 <= 144 ? 32 : 16;
+    __shared__ unsigned ring_s[kWarpsPerBlock][kListRing];
+    __shared__ int bpp0_s[kWarpsPerBlock][SL], kpp0_s[kWarpsPerBlock][SL];
+    __shared__ double V_s[kWarpsPerBlock][SL * NV];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    unsigned *ring = ring_s[wid];
+    int *bpp0 = bpp0_s[wid], *kpp0 = kpp0_s[wid];
+    double *Vs = V_s[wid];
+    const unsigned total = min(*nbig, cap), nwarps = gridDim.x * kWarpsPerBlock, warp = blockIdx.x * kWarpsPerBlock + wid;
+    const unsigned per = min((unsigned)SL, max(1u, total / (8 * nwarps)));
     const int n = pl.nbf;
+    const float lbc = 3.2094f - pl.log_ewald_R;  // ln(2 pi^{5/2} / sqrt 2) + 1e-3
+    const float r1min = pl.nr1 > 1 ? pl.r1f[7] : 1e30f;
+    const float Lc = radius_correction<L>(pl, 2.0f * pl.lb_max + lbc);
     Tally tl;
-    unsigned used = 0, slots = 0;
-    unsigned done = 0;
-    const unsigned nwarps = gridDim.x * kWarpsPerBlock;
-    for (unsigned q = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5); q < total; q += nwarps) {
-        const int2 pr = big[q];
-        const SpiRec sb = pl.spi[pr.x], sk = pl.spi[pr.y];
-        const int nterm = sb.npp * sk.npp;
-        double V[NV];
+    unsigned used = 0, slots = 0, done = 0;
+#pragma unroll 1
+    for (unsigned base = warp * per; base < total; base += nwarps * per) {
+        const int cnt_e = (int)min(per, total - base);
+        int nk = 1, nterm = 0;
+        if (lane < cnt_e) {
+            const int2 pr = big[base + lane];
+            const int b0 = __float_as_int(__ldg(&pl.spr[pr.x].w)), k0 = __float_as_int(__ldg(&pl.spr[pr.y].w));
+            nk = __float_as_int(__ldg(&pl.spr[pr.y + 1].w)) - k0;
+            nterm = (__float_as_int(__ldg(&pl.spr[pr.x + 1].w)) - b0) * nk;
+            bpp0[lane] = b0;
+            kpp0[lane] = k0;
+        }
+        for (int q = lane; q < cnt_e * NV; q += 32) Vs[q] = 0.0;
+        int incl = nterm;
 #pragma unroll
-        for (int k = 0; k < NV; ++k) V[k] = 0.0;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        const int all = __shfl_sync(0xffffffffu, incl, 31), excl = incl - nterm;
+        __syncwarp();
         unsigned qn = 0, qd = 0;
-        auto drain = [&](unsigned count) {
-            if (lane < count) {
-                const int t = qbuf[(qd + lane) & 63];
-                const int i = t / sk.npp, j = t - i * sk.npp;
-                PrimE<LA, LB, double> bp;
-                PrimE<LC, LD, double> kp;
-                PpiF bf, kf;
-                load_prim<LA, LB, double>(pl, sb.pp0 + i, bp, bf);
-                load_prim<LC, LD, double>(pl, sk.pp0 + j, kp, kf);
-                ++tl.brap;
-                ++tl.ketp;
-                prim_term<LA, LB, LC, LD, double>(pl, bp, bf, kp, kf, V, tl);
-                ++used;
+#pragma unroll 1
+        for (int e0 = 0; e0 < all; e0 += 32) {
+            const int e = e0 + lane;
+            // owner: the first lane whose inclusive prefix exceeds e
+            int own = 0;
+#pragma unroll
+            for (int step = 16; step > 0; step >>= 1) {
+                const int v = __shfl_sync(0xffffffffu, incl, own + step - 1);
+                if (v <= e) own += step;
             }
-            if (lane == 0) slots += 32;
-            qd += count;
-            __syncwarp();
-        };
-        for (int t0 = 0; t0 < nterm; t0 += 32) {
-            const int t = t0 + lane;
+            const int t = e - __shfl_sync(0xffffffffu, excl, own), k = __shfl_sync(0xffffffffu, nk, own);
+            const int i = t / k, j = t - i * k;
             bool pass = false;
-            if (t < nterm) {
-                const int i = t / sk.npp, j = t - i * sk.npp;
-                pass = __ldg(pl.ppB + sb.pp0 + i) * __ldg(pl.ppB + sk.pp0 + j) >= pl.mag_thr &&
-                       prim_reaches<L>(pl, pl.ppf[sb.pp0 + i], pl.ppf[sk.pp0 + j]);
+            if (e < all) {
+                const int ib = bpp0[own] + i, ik = kpp0[own] + j;
+                const float s = __ldg(pl.pplb + ib) + __ldg(pl.pplb + ik) + lbc;
                 ++tl.screen;
+                pass = s > 0.0f && prim_maybe<L>(pl, __ldg(pl.pps + ib), __ldg(pl.pps + ik), s, Lc, r1min);
             }
             const unsigned m = __ballot_sync(0xffffffffu, pass);
-            if (pass) qbuf[(qn + __popc(m & ((1u << lane) - 1u))) & 63] = t;
+            if (pass)
+                ring[(qn + __popc(m & ((1u << lane) - 1u))) & (kListRing - 1)] = (unsigned)own | ((unsigned)i << 7) | ((unsigned)j << 15);
             qn += __popc(m);
             __syncwarp();
-            if (qn - qd >= 32) drain(32);
+            const unsigned lim = e0 + 32 < all ? 32u : 1u;
+#pragma unroll 1
+            while (qn - qd >= lim) {
+                const unsigned count = min(32u, qn - qd);
+                eval_terms<LA, LB, LC, LD, double, kListRing, false>(
+                    pl, ring, qd, count, [&](unsigned s) { return bpp0[s]; }, [&](unsigned s) { return kpp0[s]; }, false, Vs, tl, used);
+                qd += count;
+                slots += lane == 0 ? 32u : 0u;
+            }
         }
-        while (qn > qd) drain(min(32u, qn - qd));
-#pragma unroll
-        for (int k = 0; k < NV; ++k) V[k] = warp_sum(V[k]);
-        if (lane == 0) {
-            ++done;
+        __syncwarp();
+        if (lane < cnt_e) {
+            const int2 pr = big[base + lane];
+            const int4 b4 = __ldg(pl.spd + pr.x), k4 = __ldg(pl.spd + pr.y);
+            double V[NV], Dij[NA * NB];
             Acc<double> jb[NA * NB];
-            double Dij[NA * NB];
-            const int aoI = pl.shells[sb.I].ao, aoJ = pl.shells[sb.J].ao;
+#pragma unroll
+            for (int q = 0; q < NV; ++q) V[q] = Vs[lane * NV + q];
 #pragma unroll
             for (int a = 0; a < NA; ++a)
 #pragma unroll
-                for (int b = 0; b < NB; ++b) Dij[a * NB + b] = __ldg(Dp + (size_t)(aoI + a) * n + aoJ + b);
-            const double w = double(sb.w) * double(sk.w) * ((same && pr.x == pr.y) ? 0.5 : 1.0);
-            digest<LA, LB, LC, LD, double>(n, aoI, aoJ, pl.shells[sk.I].ao, pl.shells[sk.J].ao, V, w, Dp, Dij, jb, X, Y);
+                for (int b = 0; b < NB; ++b) Dij[a * NB + b] = __ldg(Dp + (size_t)(b4.x + a) * n + b4.y + b);
+            const double w = (double)__int_as_float(b4.z) * (double)__int_as_float(k4.z) * ((same && pr.x == pr.y) ? 0.5 : 1.0);
+            digest<LA, LB, LC, LD, double>(n, b4.x, b4.y, k4.x, k4.y, V, w, Dp, Dij, jb, X, Y);
+#pragma unroll
+            for (int a = 0; a < NA; ++a)
+#pragma unroll
+                for (int b = 0; b < NB; ++b) atomicAdd(X + (size_t)(b4.x + a) * n + b4.y + b, jb[a * NB + b].value());
             ++tl.quart;
-#pragma unroll
-            for (int a = 0; a < NA; ++a)
-#pragma unroll
-                for (int b = 0; b < NB; ++b) {
-                    const double v = jb[a * NB + b].value();
-                    if (v != 0.0) atomicAdd(X + (size_t)(aoI + a) * n + aoJ + b, v);
-                }
+            ++done;
         }
         __syncwarp();
     }
-    unsigned long long fl = tally_alg<LA, LB, LC, LD>(tl), fs = tally_screen<LA, LB, LC, LD>(tl), u64 = used, s64 = slots;
+    unsigned long long fl = tally_alg<LA, LB, LC, LD>(tl), fs = tally_screen<LA, LB, LC, LD>(tl), u64 = used, s64 = slots, d64 = done;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         fl += __shfl_xor_sync(0xffffffffu, fl, o);
         fs += __shfl_xor_sync(0xffffffffu, fs, o);
         u64 += __shfl_xor_sync(0xffffffffu, u64, o);
         s64 += __shfl_xor_sync(0xffffffffu, s64, o);
+        d64 += __shfl_xor_sync(0xffffffffu, d64, o);
     }
     if (lane == 0) {
-        if (done) atomicAdd(cnt, (unsigned long long)done);
+        if (d64) atomicAdd(cnt, d64);
         if (fl) atomicAdd(cnt + 4, fl);
         if (fs) atomicAdd(cnt + 8, fs);
         if (u64) atomicAdd(cnt + 12, u64);

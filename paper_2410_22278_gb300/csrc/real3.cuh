@@ -219,7 +219,7 @@ __device__ __forceinline__ bool coop_quartet(const PlanDev &pl, const SpiRec &sb
                             PairT<T> b;
                             const PpiF bf = pl.ppf[sb.pp0 + i];
                             load_pair(pl, sb.pp0 + i, bf, b);
-                            sc = T(kTwoPi52) * b.K * p.K * b.ip * p.ip / sqrt(b.p + p.p);
+                            sc = T(kTwoPi52) * b.K * p.K * b.ip * p.ip * inv_sqrt(b.p + p.p);
                         }
 #pragma unroll
                         for (int q = 0; q < S::EC; ++q) s.Ec[ax * S::EC + q] = ((q % NTC) & 1) ? -sc * E[q] : sc * E[q];
