@@ -459,7 +459,7 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
     cudaMemsetAsync(w.KLR, 0, n2 * sizeof(double), st);
     cudaMemsetAsync(w.scal, 0, 16 * sizeof(double), st);
     cudaMemsetAsync(w.cnt, 0, kCounters * sizeof(unsigned long long), st);
-    if (w.nbig) cudaMemsetAsync(w.nbig, 0, 2 * sizeof(unsigned), st);
+    if (w.nbig) cudaMemsetAsync(w.nbig, 0, 2 * sizeof(unsigned) * w.nlist, st);
     int rc;
     if ((rc = cuda_check("prologue"))) return rc;
     // mixed precision: slices of D' and its low-rank factorisation for the
@@ -481,12 +481,25 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
         tm.stop(0, eh, JK_NCLASS_MAX - kJengClass + 1);
     }
 
-    // ---- real space (the phases run one after another on the caller's
-    // stream: run on streams of their own they gained nothing on the water
-    // box -- the tile kernels fill every SM, and the tensor-core GEMMs, which
-    // need a whole SM each, only start as the tile grids drain)
+    // ---- real space.  Large cells: one class pair after another on the
+    // caller's stream (the tile kernels fill every SM; on streams of their own
+    // they gained nothing on the water box).  Small plans deal the class pairs
+    // out over the caller's stream and Plan::kSide more, forked and joined by
+    // events; they only meet in the atomics on X, Y and the counters.
     ev = tm.start(1);
     int nreal = 0;
+    if (P->nside > 0) {
+        cudaEventRecord(P->side_fork, st);
+        for (int i = 0; i < P->nside; ++i) cudaStreamWaitEvent(P->side[i], P->side_fork, 0);
+    }
+    const auto join = [&] {
+        tm.use(st);
+        for (int i = 0; i < P->nside; ++i) {
+            cudaEventRecord(P->side_join[i], P->side[i]);
+            cudaStreamWaitEvent(st, P->side_join[i], 0);
+        }
+    };
+    int turn = 0;
     for (int cb = 0; cb < JK_NCLASS_MAX; ++cb)
         for (int ck = cb; ck < JK_NCLASS_MAX; ++ck) {
             const ClassRange &B = P->classes[cb], &Kc = P->classes[ck];
@@ -508,7 +521,12 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
             a.dmaxf = w.dmaxf;
             a.X = w.X;
             a.Y = K ? w.Y : nullptr;
-            a.st = st;
+            const int lane = P->nside > 0 ? turn++ % (P->nside + 1) : 0;
+            cudaStream_t ls = lane ? P->side[lane - 1] : st;
+            tm.use(ls);
+            int2 *big = w.big ? w.big + (size_t)lane * w.cap : nullptr;
+            unsigned *nbig = w.nbig ? w.nbig + 2 * lane : nullptr;
+            a.st = ls;
             a.DhD = w.DhD;
             a.DhF = w.DhF;
             a.JH = w.JH;
@@ -529,13 +547,13 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
                 tm.stop(10, et, 1);
                 nreal += 1;
             } else if (use_jeng) {
-                cudaMemsetAsync(w.nbig, 0, sizeof(unsigned), st);
+                cudaMemsetAsync(nbig, 0, sizeof(unsigned), ls);
                 a.mode = 2;
                 a.fp32 = true;
                 a.cnt = w.cnt + 1;
-                a.big = w.big;
-                a.nbig = w.nbig;
-                a.ovf = w.nbig + 1;
+                a.big = big;
+                a.nbig = nbig;
+                a.ovf = nbig + 1;
                 a.cap = w.cap;
                 const int et = tm.start(10);
                 launch_jeng(cb, ck, a);
@@ -557,13 +575,13 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
                 nreal += 1;
             } else {
                 // FP32 pass over every quartet, collecting the large ones ...
-                cudaMemsetAsync(w.nbig, 0, sizeof(unsigned), st);
+                cudaMemsetAsync(nbig, 0, sizeof(unsigned), ls);
                 a.mode = 2;
                 a.fp32 = true;
                 a.cnt = w.cnt + 1;
-                a.big = w.big;
-                a.nbig = w.nbig;
-                a.ovf = w.nbig + 1;
+                a.big = big;
+                a.nbig = nbig;
+                a.ovf = nbig + 1;
                 a.cap = w.cap;
                 const int et = tm.start(10);
                 launch_real(cb, ck, a);
@@ -576,8 +594,12 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
                 tm.stop(9, el, 1);
                 nreal += 2;
             }
-            if ((rc = cuda_check("real-space kernel"))) return rc;
+            if ((rc = cuda_check("real-space kernel"))) {
+                join();
+                return rc;
+            }
         }
+    join();
     if (jeng) {
         // Hermite J of every primitive pair back to Cartesian, into X
         for (int c = kJengClass; c < JK_NCLASS_MAX; ++c)
@@ -761,12 +783,13 @@ int set_schedule(Plan *P, const int *sched, int n)
 int build_counts(Plan *P, long long *counts, int n)
 {
     unsigned long long h[kCounters] = {};
-    unsigned hb[2] = {0, 0};
+    unsigned hb[2 * (1 + Plan::kSide)] = {};
     if (P->timer.next > 0 && cudaEventSynchronize(P->timer.pool[P->timer.next - 1]) != cudaSuccess)
         return fail(JK_ERR_CUDA, "build did not finish");
     if (cudaMemcpy(h, P->ws.cnt, sizeof h, cudaMemcpyDeviceToHost) != cudaSuccess) return fail(JK_ERR_CUDA, "count copy failed");
-    if (P->ws.nbig && cudaMemcpy(hb, P->ws.nbig, sizeof hb, cudaMemcpyDeviceToHost) != cudaSuccess)
+    if (P->ws.nbig && cudaMemcpy(hb, P->ws.nbig, 2 * sizeof(unsigned) * P->ws.nlist, cudaMemcpyDeviceToHost) != cudaSuccess)
         return fail(JK_ERR_CUDA, "count copy failed");
+    for (int i = 1; i < P->ws.nlist; ++i) hb[1] += hb[2 * i + 1];
     // rank and form of the density factorisation (mixed builds with K)
     int dyn[4] = {0, 0, 0, 0};
     if (P->precision == JK_MIXED && P->ws.lr.dyn && cudaMemcpy(dyn, P->ws.lr.dyn, sizeof dyn, cudaMemcpyDeviceToHost) != cudaSuccess)

@@ -507,9 +507,10 @@ static int alloc_ws(Plan *P)
         // the FP64 share is a small fraction; the list holds up to 2% of all image quartets (at most 64 Mi entries)
         const long long want = std::min<long long>(std::max<long long>(P->n_quartets / 50, 1 << 20), 64ll << 20);
         w.cap = (unsigned)want;
-        if (cudaMalloc((void **)&w.big, sizeof(int2) * w.cap) != cudaSuccess) return fail(JK_ERR_OOM, "cudaMalloc failed for quartet list");
-        if (cudaMalloc((void **)&w.nbig, 2 * sizeof(unsigned)) != cudaSuccess) return fail(JK_ERR_OOM, "cudaMalloc failed");
-        bytes += sizeof(int2) * w.cap + 2 * sizeof(unsigned);
+        w.nlist = 1 + P->nside;
+        if (cudaMalloc((void **)&w.big, sizeof(int2) * w.cap * w.nlist) != cudaSuccess) return fail(JK_ERR_OOM, "cudaMalloc failed for quartet list");
+        if (cudaMalloc((void **)&w.nbig, 2 * sizeof(unsigned) * w.nlist) != cudaSuccess) return fail(JK_ERR_OOM, "cudaMalloc failed");
+        bytes += (sizeof(int2) * w.cap + 2 * sizeof(unsigned)) * w.nlist;
     }
     cudaMemset(w.err, 0, sizeof(unsigned));
     w.bytes = bytes + sizeof(unsigned) + kCounters * sizeof(unsigned long long);
@@ -1160,6 +1161,18 @@ int finish_plan_device(Plan *P)
     }
     std::vector<double> zeros((size_t)P->nbf * P->nbf, 0.0);
     if ((rc = upload(zeros, &P->d_S, b))) return rc;
+    // side streams for plans of at most 2e8 image quartets: above that the
+    // (ss|ss) launch alone keeps the chip busy, and each lane needs a list of
+    // large quartets of its own
+    if (P->n_quartets <= 200000000LL) {
+        if (cudaEventCreateWithFlags(&P->side_fork, cudaEventDisableTiming) != cudaSuccess) return fail(JK_ERR_CUDA, "cudaEventCreate failed");
+        for (int i = 0; i < Plan::kSide; ++i) {
+            if (cudaStreamCreateWithFlags(&P->side[i], cudaStreamNonBlocking) != cudaSuccess) return fail(JK_ERR_CUDA, "cudaStreamCreate failed");
+            P->nside = i + 1;
+            if (cudaEventCreateWithFlags(&P->side_join[i], cudaEventDisableTiming) != cudaSuccess)
+                return fail(JK_ERR_CUDA, "cudaEventCreate failed");
+        }
+    }
     if ((rc = alloc_ws(P))) return rc;
     if ((rc = energy_reserve(P))) return rc;
     if ((rc = compute_overlap_raw(P, 0))) return rc;
@@ -1173,6 +1186,11 @@ void destroy_plan(Plan *P)
     cudaSetDevice(P->device);
     release_cache(P);
     energy_release(P);
+    for (int i = 0; i < P->nside; ++i) {
+        cudaStreamDestroy(P->side[i]);
+        if (P->side_join[i]) cudaEventDestroy(P->side_join[i]);
+    }
+    if (P->side_fork) cudaEventDestroy(P->side_fork);
     void *ptrs[] = {P->d_shells, P->d_spi, P->d_ppi, P->d_ppf, P->d_ppB, P->d_pps, P->d_pplb, P->d_r1f, P->d_spair, P->d_spi_order, P->d_boys, P->d_boys_f, P->d_boys_t, P->d_r1, P->d_gvec,
                     P->d_g0, P->d_compf, P->d_ppi_ab, P->d_kblk, P->d_kblk2, P->d_spq, P->d_spr, P->d_spd, P->d_pvals, P->d_gtab0, P->d_ppi_pidx, P->d_phase, P->d_ppdf, P->d_gdf, P->d_phasef, P->ws.gtab, P->ws.gtab2, P->d_S, P->ws.Dp, P->ws.X, P->ws.Y, P->ws.JLR, P->ws.KLR, P->ws.T1, P->ws.T2,
                     P->ws.M, P->ws.Z, P->ws.rho, P->ws.rho_part, P->ws.DhD, P->ws.JH, P->ws.DhF, P->ws.dmax, P->ws.scal, P->ws.err, P->ws.cnt, P->ws.big, P->ws.nbig,

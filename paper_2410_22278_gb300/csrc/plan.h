@@ -55,6 +55,7 @@ struct Workspace {
     int2 *big = nullptr;                // compact list of quartets sent to FP64 (mixed precision)
     unsigned *nbig = nullptr;           // [0] list length, [1] overflow count (accumulated over a build)
     unsigned cap = 0;
+    int nlist = 1;                      // lists (big: nlist * cap entries, nbig: nlist pairs), one per lane of the real-space phase
     int gc = 0;               // G vectors per chunk
     double *gtab = nullptr;   // [distinct p][gc]: (pi/p)^{3/2} e^{-G^2/4p} of the current G chunk
     float2 *gtab2 = nullptr;  // the same as double-floats (mixed-precision structure factors)
@@ -189,6 +190,12 @@ struct Plan {
     Workspace ws;
     RecipCache cache;
     PhaseTimer timer;
+    // lanes of the real-space phase beside the caller's stream (small plans; the
+    // class pairs of a small cell do not fill the chip one at a time)
+    static constexpr int kSide = 3;
+    int nside = 0;
+    cudaStream_t side[kSide] = {};
+    cudaEvent_t side_fork = nullptr, side_join[kSide] = {};
     std::mutex build_mu;
     std::mutex energy_mu;
     std::vector<EnergySlot> energy_free;  // not in use by a call
