@@ -8,7 +8,7 @@ CLASSES = [(0, 0), (1, 0), (1, 1), (2, 0), (2, 1), (2, 2)]
 #   * one warp per bra with its stages refilled (k_real_w, real2.cuh) while a
 #     lane can hold the block: NV <= 36 in FP32, NV <= 27 in FP64;
 #   * one warp per image quartet (k_real_c, real3.cuh) above that.
-# The FP64 list pass takes k_real_list_w up to NV = 27 and k_real_list_c above.
+# The FP64 list pass takes k_real_list_w up to NV = 36 and k_real_list_c above.
 # Class pairs of s and p shells have two more tile-kernel families, the
 # lane-per-bra kernels of kernels.cuh and the pair-queue kernels of real2.cuh,
 # and the autotuner picks one per class pair (RealLaunch::variant).
@@ -95,7 +95,7 @@ def unit(cb, ck):
         return "k_real_c<%s, %s><<<(unsigned)a.map.items, 32, 0, a.st>>>" % (q, t)
 
     lst = "(a.pl, a.big, a.nbig, a.cap, a.same, a.Dp, a.X, a.Y, a.cnt64)"
-    if nv <= 27:
+    if nv <= 36:
         lst = "k_real_list_w<%s><<<152 * 8, 32 * kWarpsPerBlock, 0, a.st>>>%s" % (q, lst)
     else:
         lst = "k_real_list_c<%s><<<152 * 16, 32, 0, a.st>>>%s" % (q, lst)

@@ -784,18 +784,21 @@ int build_plan(const jk_cell *cell, const jk_shell *shells, int nshell, double o
         if (cr.b1 <= cr.b0) cr.b0 = cr.b1 = 0;
         P->classes.push_back(cr);
     }
-    // untuned schedule: kets per warp for about a thousand warps per SM (half
-    // of them empty for a class with itself), at least 8 and at most 2048 --
-    // few enough that a small cell still fills the chip and the last warps do
-    // not hold up a launch, enough to fill the batches of a warp; the kernels that give an
-    // image quartet a whole warp (real3.cuh) have no batches and take 1 to 64
+    // untuned schedule: kets per warp for about 256 warps per SM (half of them
+    // empty for a class with itself) up to 512 kets, then for a thousand warps
+    // per SM up to 2048 -- few enough that a small cell still fills the chip
+    // and the last warps do not hold up a launch, enough to fill the batches of
+    // a warp; the kernels that give an image quartet a whole warp (real3.cuh)
+    // have no batches and take 1 to 64
     for (int i = 0; i < JK_NCLASS_MAX; ++i)
         for (int j = i; j < JK_NCLASS_MAX; ++j) {
             const ClassRange &B = P->classes[i], &K = P->classes[j];
             const long long nb = B.b1 - B.b0, nk = K.b1 - K.b0;
             const auto nc = [](int l) { return (l + 1) * (l + 2) / 2; };
             const bool coop = nc(B.la) * nc(B.lb) * nc(K.la) * nc(K.lb) > 36;
-            P->kchunk[i][j] = (int)std::min(coop ? 64LL : 2048LL, std::max(coop ? 1LL : 8LL, nb * nk / (152 * 1024)));
+            const long long few = nb * nk / (152 * 1024);
+            P->kchunk[i][j] = (int)(coop ? std::min(64LL, std::max(1LL, few))
+                                         : std::max(std::min(512LL, std::max(8LL, 4 * few)), std::min(2048LL, few)));
         }
     // ---- unique shell pairs with their images (reciprocal-space build), grouped by class
     {

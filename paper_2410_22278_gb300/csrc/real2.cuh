@@ -1207,14 +1207,14 @@ __global__ void __launch_bounds__(kRealThreads) k_real_q(PlanDev pl, int b0, int
 // (ss|pp) of the 64-water box: two batches) and one lane digested alone.
 // Counters as k_real_w (cnt points at the FP64 slots).
 template <int LA, int LB, int LC, int LD>
-__global__ void __launch_bounds__(32 * kWarpsPerBlock, 3) k_real_list_w(PlanDev pl, const int2 *__restrict__ big,
+__global__ void __launch_bounds__(32 * kWarpsPerBlock, LA + LB + LC + LD <= 3 ? 3 : 2) k_real_list_w(PlanDev pl, const int2 *__restrict__ big,
                                                                         const unsigned *__restrict__ nbig, unsigned cap, int same,
                                                                         const double *__restrict__ Dp, double *__restrict__ X,
                                                                         double *__restrict__ Y, unsigned long long *__restrict__ cnt)
 {
     constexpr int NA = ncart(LA), NB = ncart(LB), NC = ncart(LC), ND = ncart(LD), NV = NA * NB * NC * ND;
     constexpr int L = LA + LB + LC + LD;
-    constexpr int SL = NV * 8 <= 144 ? 32 : 16;
+    constexpr int SL = NV <= 18 ? 32 : 16;
     __shared__ unsigned ring_s[kWarpsPerBlock][kListRing];
     __shared__ int bpp0_s[kWarpsPerBlock][SL], kpp0_s[kWarpsPerBlock][SL];
     __shared__ double V_s[kWarpsPerBlock][SL * NV];
