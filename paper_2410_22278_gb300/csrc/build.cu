@@ -484,8 +484,9 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
     // ---- real space.  Large cells: one class pair after another on the
     // caller's stream (the tile kernels fill every SM; on streams of their own
     // they gained nothing on the water box).  Small plans deal the class pairs
-    // out over the caller's stream and Plan::kSide more, forked and joined by
-    // events; they only meet in the atomics on X, Y and the counters.
+    // out over the caller's stream and three more, forked and joined by events
+    // (they only meet in the atomics on X, Y and the counters), with the
+    // reciprocal phase, which shares nothing with them, on a fifth.
     ev = tm.start(1);
     int nreal = 0;
     if (P->nside > 0) {
@@ -499,6 +500,14 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
             cudaStreamWaitEvent(st, P->side_join[i], 0);
         }
     };
+    if (P->nside > 0) {
+        tm.use(P->side[P->nside - 1]);
+        if ((rc = reciprocal_phase(P, J, K, P->side[P->nside - 1]))) {
+            join();
+            return rc;
+        }
+        tm.use(st);
+    }
     int turn = 0;
     for (int cb = 0; cb < JK_NCLASS_MAX; ++cb)
         for (int ck = cb; ck < JK_NCLASS_MAX; ++ck) {
@@ -521,7 +530,7 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
             a.dmaxf = w.dmaxf;
             a.X = w.X;
             a.Y = K ? w.Y : nullptr;
-            const int lane = P->nside > 0 ? turn++ % (P->nside + 1) : 0;
+            const int lane = P->nside > 0 ? turn++ % P->nside : 0;
             cudaStream_t ls = lane ? P->side[lane - 1] : st;
             tm.use(ls);
             int2 *big = w.big ? w.big + (size_t)lane * w.cap : nullptr;
@@ -609,7 +618,7 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
     tm.stop(1, ev, nreal);
 
     // ---- reciprocal space
-    if ((rc = reciprocal_phase(P, J, K, st))) return rc;
+    if (P->nside == 0 && (rc = reciprocal_phase(P, J, K, st))) return rc;
 
     ev = tm.start(5);
 

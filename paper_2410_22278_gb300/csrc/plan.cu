@@ -507,7 +507,7 @@ static int alloc_ws(Plan *P)
         // the FP64 share is a small fraction; the list holds up to 2% of all image quartets (at most 64 Mi entries)
         const long long want = std::min<long long>(std::max<long long>(P->n_quartets / 50, 1 << 20), 64ll << 20);
         w.cap = (unsigned)want;
-        w.nlist = 1 + P->nside;
+        w.nlist = std::max(1, P->nside);  // the caller's stream and all but the last side stream
         if (cudaMalloc((void **)&w.big, sizeof(int2) * w.cap * w.nlist) != cudaSuccess) return fail(JK_ERR_OOM, "cudaMalloc failed for quartet list");
         if (cudaMalloc((void **)&w.nbig, 2 * sizeof(unsigned) * w.nlist) != cudaSuccess) return fail(JK_ERR_OOM, "cudaMalloc failed");
         bytes += (sizeof(int2) * w.cap + 2 * sizeof(unsigned)) * w.nlist;

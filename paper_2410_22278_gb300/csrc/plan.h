@@ -190,9 +190,10 @@ struct Plan {
     Workspace ws;
     RecipCache cache;
     PhaseTimer timer;
-    // lanes of the real-space phase beside the caller's stream (small plans; the
-    // class pairs of a small cell do not fill the chip one at a time)
-    static constexpr int kSide = 3;
+    // streams beside the caller's (small plans; the class pairs of a small cell
+    // do not fill the chip one at a time): all but the last are lanes of the
+    // real-space phase, the last takes the reciprocal phase
+    static constexpr int kSide = 4;
     int nside = 0;
     cudaStream_t side[kSide] = {};
     cudaEvent_t side_fork = nullptr, side_join[kSide] = {};
