@@ -536,7 +536,7 @@ def roofline(phases, real_flops, pk, pk_kind, fma):
     tile_ms = max(phases["real_tiles"][0], 1e-9)
     mk = "measured on this GPU (jk_microbench_fma: independent FMA chains, %d SMs, CUDA events)" % fma["sms"]
     out = [
-        {"bound": "alu", "kernel": "k_real<..., float> (FP32 real-space quartet tiles)", "achieved": fl32 / (tile_ms / 1e3) / 1e12,
+        {"bound": "alu", "kernel": "k_real*<..., float> (FP32 real-space quartet tiles)", "achieved": fl32 / (tile_ms / 1e3) / 1e12,
          "peak": fma["fp32_tflops"], "unit": "TFLOP/s", "frac": fl32 / (tile_ms / 1e3) / 1e12 / fma["fp32_tflops"],
          "traffic": REAL_TILE_TRAFFIC, "ms": tile_ms, "launches": phases["real_tiles"][1],
          "peak_kind": "FP32 FMA rate " + mk,
@@ -544,7 +544,7 @@ def roofline(phases, real_flops, pk, pk_kind, fma):
     ]
     if list_ms > 0:
         ach = fl64 / (list_ms / 1e3) / 1e12
-        out.append({"bound": "alu", "kernel": "k_real_list (FP64 large quartets)", "achieved": ach, "peak": fma["fp64_tflops"],
+        out.append({"bound": "alu", "kernel": "k_real_list_* (FP64 large quartets)", "achieved": ach, "peak": fma["fp64_tflops"],
                     "unit": "TFLOP/s", "frac": ach / fma["fp64_tflops"], "traffic": None, "ms": list_ms, "launches": list_n,
                     "peak_kind": "FP64 FMA rate " + mk, "work": "algorithmic flops of the MD steps (csrc/flops.h)"})
     gemm_ms, gemm_n = phases.get("tensor_gemm", (0.0, 0))

@@ -222,17 +222,18 @@ int jk_energy_noalloc(const jk_plan *plan, const double *D, const double *J, con
 int jk_build_times(jk_plan *plan, double *ms, int *launches, int n);
 
 /* Autotuner (no counterpart in the paper): choose the tile shape of every
- * real-space class-pair kernel -- the family (0 lane-per-bra, 8 .. 128 kets
- * per tile; for class pairs of s and p shells also 1 warp-per-bra, 128 ..
- * 2048 kets per warp, and 2 pair queue, 32 .. 512 kets per tile) and its
- * tile -- by timing the candidates on two sub-ranges of bras with CUDA
+ * real-space class-pair kernel -- for class pairs of s and p shells the
+ * family (0 lane-per-bra, 8 .. 128 kets per tile; 1 warp-per-bra, 128 ..
+ * 2048 kets per warp on average; 2 pair queue, 32 .. 512 kets per tile),
+ * for class pairs with a d shell, which have one kernel (family 0, a bra or
+ * a quartet per warp), 1 .. 2048 kets per warp -- by timing the candidates on two sub-ranges of bras with CUDA
  * events, on
  * `cuda_stream`, using density D (device, as in jk_build) for realistic
  * work.  If cache_path is not NULL, choices are read from and written to
  * that text file, keyed by GPU name, precision, class pair and size
  * bucket.  chosen (may be NULL) receives 42 ints: (family, kets) for each
  * of the 21 class pairs (bra class <= ket class, classes ss, ps, pp, ds,
- * dp, dd), family 0 lane-per-bra, 1 warp, 2 pair queue.  Overwrites the
+ * dp, dd).  Overwrites the
  * plan's build workspace; synchronises the stream. */
 int jk_autotune(jk_plan *plan, const double *D, void *cuda_stream, const char *cache_path, int *chosen);
 

@@ -236,7 +236,8 @@ class Plan:
 
     def autotune(self, D_ptr: int, stream: int = 0, cache_path: str = None):
         """Real-space schedule chosen by timing (jk_autotune): a list of 21
-        (family, kets) pairs, family 0 lane-per-bra, 1 warp."""
+        (family, kets) pairs; families 0 lane-per-bra, 1 warp and 2 pair
+        queue for s and p class pairs, 0 for the others."""
         chosen = (ctypes.c_int * 42)()
         _check(lib().jk_autotune(self._h, D_ptr, stream or None, cache_path.encode() if cache_path else None, chosen),
                "jk_autotune")
