@@ -20,6 +20,7 @@ struct jk_plan {
 };
 
 using jk::fail;
+using jk::fail_cuda;
 
 extern "C" {
 
@@ -48,7 +49,7 @@ int jk_plan_create(const jk_cell *cell, const jk_shell *shells, int nshell, doub
         if (!out) return fail(JK_ERR_INVALID, "out is NULL");
         *out = nullptr;
         int ndev = 0;
-        if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev == 0) return fail(JK_ERR_CUDA, "no CUDA device");
+        if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev == 0) return fail_cuda(JK_ERR_CUDA, "no CUDA device");
         if (device < 0 || device >= ndev) return fail(JK_ERR_INVALID, "device index out of range");
         jk::Plan *P = nullptr;
         int rc = jk::build_plan(cell, shells, nshell, omega, cut, precision, device, &P);
@@ -62,7 +63,7 @@ int jk_plan_create(const jk_cell *cell, const jk_shell *shells, int nshell, doub
         if (cudaEventCreateWithFlags(&h->done, cudaEventDisableTiming) != cudaSuccess) {
             jk::destroy_plan(P);
             delete h;
-            return fail(JK_ERR_CUDA, "cudaEventCreate failed");
+            return fail_cuda(JK_ERR_CUDA, "cudaEventCreate failed");
         }
         cudaEventRecord(h->done, 0);
         *out = h;
@@ -142,7 +143,7 @@ int jk_build(jk_plan *plan, const double *D, double *J, double *K, void *cuda_st
     if (!J && !K) return JK_OK;
     try {
         cudaStream_t st = (cudaStream_t)cuda_stream;
-        if (cudaSetDevice(plan->p->device) != cudaSuccess) return fail(JK_ERR_CUDA, "cudaSetDevice failed");
+        if (cudaSetDevice(plan->p->device) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "cudaSetDevice failed");
         // one critical section: order after the previous build on this plan,
         // enqueue, and publish this build's completion event, so builds from
         // several host threads on several streams run one after another on
@@ -161,10 +162,10 @@ int jk_plan_cache(jk_plan *plan, size_t max_bytes, size_t *bytes)
 {
     if (!plan) return fail(JK_ERR_INVALID, "plan is NULL");
     try {
-        if (cudaSetDevice(plan->p->device) != cudaSuccess) return fail(JK_ERR_CUDA, "cudaSetDevice failed");
+        if (cudaSetDevice(plan->p->device) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "cudaSetDevice failed");
         std::lock_guard<std::mutex> g(plan->p->build_mu);
         // the cache may be in use by the plan's last build
-        if (cudaEventSynchronize(plan->done) != cudaSuccess) return fail(JK_ERR_CUDA, "previous build failed");
+        if (cudaEventSynchronize(plan->done) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "previous build failed");
         int rc = jk::cache_reciprocal(plan->p, max_bytes);
         if (bytes) *bytes = plan->p->cache.bytes;
         return rc;
@@ -185,7 +186,7 @@ int jk_autotune(jk_plan *plan, const double *D, void *cuda_stream, const char *c
     if (!plan || !D) return fail(JK_ERR_INVALID, "plan or D is NULL");
     try {
         cudaStream_t st = (cudaStream_t)cuda_stream;
-        if (cudaSetDevice(plan->p->device) != cudaSuccess) return fail(JK_ERR_CUDA, "cudaSetDevice failed");
+        if (cudaSetDevice(plan->p->device) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "cudaSetDevice failed");
         std::lock_guard<std::mutex> g(plan->p->build_mu);
         cudaStreamWaitEvent(st, plan->done, 0);
         int rc = jk::autotune(plan->p, D, st, cache_path, chosen);
@@ -215,23 +216,23 @@ int jk_build_host(jk_plan *plan, const double *Dh, double *Jh, double *Kh, void 
     if (!plan || !Dh) return fail(JK_ERR_INVALID, "plan or D is NULL");
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const size_t bytes = sizeof(double) * plan->p->nbf * plan->p->nbf;
-    if (cudaSetDevice(plan->p->device) != cudaSuccess) return fail(JK_ERR_CUDA, "cudaSetDevice failed");
+    if (cudaSetDevice(plan->p->device) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "cudaSetDevice failed");
     double *d = nullptr, *j = nullptr, *k = nullptr;
     if (cudaMallocAsync((void **)&d, bytes, st) != cudaSuccess || (Jh && cudaMallocAsync((void **)&j, bytes, st) != cudaSuccess) ||
         (Kh && cudaMallocAsync((void **)&k, bytes, st) != cudaSuccess)) {
         if (d) cudaFreeAsync(d, st);
         if (j) cudaFreeAsync(j, st);
-        return fail(JK_ERR_OOM, "device buffers for host build");
+        return fail_cuda(JK_ERR_OOM, "device buffers for host build");
     }
     int rc = JK_OK;
-    if (cudaMemcpyAsync(d, Dh, bytes, cudaMemcpyHostToDevice, st) != cudaSuccess) rc = fail(JK_ERR_CUDA, "copy of D failed");
+    if (cudaMemcpyAsync(d, Dh, bytes, cudaMemcpyHostToDevice, st) != cudaSuccess) rc = fail_cuda(JK_ERR_CUDA, "copy of D failed");
     if (!rc) rc = jk_build(plan, d, j, k, cuda_stream);
-    if (!rc && Jh && cudaMemcpyAsync(Jh, j, bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess) rc = fail(JK_ERR_CUDA, "copy of J failed");
-    if (!rc && Kh && cudaMemcpyAsync(Kh, k, bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess) rc = fail(JK_ERR_CUDA, "copy of K failed");
+    if (!rc && Jh && cudaMemcpyAsync(Jh, j, bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess) rc = fail_cuda(JK_ERR_CUDA, "copy of J failed");
+    if (!rc && Kh && cudaMemcpyAsync(Kh, k, bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess) rc = fail_cuda(JK_ERR_CUDA, "copy of K failed");
     cudaFreeAsync(d, st);
     if (j) cudaFreeAsync(j, st);
     if (k) cudaFreeAsync(k, st);
-    if (cudaStreamSynchronize(st) != cudaSuccess && !rc) rc = fail(JK_ERR_CUDA, "host build failed");
+    if (cudaStreamSynchronize(st) != cudaSuccess && !rc) rc = fail_cuda(JK_ERR_CUDA, "host build failed");
     return rc;
 }
 
@@ -239,7 +240,7 @@ int jk_energy(const jk_plan *plan, const double *D, const double *J, const doubl
 {
     if (!plan || !D || !e_coul || !e_exch) return fail(JK_ERR_INVALID, "NULL argument");
     try {
-        if (cudaSetDevice(plan->p->device) != cudaSuccess) return fail(JK_ERR_CUDA, "cudaSetDevice failed");
+        if (cudaSetDevice(plan->p->device) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "cudaSetDevice failed");
         return jk::energy(plan->p, D, J, K, e_coul, e_exch, (cudaStream_t)cuda_stream);
     } catch (...) {
         return fail(JK_ERR_INVALID, "unexpected host exception");
@@ -259,7 +260,7 @@ int jk_overlap(const jk_plan *plan, double *S, void *cuda_stream)
 {
     if (!plan || !S) return fail(JK_ERR_INVALID, "NULL argument");
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    if (cudaSetDevice(plan->p->device) != cudaSuccess) return fail(JK_ERR_CUDA, "cudaSetDevice failed");
+    if (cudaSetDevice(plan->p->device) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "cudaSetDevice failed");
     const size_t n2 = (size_t)plan->p->nbf * plan->p->nbf;
     jk_scale_kernel<<<(unsigned)std::min<size_t>((n2 + 255) / 256, 2432), 256, 0, st>>>(plan->p->nbf, plan->p->d_compf, plan->p->d_S, S);
     if (cudaGetLastError() != cudaSuccess) return fail(JK_ERR_CUDA, "overlap kernel failed");
@@ -271,7 +272,7 @@ int jk_one_electron(jk_plan *plan, int natom, const double *Z, const double *xyz
     if (!plan || natom < 0 || (V && natom > 0 && (!Z || !xyz))) return fail(JK_ERR_INVALID, "bad one-electron arguments");
     try {
         cudaStream_t st = (cudaStream_t)cuda_stream;
-        if (cudaSetDevice(plan->p->device) != cudaSuccess) return fail(JK_ERR_CUDA, "cudaSetDevice failed");
+        if (cudaSetDevice(plan->p->device) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "cudaSetDevice failed");
         std::lock_guard<std::mutex> g(plan->p->build_mu);
         cudaStreamWaitEvent(st, plan->done, 0);
         int rc = jk::one_electron(plan->p, natom, Z, xyz, T, V, st);
@@ -401,7 +402,7 @@ int jk_server_create(int device, size_t hbm_budget_bytes, int max_slots, jk_serv
         s->budget = hbm_budget_bytes;
         if (cudaSetDevice(device) != cudaSuccess) {
             delete s;
-            return fail(JK_ERR_CUDA, "cudaSetDevice failed");
+            return fail_cuda(JK_ERR_CUDA, "cudaSetDevice failed");
         }
         s->slots.resize(max_slots);
         for (auto &sl : s->slots) {
@@ -412,7 +413,7 @@ int jk_server_create(int device, size_t hbm_budget_bytes, int max_slots, jk_serv
                     if (x.ev) cudaEventDestroy(x.ev);
                 }
                 delete s;
-                return fail(JK_ERR_CUDA, "stream creation failed");
+                return fail_cuda(JK_ERR_CUDA, "stream creation failed");
             }
         }
         s->worker = std::thread([s] { s->loop(); });

@@ -435,7 +435,7 @@ static int reciprocal_phase(Plan *P, double *J, double *K, cudaStream_t st)
 // critical section.
 int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
 {
-    if (cudaSetDevice(P->device) != cudaSuccess) return fail(JK_ERR_CUDA, "cudaSetDevice failed");
+    if (cudaSetDevice(P->device) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "cudaSetDevice failed");
     const int n = P->nbf;
     const size_t n2 = (size_t)n * n;
     PlanDev pl = P->dev();
@@ -643,7 +643,7 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
 // precision, class pair and size bucket) when cache_path is given.
 int autotune(Plan *P, const double *D, cudaStream_t st, const char *cache_path, int *chosen)
 {
-    if (cudaSetDevice(P->device) != cudaSuccess) return fail(JK_ERR_CUDA, "cudaSetDevice failed");
+    if (cudaSetDevice(P->device) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "cudaSetDevice failed");
     cudaDeviceProp prop;
     cudaGetDeviceProperties(&prop, P->device);
     const bool mixed = P->precision == JK_MIXED;
@@ -732,7 +732,7 @@ int autotune(Plan *P, const double *D, cudaStream_t st, const char *cache_path, 
                         if (cudaEventSynchronize(e1) != cudaSuccess) {
                             cudaEventDestroy(e0);
                             cudaEventDestroy(e1);
-                            return fail(JK_ERR_CUDA, "autotune launch failed");
+                            return fail_cuda(JK_ERR_CUDA, "autotune launch failed");
                     }
                         float ms = 0;
                         cudaEventElapsedTime(&ms, e0, e1);
@@ -794,21 +794,21 @@ int build_counts(Plan *P, long long *counts, int n)
     unsigned long long h[kCounters] = {};
     unsigned hb[2 * (1 + Plan::kSide)] = {};
     if (P->timer.next > 0 && cudaEventSynchronize(P->timer.pool[P->timer.next - 1]) != cudaSuccess)
-        return fail(JK_ERR_CUDA, "build did not finish");
-    if (cudaMemcpy(h, P->ws.cnt, sizeof h, cudaMemcpyDeviceToHost) != cudaSuccess) return fail(JK_ERR_CUDA, "count copy failed");
+        return fail_cuda(JK_ERR_CUDA, "build did not finish");
+    if (cudaMemcpy(h, P->ws.cnt, sizeof h, cudaMemcpyDeviceToHost) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "count copy failed");
     if (P->ws.nbig && cudaMemcpy(hb, P->ws.nbig, 2 * sizeof(unsigned) * P->ws.nlist, cudaMemcpyDeviceToHost) != cudaSuccess)
-        return fail(JK_ERR_CUDA, "count copy failed");
+        return fail_cuda(JK_ERR_CUDA, "count copy failed");
     for (int i = 1; i < P->ws.nlist; ++i) hb[1] += hb[2 * i + 1];
     // rank and form of the density factorisation (mixed builds with K)
     int dyn[4] = {0, 0, 0, 0};
     if (P->precision == JK_MIXED && P->ws.lr.dyn && cudaMemcpy(dyn, P->ws.lr.dyn, sizeof dyn, cudaMemcpyDeviceToHost) != cudaSuccess)
-        return fail(JK_ERR_CUDA, "status copy failed");
+        return fail_cuda(JK_ERR_CUDA, "status copy failed");
     // public layout (jk_build_counts)
     const long long out[13] = {(long long)h[0], (long long)h[1], (long long)hb[1], dyn[3], (long long)h[4], (long long)h[5], dyn[0],
                                (long long)h[8], (long long)h[9], (long long)h[12], (long long)h[14], (long long)h[13], (long long)h[15]};
     for (int i = 0; i < n && i < 13; ++i) counts[i] = out[i];
     unsigned e = 0;
-    if (cudaMemcpy(&e, P->ws.err, sizeof e, cudaMemcpyDeviceToHost) != cudaSuccess) return fail(JK_ERR_CUDA, "check word copy failed");
+    if (cudaMemcpy(&e, P->ws.err, sizeof e, cudaMemcpyDeviceToHost) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "check word copy failed");
     if (e) return fail(JK_ERR_TIMEOUT, "a bounded wait in a tensor-core GEMM ran out; J and K of that build are NaN");
     return JK_OK;
 }
@@ -821,7 +821,7 @@ int build_times(Plan *P, double *ms, int *launches, int n)
         if (launches) launches[i] = 0;
     }
     if (tm.marks.empty()) return JK_OK;
-    if (cudaEventSynchronize(tm.pool[tm.next - 1]) != cudaSuccess) return fail(JK_ERR_CUDA, "build did not finish");
+    if (cudaEventSynchronize(tm.pool[tm.next - 1]) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "build did not finish");
     for (auto &m : tm.marks) {
         float t = 0;
         cudaEventElapsedTime(&t, tm.pool[m.second.first], tm.pool[m.second.second]);
@@ -838,7 +838,7 @@ int build_times(Plan *P, double *ms, int *launches, int n)
         int dyn[3] = {0, 0, 0};
         if (P->precision == JK_MIXED && P->ws.lr.dyn &&
             cudaMemcpy(dyn, P->ws.lr.dyn, sizeof dyn, cudaMemcpyDeviceToHost) != cudaSuccess)
-            return fail(JK_ERR_CUDA, "status copy failed");
+            return fail_cuda(JK_ERR_CUDA, "status copy failed");
         ms[11] = P->precision == JK_MIXED ? ozaki_mma_flops(P, dyn) : 0.0;
     }
     return JK_OK;

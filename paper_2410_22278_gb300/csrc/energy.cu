@@ -103,10 +103,10 @@ __global__ void __launch_bounds__(kEnergyBlock) k_energy(size_t n2, const double
 int make_slot(EnergySlot &s, cudaStream_t st)
 {
     const size_t bytes = (2 * kEnergyGrid + 1) * sizeof(double);
-    if (cudaMalloc((void **)&s.part, bytes) != cudaSuccess) return fail(JK_ERR_OOM, "energy scratch");
+    if (cudaMalloc((void **)&s.part, bytes) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "energy scratch");
     if (cudaMemsetAsync(s.part, 0, bytes, st) != cudaSuccess || cudaHostAlloc((void **)&s.host, 2 * sizeof(double), cudaHostAllocMapped) != cudaSuccess) {
         cudaFree(s.part);
-        return fail(JK_ERR_OOM, "energy scratch");
+        return fail_cuda(JK_ERR_OOM, "energy scratch");
     }
     return JK_OK;
 }
@@ -124,11 +124,13 @@ int energy_reserve(Plan *P)
 
 void energy_release(Plan *P)
 {
-    for (auto &s : P->energy_free) {
-        cudaFree(s.part);
-        cudaFreeHost(s.host);
+    for (auto *slots : {&P->energy_free, &P->energy_lost}) {
+        for (auto &s : *slots) {
+            cudaFree(s.part);
+            cudaFreeHost(s.host);
+        }
+        slots->clear();
     }
-    P->energy_free.clear();
 }
 
 int energy(Plan *P, const double *D, const double *J, const double *K, double *e_coul, double *e_exch, cudaStream_t st)
@@ -148,17 +150,25 @@ int energy(Plan *P, const double *D, const double *J, const double *K, double *e
     const size_t n2 = (size_t)P->nbf * P->nbf;
     const int vec = (((uintptr_t)D | (uintptr_t)J | (uintptr_t)K) & 15) == 0;
     const unsigned grid = (unsigned)std::min<size_t>((n2 + 2 * kEnergyBlock - 1) / (2 * kEnergyBlock), kEnergyGrid);
-    k_energy<<<grid, kEnergyBlock, 0, st>>>(n2, D, J, K, vec, s.part, s.host);
-    const bool ok = cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(st) == cudaSuccess;
+    // The launch is judged by its own status, not by an error that an earlier
+    // call left in this thread, and the stream is waited for whatever it says:
+    // the kernel reads the caller's matrices and owns the slot until it ends.
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kEnergyBlock);
+    cfg.stream = st;
+    const cudaError_t launched = cudaLaunchKernelEx(&cfg, k_energy, n2, D, J, K, vec, s.part, s.host);
+    const cudaError_t done = cudaStreamSynchronize(st);
+    const bool ok = launched == cudaSuccess && done == cudaSuccess;
     if (ok) {
         *e_coul = 0.5 * s.host[0];
         *e_exch = -0.25 * s.host[1];
     }
     {
         std::lock_guard<std::mutex> g(P->energy_mu);
-        P->energy_free.push_back(s);
+        (ok ? P->energy_free : P->energy_lost).push_back(s);
     }
-    return ok ? JK_OK : fail(JK_ERR_CUDA, "energy reduction failed");
+    return ok ? JK_OK : fail_cuda(JK_ERR_CUDA, "energy reduction failed");
 }
 
 }  // namespace jk

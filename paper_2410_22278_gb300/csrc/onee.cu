@@ -432,7 +432,7 @@ int one_electron(Plan *P, int natom, const double *Z, const double *xyz, double 
     auto ok = [](cudaError_t e) { return e == cudaSuccess; };
     const int grid = (int)std::min<size_t>((n2 + 255) / 256, 152 * 16);
     if (T) {
-        if (!ok(cudaMemsetAsync(w.T1, 0, n2 * sizeof(double), st))) return fail(JK_ERR_CUDA, "memset failed");
+        if (!ok(cudaMemsetAsync(w.T1, 0, n2 * sizeof(double), st))) return fail_cuda(JK_ERR_CUDA, "memset failed");
         OneeArgs a{};
         a.pl = pl;
         a.op = 0;
@@ -443,7 +443,7 @@ int one_electron(Plan *P, int natom, const double *Z, const double *xyz, double 
         k_onee_final<<<grid, 256, 0, st>>>(n, P->d_compf, w.T1, P->d_S, 0.0, T);
         if (!ok(cudaGetLastError())) return fail(JK_ERR_CUDA, "kinetic-energy kernels failed");
     }
-    if (!V || natom <= 0) return ok(cudaStreamSynchronize(st)) ? JK_OK : fail(JK_ERR_CUDA, "one-electron kernels failed");
+    if (!V || natom <= 0) return ok(cudaStreamSynchronize(st)) ? JK_OK : fail_cuda(JK_ERR_CUDA, "one-electron kernels failed");
 
     // lattice candidates for the charges' images: |R| up to the largest
     // screening radius plus the cell's circumradius (the reduced X0 is at
@@ -496,7 +496,7 @@ int one_electron(Plan *P, int natom, const double *Z, const double *xyz, double 
     const int ng = (int)(P->gvec.size() / 4);
     const size_t oX = ((size_t)natom + 1) / 2 * 2, oC = oX + (3 * (size_t)natom + 1) / 2 * 2, oN = oC + 4 * (size_t)std::max(1, ncand);
     double *dZ = nullptr;
-    if (!ok(cudaMallocAsync((void **)&dZ, sizeof(double) * (oN + 2 * (size_t)std::max(1, ng)), st))) return fail(JK_ERR_OOM, "one-electron scratch");
+    if (!ok(cudaMallocAsync((void **)&dZ, sizeof(double) * (oN + 2 * (size_t)std::max(1, ng)), st))) return fail_cuda(JK_ERR_OOM, "one-electron scratch");
     double *dX = dZ + oX, *dC = dZ + oC;
     double2 *dn = reinterpret_cast<double2 *>(dZ + oN);
     cudaMemcpyAsync(dZ, Z, sizeof(double) * natom, cudaMemcpyHostToDevice, st);
@@ -547,8 +547,10 @@ int one_electron(Plan *P, int natom, const double *Z, const double *xyz, double 
     // self term +(pi/(V w^2)) Z_tot S and the component factors
     k_onee_final<<<grid, 256, 0, st>>>(n, P->d_compf, w.T2, P->d_S, kPi / (P->volume * w2) * ztot, V);
     cudaFreeAsync(dZ, st);
-    if (!good || !ok(cudaGetLastError()) || !ok(cudaStreamSynchronize(st))) return fail(JK_ERR_CUDA, "nuclear-attraction kernels failed");
-    return JK_OK;
+    // waited for on every path: the copies above read the caller's host arrays
+    good = ok(cudaGetLastError()) && good;
+    good = ok(cudaStreamSynchronize(st)) && good;
+    return good ? JK_OK : fail_cuda(JK_ERR_CUDA, "nuclear-attraction kernels failed");
 }
 
 }  // namespace jk

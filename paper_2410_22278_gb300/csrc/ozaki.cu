@@ -595,11 +595,11 @@ int ozaki_setup_tc(Plan *P)
     const int nt = npad / TC_BM, ntri = nt * (nt + 1) / 2;
     w.kpart_splits = std::max(1, std::min(32, (4 * 152 + ntri / 2) / ntri));
     const size_t bytes = (size_t)w.kpart_splits * n * n * sizeof(double);
-    if (cudaMalloc((void **)&w.Kpart, bytes) != cudaSuccess) return fail(JK_ERR_OOM, "cudaMalloc failed for exchange partial sums");
+    if (cudaMalloc((void **)&w.Kpart, bytes) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed for exchange partial sums");
     w.bytes += bytes;
     if (cudaFuncSetAttribute(k_ozaki_tc<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM) != cudaSuccess ||
         cudaFuncSetAttribute(k_ozaki_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM) != cudaSuccess)
-        return fail(JK_ERR_CUDA, "cudaFuncSetAttribute failed for the tensor-core GEMM");
+        return fail_cuda(JK_ERR_CUDA, "cudaFuncSetAttribute failed for the tensor-core GEMM");
     w.tc = true;
     return JK_OK;
 }
@@ -768,14 +768,13 @@ int cache_reciprocal(Plan *P, size_t max_bytes)
     }
     if (cudaMalloc((void **)&c.M, bM) != cudaSuccess || (mixed && cudaMalloc((void **)&c.Ms, bS) != cudaSuccess) ||
         (mixed && cudaMalloc((void **)&c.Mex, bX) != cudaSuccess)) {
-        cudaGetLastError();
         release_cache(P);
-        return fail(JK_ERR_OOM, "cudaMalloc failed for the reciprocal cache");
+        return fail_cuda(JK_ERR_OOM, "cudaMalloc failed for the reciprocal cache");
     }
     // entries of shell pairs without images are never written
     if (cudaMemset(c.M, 0, bM) != cudaSuccess) {
         release_cache(P);
-        return fail(JK_ERR_CUDA, "cudaMemset failed for the reciprocal cache");
+        return fail_cuda(JK_ERR_CUDA, "cudaMemset failed for the reciprocal cache");
     }
     if (mixed && !slice_map(&c.tm_Ms, c.Ms, rows, w.npad)) {
         release_cache(P);

@@ -19,6 +19,11 @@ int fail(int status, const std::string &msg)
     g_last_error = msg;
     return status;
 }
+int fail_cuda(int status, const std::string &msg)
+{
+    (void)cudaGetLastError();
+    return fail(status, msg);
+}
 const char *last_error_str() { return g_last_error.c_str(); }
 
 static const double kPi = 3.14159265358979323846;
@@ -401,9 +406,9 @@ template <class T>
 static int upload(const std::vector<T> &h, T **d, size_t &bytes)
 {
     size_t n = std::max<size_t>(h.size(), 1) * sizeof(T);
-    if (cudaMalloc((void **)d, n) != cudaSuccess) return fail(JK_ERR_OOM, "cudaMalloc failed for plan array");
+    if (cudaMalloc((void **)d, n) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed for plan array");
     if (!h.empty() && cudaMemcpy(*d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice) != cudaSuccess)
-        return fail(JK_ERR_CUDA, "cudaMemcpy failed for plan array");
+        return fail_cuda(JK_ERR_CUDA, "cudaMemcpy failed for plan array");
     bytes += n;
     return JK_OK;
 }
@@ -466,12 +471,12 @@ static int alloc_ws(Plan *P)
         const size_t nh = std::max<size_t>(1, P->ppi.size()) * w.hs;
         ok = ok && al(&w.DhD, nh) && al(&w.JH, nh) && al((double **)&w.DhF, (nh + 1) / 2);
     }
-    if (!ok) return fail(JK_ERR_OOM, "cudaMalloc failed for build workspace");
+    if (!ok) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed for build workspace");
     // the structure-factor kernels write only the entries of shell pairs with
     // images, the same ones for every G; the others must read as zero
     if (cudaMemset(w.M, 0, 2 * (size_t)gc * n2 * sizeof(double)) != cudaSuccess ||
         cudaMemset(w.Z, 0, 2 * (size_t)gc * n2 * sizeof(double)) != cudaSuccess)
-        return fail(JK_ERR_CUDA, "cudaMemset failed for the structure-factor slab");
+        return fail_cuda(JK_ERR_CUDA, "cudaMemset failed for the structure-factor slab");
     if (mixed) {
         const size_t sl = (size_t)w.oz_slices * w.npad * w.npad;
         auto alb = [&](__nv_bfloat16 **ptr, size_t count) -> bool {
@@ -485,12 +490,12 @@ static int alloc_ws(Plan *P)
             return true;
         };
         if (cudaMalloc((void **)&w.gtab2, std::max<size_t>(1, P->pvals.size()) * (size_t)gc * sizeof(float2)) != cudaSuccess)
-            return fail(JK_ERR_OOM, "cudaMalloc failed for the double-float Gaussian table");
+            return fail_cuda(JK_ERR_OOM, "cudaMalloc failed for the double-float Gaussian table");
         bytes += std::max<size_t>(1, P->pvals.size()) * (size_t)gc * sizeof(float2);
         if (!alb(&w.Ms, 2 * (size_t)gc * sl) || !alb(&w.Zs, 2 * (size_t)gc * sl) || !alb(&w.Ds, sl) || !alb(&w.Cs, sl) ||
             !ali(&w.Mex, 2 * (size_t)gc * w.npad) || !ali(&w.Zex, 2 * (size_t)gc * w.npad) || !ali(&w.Dex, w.npad) ||
             !ali(&w.Cex, w.npad))
-            return fail(JK_ERR_OOM, "cudaMalloc failed for tensor-core exchange workspace");
+            return fail_cuda(JK_ERR_OOM, "cudaMalloc failed for tensor-core exchange workspace");
         // low-rank form of D: worth it while the padded rank stays within 60%
         // of npad (closed-shell densities have rank n_occ)
         LowRankWs &lr = w.lr;
@@ -498,18 +503,18 @@ static int alloc_ws(Plan *P)
         const size_t rc = (size_t)std::max(lr.rcap, 1);
         if (!al(&lr.Vt, (size_t)P->nbf * rc) || !al(&lr.diag, P->nbf) || !ali(&lr.done_row, P->nbf) || !al(&lr.sgn, rc) ||
             !ali(&lr.rowmap, rc) || !ali(&lr.dyn, 8) || !ali((int **)&lr.bar, 1) || !al(&lr.Ct, rc * P->nbf))
-            return fail(JK_ERR_OOM, "cudaMalloc failed for the low-rank factorisation");
+            return fail_cuda(JK_ERR_OOM, "cudaMalloc failed for the low-rank factorisation");
         cudaMemset(lr.dyn, 0, 8 * sizeof(int));
     }
-    if (cudaMalloc((void **)&w.err, sizeof(unsigned)) != cudaSuccess) return fail(JK_ERR_OOM, "cudaMalloc failed");
-    if (cudaMalloc((void **)&w.cnt, kCounters * sizeof(unsigned long long)) != cudaSuccess) return fail(JK_ERR_OOM, "cudaMalloc failed");
+    if (cudaMalloc((void **)&w.err, sizeof(unsigned)) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed");
+    if (cudaMalloc((void **)&w.cnt, kCounters * sizeof(unsigned long long)) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed");
     if (P->precision == JK_MIXED) {
         // the FP64 share is a small fraction; the list holds up to 2% of all image quartets (at most 64 Mi entries)
         const long long want = std::min<long long>(std::max<long long>(P->n_quartets / 50, 1 << 20), 64ll << 20);
         w.cap = (unsigned)want;
         w.nlist = std::max(1, P->nside);  // the caller's stream and all but the last side stream
-        if (cudaMalloc((void **)&w.big, sizeof(int2) * w.cap * w.nlist) != cudaSuccess) return fail(JK_ERR_OOM, "cudaMalloc failed for quartet list");
-        if (cudaMalloc((void **)&w.nbig, 2 * sizeof(unsigned) * w.nlist) != cudaSuccess) return fail(JK_ERR_OOM, "cudaMalloc failed");
+        if (cudaMalloc((void **)&w.big, sizeof(int2) * w.cap * w.nlist) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed for quartet list");
+        if (cudaMalloc((void **)&w.nbig, 2 * sizeof(unsigned) * w.nlist) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed");
         bytes += (sizeof(int2) * w.cap + 2 * sizeof(unsigned)) * w.nlist;
     }
     cudaMemset(w.err, 0, sizeof(unsigned));
@@ -976,7 +981,7 @@ int build_plan(const jk_cell *cell, const jk_shell *shells, int nshell, double o
 // Device side of plan creation: uploads, Boys tables, workspace, overlap.
 int finish_plan_device(Plan *P)
 {
-    if (cudaSetDevice(P->device) != cudaSuccess) return fail(JK_ERR_CUDA, "cudaSetDevice failed");
+    if (cudaSetDevice(P->device) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "cudaSetDevice failed");
     int rc;
     size_t &b = P->device_bytes;
     {
@@ -1168,18 +1173,18 @@ int finish_plan_device(Plan *P)
     // (ss|ss) launch alone keeps the chip busy, and each lane needs a list of
     // large quartets of its own
     if (P->n_quartets <= 200000000LL) {
-        if (cudaEventCreateWithFlags(&P->side_fork, cudaEventDisableTiming) != cudaSuccess) return fail(JK_ERR_CUDA, "cudaEventCreate failed");
+        if (cudaEventCreateWithFlags(&P->side_fork, cudaEventDisableTiming) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "cudaEventCreate failed");
         for (int i = 0; i < Plan::kSide; ++i) {
-            if (cudaStreamCreateWithFlags(&P->side[i], cudaStreamNonBlocking) != cudaSuccess) return fail(JK_ERR_CUDA, "cudaStreamCreate failed");
+            if (cudaStreamCreateWithFlags(&P->side[i], cudaStreamNonBlocking) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "cudaStreamCreate failed");
             P->nside = i + 1;
             if (cudaEventCreateWithFlags(&P->side_join[i], cudaEventDisableTiming) != cudaSuccess)
-                return fail(JK_ERR_CUDA, "cudaEventCreate failed");
+                return fail_cuda(JK_ERR_CUDA, "cudaEventCreate failed");
         }
     }
     if ((rc = alloc_ws(P))) return rc;
     if ((rc = energy_reserve(P))) return rc;
     if ((rc = compute_overlap_raw(P, 0))) return rc;
-    if (cudaDeviceSynchronize() != cudaSuccess) return fail(JK_ERR_CUDA, "plan setup kernels failed");
+    if (cudaDeviceSynchronize() != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "plan setup kernels failed");
     return JK_OK;
 }
 

@@ -17,6 +17,10 @@ namespace jk {
 
 // thread-local last error; returns the status for convenience
 int fail(int status, const std::string &msg);
+// the same for a CUDA call that failed: the runtime keeps a thread's last error
+// until it is read, and here it is reported, so that a later call's check of
+// its own launches does not find it again
+int fail_cuda(int status, const std::string &msg);
 
 struct ClassRange {
     int la, lb;
@@ -115,7 +119,8 @@ struct RecipCache {
 
 // Scratch of one jk_energy call: block partials and a block counter on the
 // device, the two sums in pinned host memory.  A plan keeps one per call that
-// was ever in flight on it at once.
+// was ever in flight on it at once.  The slot of a call whose kernel was not
+// seen to finish is not used again and is freed with the plan.
 struct EnergySlot {
     double *part = nullptr;
     double *host = nullptr;
@@ -200,6 +205,7 @@ struct Plan {
     std::mutex build_mu;
     std::mutex energy_mu;
     std::vector<EnergySlot> energy_free;  // not in use by a call
+    std::vector<EnergySlot> energy_lost;  // left by a failed call
     PlanDev dev() const;
 };
 
