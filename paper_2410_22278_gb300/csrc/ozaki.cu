@@ -38,6 +38,7 @@
 #include <string>
 #include <vector>
 
+#include "digits.cuh"
 #include "plan.h"
 #include "tc.cuh"
 
@@ -57,40 +58,46 @@ __device__ __forceinline__ void two_sum_add(float &hi, float &lo, float x)
 
 }  // namespace
 
-// The first S digits of two adjacent values, stored as one bf16 pair per slice.
-// With W = V + sum_{s>=1} 128 * 2^{55 - 8s} + 64 the balanced digits are plain bits
-// of W: d_0 = W >> 55 and d_s = ((W >> (55 - 8s)) & 255) - 128 (V = sum_s d_s
-// 2^{55 - 8s} + the low bits - 64, identically), so a digit costs a shift, a mask
-// and one exact float subtraction instead of a 64-bit rounding, shift, multiply
-// and subtraction and an integer conversion (which runs at an eighth of the
-// FP32 rate); the slicing is left to the memory system.
+// The first S digits of two adjacent values (digits.cuh; off = digit_offset(S)),
+// stored as one bf16 pair per slice: a digit costs a shift, a mask and one
+// exact float subtraction instead of a 64-bit rounding, shift, multiply and
+// subtraction and an integer conversion (which runs at an eighth of the FP32
+// rate); the slicing is left to the memory system.
+__device__ __forceinline__ float int_f(int d) { return __int_as_float(0x4b400000 + d) - 12582912.0f; }                       // 1.5 * 2^23
 __device__ __forceinline__ float digit_f(unsigned byte) { return __uint_as_float(0x4b000000u | byte) - 8388736.0f; }  // 2^23 + 128
-__device__ __forceinline__ void store_digits(long long V0, long long V1, int S, __nv_bfloat16 *o, size_t sstride)
+__device__ __forceinline__ void store_digits(long long V0, long long V1, int S, long long off, __nv_bfloat16 *o, size_t sstride)
 {
-    constexpr long long B = (128LL << 47) + (128LL << 39) + (128LL << 31) + (128LL << 23) + (128LL << 15) + (128LL << 7) + 64;
-    const long long W0 = V0 + B, W1 = V1 + B;
-    const int t0 = (int)(W0 >> 55), t1 = (int)(W1 >> 55);  // in [-128, 128]
-    *reinterpret_cast<__nv_bfloat162 *>(o) =
-        __floats2bfloat162_rn(__int_as_float(0x4b400000 + t0) - 12582912.0f, __int_as_float(0x4b400000 + t1) - 12582912.0f);
+    const long long W0 = V0 + off, W1 = V1 + off;
+    *reinterpret_cast<__nv_bfloat162 *>(o) = __floats2bfloat162_rn(int_f(digit_top(W0)), int_f(digit_top(W1)));
 #pragma unroll
     for (int s = 1; s < 7; ++s)
         if (s < S)
             *reinterpret_cast<__nv_bfloat162 *>(o + s * sstride) =
-                __floats2bfloat162_rn(digit_f((unsigned)(W0 >> (55 - 8 * s)) & 255u), digit_f((unsigned)(W1 >> (55 - 8 * s)) & 255u));
+                __floats2bfloat162_rn(digit_f(digit_byte(W0, s)), digit_f(digit_byte(W1, s)));
+}
+// the form whose every prefix is rounded to nearest
+__device__ __forceinline__ void store_digits_prefix(long long V0, long long V1, int S, __nv_bfloat16 *o, size_t sstride)
+{
+    unsigned p0 = 0, p1 = 0;
+#pragma unroll 1
+    for (int s = 0; s < S; ++s) {
+        const unsigned q0 = digit_prefix(V0, s), q1 = digit_prefix(V1, s);
+        *reinterpret_cast<__nv_bfloat162 *>(o + s * sstride) = __floats2bfloat162_rn(int_f((int)(q0 - 256u * p0)), int_f((int)(q1 - 256u * p1)));
+        p0 = q0;
+        p1 = q1;
+    }
 }
 
 // Slices of a batch of rows x cols FP64 matrices (row-major, leading dim ld,
 // batch stride bstride elements): one warp per row.  sigma = E_max - 1022
 // with E_max the largest biased exponent in the row (so |x| < 2^sigma);
 // V = x 2^{62 - sigma} (|V| < 2^62) is formed exactly as a signed 64-bit
-// integer by shifting the 53-bit significand, and the digits are read off
-// store_digits' shifted form: d_0 in [-128, 128], the others in [-128, 127],
-// and what is left after S of them is at most 0.51 of the last place.  S <= 7.
-// Output:
+// integer by shifting the 53-bit significand, and cut into S <= 7 digits
+// (digits.cuh; prefix: the operand is read through fewer digits too).  Output:
 // out[((b*S + s)*rows_pad + r)*cols_pad + k] (zero outside rows x cols),
 // ex[b*rows_pad + r].
 __global__ void k_ozaki_slice(const double *__restrict__ X, int rows, int cols, int ld, long long bstride, int rows_pad, int cols_pad,
-                              int S, int B, __nv_bfloat16 *__restrict__ out, int *__restrict__ ex)
+                              int S, bool prefix, int B, __nv_bfloat16 *__restrict__ out, int *__restrict__ ex)
 {
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -106,6 +113,7 @@ __global__ void k_ozaki_slice(const double *__restrict__ X, int rows, int cols, 
     if (lane == 0) ex[(size_t)b * rows_pad + r] = sigma;
     __nv_bfloat16 *o = out + ((size_t)b * S * rows_pad + r) * cols_pad;
     const size_t sstride = (size_t)rows_pad * cols_pad;
+    const long long off = digit_offset(S);
     auto scaled = [&](int k) -> long long {
         if (r >= rows || k >= cols) return 0;
         const unsigned long long bits = row[k];
@@ -119,8 +127,9 @@ __global__ void k_ozaki_slice(const double *__restrict__ X, int rows, int cols, 
     // two adjacent columns per lane, stored as one bf16 pair per slice
     // (cols_pad and the slice stride are even)
     for (int k = 2 * lane; k < cols_pad; k += 64) {
-        long long V0 = scaled(k), V1 = scaled(k + 1);
-        store_digits(V0, V1, S, o + k, sstride);
+        const long long V0 = scaled(k), V1 = scaled(k + 1);
+        if (prefix) store_digits_prefix(V0, V1, S, o + k, sstride);
+        else store_digits(V0, V1, S, off, o + k, sstride);
     }
 }
 
@@ -490,6 +499,7 @@ __global__ void k_ozaki_slice_pair(const float2 *__restrict__ X, int rows, int c
     if (lane == 0) ex[(size_t)b * rows_pad + r] = sigma;
     __nv_bfloat16 *o = out + ((size_t)b * S * rows_pad + r) * cols_pad;
     const size_t sstride = (size_t)rows_pad * cols_pad;
+    const long long off = digit_offset(S);
     auto part = [&](float f) -> long long {
         const unsigned u = __float_as_uint(f);
         const int E = (int)((u >> 23) & 0xff);
@@ -516,16 +526,17 @@ __global__ void k_ozaki_slice_pair(const float2 *__restrict__ X, int rows, int c
                 V1 = part(x.x) + part(x.y);
             }
         }
-        store_digits(V0, V1, S, o + k, sstride);
+        store_digits(V0, V1, S, off, o + k, sstride);
     }
 }
 
 static unsigned blocks_for_rows(long long rows) { return (unsigned)((rows * 32 + 255) / 256); }
 
-static void slice(const double *X, int rows, int cols, int ld, long long bstride, int rows_pad, int cols_pad, int S, int B,
-                  __nv_bfloat16 *out, int *ex, cudaStream_t st)
+static void slice(const double *X, int rows, int cols, int ld, long long bstride, int rows_pad, int cols_pad, int S, bool prefix,
+                  int B, __nv_bfloat16 *out, int *ex, cudaStream_t st)
 {
-    k_ozaki_slice<<<blocks_for_rows((long long)B * rows_pad), 256, 0, st>>>(X, rows, cols, ld, bstride, rows_pad, cols_pad, S, B, out, ex);
+    k_ozaki_slice<<<blocks_for_rows((long long)B * rows_pad), 256, 0, st>>>(X, rows, cols, ld, bstride, rows_pad, cols_pad, S, prefix, B, out,
+                                                                             ex);
 }
 
 static void slice_pair(const float2 *X, int rows, int cols, int ld, long long bstride, int rows_pad, int cols_pad, int S, int B,
@@ -628,11 +639,11 @@ int ozaki_begin(Plan *P, cudaStream_t st)
     Workspace &w = P->ws;
     const int n = P->nbf;
     w.chunk_log.clear();
-    slice(w.Dp, n, n, n, 0, w.npad, w.npad, w.oz_slices, 1, w.Ds, w.Dex, st);
+    slice(w.Dp, n, n, n, 0, w.npad, w.npad, w.oz_slices, true, 1, w.Ds, w.Dex, st);
     cudaMemsetAsync(w.Kpart, 0, (size_t)w.kpart_splits * n * n * sizeof(double), st);
     int rc = lowrank_factor(w.Dp, n, w.lr.rcap, 1e-12, w.lr, w.err, st);
     if (rc) return rc;
-    if (w.lr.rcap > 0) slice(w.lr.Ct, w.lr.rcap, n, n, 0, w.lr.rcap, w.npad, w.oz_slices, 1, w.Cs, w.Cex, st);
+    if (w.lr.rcap > 0) slice(w.lr.Ct, w.lr.rcap, n, n, 0, w.lr.rcap, w.npad, w.oz_slices, true, 1, w.Cs, w.Cex, st);
     return check("density slices and low-rank factor");
 }
 
@@ -659,7 +670,7 @@ int ozaki_exchange_chunk(Plan *P, int chunk, const double *Mc, int m2, int S, cu
     const CUtensorMap &tmM = cached ? cc.tm_Ms : w.tm_Ms;
     const int mrow0 = cached ? (int)cc.row0[chunk] : 0;
     int ev = tm.start(8);
-    if (!cached || !cc.s_valid) slice(Mc, n, n, n, (long long)n * n, npad, npad, S, m2, Ms, Mex, st);
+    if (!cached || !cc.s_valid) slice(Mc, n, n, n, (long long)n * n, npad, npad, S, false, m2, Ms, Mex, st);
     tm.stop(8, ev, 1);
     {
         // dense form: Zt_b = (D M_b)^T, as (hi, lo) pairs ...
