@@ -383,6 +383,7 @@ template <int NV, typename T>
 struct BatchShape {
     static constexpr int per = NV * (int)sizeof(T);
     static constexpr int SL = per <= 24 ? 128 : per <= 36 ? 64 : per <= 144 ? 32 : per <= 216 ? 16 : 8;
+    static constexpr int LO = sizeof(T) == 4 ? SL / 2 * NV : 0;  // rounding errors of the sums of a deep bra (k_real_w)
     static constexpr int KQ = SL == 128 ? 256 : SL == 64 ? 128 : 64;  // ring of queued kets, at least SL + 31
 };
 constexpr int kBraChunk = 16;    // bra primitives screened per round (bits of a lane's mask)
@@ -645,8 +646,9 @@ __device__ __forceinline__ bool prim_maybe(const PlanDev &pl, const float4 &b, c
 // A ring entry holds the slot, the positions i and j of the bra and ket
 // primitive pairs in their images (first ones: bra0(slot), ket0(slot)) and a
 // group: the entries of one slot and group are adjacent.  several: a slot may
-// come with more than one group.
-template <int LA, int LB, int LC, int LD, typename T, int RING, bool SHARE, class BraFn, class KetFn>
+// come with more than one group, and (LO > 0) the blocks are sums with their
+// rounding errors LO elements further on.
+template <int LA, int LB, int LC, int LD, typename T, int RING, bool SHARE, int LO, class BraFn, class KetFn>
 __device__ __forceinline__ void eval_terms(const PlanDev &pl, const unsigned *ring, unsigned qd, unsigned count, BraFn bra0, KetFn ket0,
                                            bool several, T *Vs, Tally &tl, unsigned &used, bool share = false,
                                            ImgShare<LA + LB + LC + LD, T> *img = nullptr)
@@ -720,6 +722,14 @@ __device__ __forceinline__ void eval_terms(const PlanDev &pl, const unsigned *ri
     const unsigned prev = __shfl_up_sync(0xffffffffu, key, 1);
     const bool head = on && (lane == 0 || prev != key);
     T *dst = Vs + (head ? key & 127u : 0u) * NV;
+    const auto add_compensated = [&] {  // two-sum
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            const T h = dst[q], t = h + V[q], b = t - h;
+            dst[q] = t;
+            dst[LO + q] += (h - (t - b)) + (V[q] - b);
+        }
+    };
     if (!several) {
         if (head)
 #pragma unroll
@@ -730,9 +740,14 @@ __device__ __forceinline__ void eval_terms(const PlanDev &pl, const unsigned *ri
         const int rank = __popc(m & ((1u << lane) - 1u));
 #pragma unroll 1
         for (int rr = 0; __any_sync(0xffffffffu, head && rank >= rr); ++rr) {
-            if (head && rank == rr)
+            if (head && rank == rr) {
+                if constexpr (LO > 0) {
+                    add_compensated();
+                } else {
 #pragma unroll
-                for (int q = 0; q < NV; ++q) dst[q] += V[q];
+                    for (int q = 0; q < NV; ++q) dst[q] += V[q];
+                }
+            }
             __syncwarp();
         }
     }
@@ -761,6 +776,10 @@ __device__ __forceinline__ void eval_terms(const PlanDev &pl, const unsigned *ri
 // each stage refills the warp; with one ket's primitives per step and the
 // screening, the terms and the digestion in one loop body about a tenth of
 // the lanes were active.
+// The sums of a deep bra are compensated in single precision: rounded at every
+// batch, the K of a diamond cell with every quartet in FP32 was 1.2e-7 off
+// (rms) against 0.7e-7 now and 0.95e-7 with the terms of a ket primitive summed
+// in a lane.
 // Counters (cnt, one precision's base): [0] image quartets evaluated, [4]
 // algorithmic flops, [8] screening and bookkeeping flops, [12] primitive
 // quartets evaluated and [14] lane slots offered to them (their ratio is the
@@ -774,7 +793,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, tile_blocks<T>(LA + LB + 
 {
     constexpr int NA = ncart(LA), NB = ncart(LB), NC = ncart(LC), ND = ncart(LD), NV = NA * NB * NC * ND;
     constexpr int L = LA + LB + LC + LD;
-    constexpr int SL = BatchShape<NV, T>::SL, KQ = BatchShape<NV, T>::KQ;
+    constexpr int SL = BatchShape<NV, T>::SL, KQ = BatchShape<NV, T>::KQ, LO = BatchShape<NV, T>::LO;
     __shared__ unsigned ring_s[kWarpsPerBlock][kTermRing];
     __shared__ int kq_s[kWarpsPerBlock][KQ], pp0_s[kWarpsPerBlock][SL];
     __shared__ T V_s[kWarpsPerBlock][SL * NV];
@@ -789,6 +808,11 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, tile_blocks<T>(LA + LB + 
     const SpiRec sb = pl.spi[bra];
     const int n = pl.nbf;
     const int aoI = pl.shells[sb.I].ao, aoJ = pl.shells[sb.J].ao;
+    // A bra of many primitives adds up to 65536 terms to a block, 32 at a time:
+    // in single precision its sums carry their rounding errors along, in the
+    // upper half of the slots (its batches are full with half as many kets).
+    const bool deep = LO > 0 && sb.npp > kBraChunk;
+    const int nslot = deep ? SL / 2 : SL;
     T Dij[NA * NB];
     Acc<T> jb[NA * NB];
 #pragma unroll
@@ -812,7 +836,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, tile_blocks<T>(LA + LB + 
     unsigned qn = 0, qd = 0;
     // evaluate the next count queued primitive quartets
     auto eval = [&](unsigned count) {
-        eval_terms<LA, LB, LC, LD, T, kTermRing, ImgShare<L, T>::on>(
+        eval_terms<LA, LB, LC, LD, T, kTermRing, ImgShare<L, T>::on, LO>(
             pl, ring, qd, count, [&](unsigned) { return sb.pp0; }, [&](unsigned slot) { return kpp0[slot]; }, sb.npp > kBraChunk, Vs, tl,
             used, share, &img_s[wid]);
         slots += lane == 0 ? 32u : 0u;
@@ -821,7 +845,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, tile_blocks<T>(LA + LB + 
     // screen, evaluate and digest the next count queued kets
     auto process = [&](int count) {
 #pragma unroll 1
-        for (int q = lane; q < count * NV; q += 32) Vs[q] = T(0);
+        for (int q = lane; q < (deep ? SL : count) * NV; q += 32) Vs[q] = T(0);
         unsigned grp = 0;
 #pragma unroll 1
         for (int s0 = 0; s0 < count; s0 += 32) {
@@ -921,6 +945,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, tile_blocks<T>(LA + LB + 
 #pragma unroll
             for (int q = 0; q < NV; ++q) {
                 V[q] = Vs[sl * NV + q];
+                if (LO > 0 && deep) V[q] += Vs[LO + sl * NV + q];
                 any = any || V[q] != T(0);
             }
             if (any) {
@@ -958,9 +983,9 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, tile_blocks<T>(LA + LB + 
             if (valid) kq[(kn + __popc(vmask & ((1u << lane) - 1u))) & (KQ - 1)] = kt;
             kn += __popc(vmask);
             __syncwarp();
-            const unsigned lim = last && !bm ? 1u : (unsigned)SL;
+            const unsigned lim = last && !bm ? 1u : (unsigned)nslot;
 #pragma unroll 1
-            while (kn - kd >= lim) process((int)min((unsigned)SL, kn - kd));
+            while (kn - kd >= lim) process((int)min((unsigned)nslot, kn - kd));
         } while (bm);
     }
     // bra-side Coulomb: one atomic per element for the warp
@@ -1280,7 +1305,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, LA + LB + LC + LD <= 3 ? 
 #pragma unroll 1
             while (qn - qd >= lim) {
                 const unsigned count = min(32u, qn - qd);
-                eval_terms<LA, LB, LC, LD, double, kListRing, false>(
+                eval_terms<LA, LB, LC, LD, double, kListRing, false, 0>(
                     pl, ring, qd, count, [&](unsigned s) { return bpp0[s]; }, [&](unsigned s) { return kpp0[s]; }, false, Vs, tl, used);
                 qd += count;
                 slots += lane == 0 ? 32u : 0u;

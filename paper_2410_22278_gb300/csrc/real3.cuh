@@ -79,7 +79,17 @@ __device__ __forceinline__ bool coop_quartet(const PlanDev &pl, const SpiRec &sb
     const int nterm = sb.npp * sk.npp;
     const float4 *lat = reinterpret_cast<const float4 *>(pl.r1f);
     bool some = false;
-    for (int o = lane; o < S::NAB * S::NCD; o += 32) s.V[o] = T(0);
+    // Rounding errors of the block's sums over the primitive quartets, in
+    // registers (single precision, up to four elements a lane: (pp|pp) and the
+    // smaller blocks with d).  (pp|pp) adds up to 1296 terms; rounded at each,
+    // the K of water boxes with every quartet in FP32 was 1.8e-7 off (rms, 5
+    // molecules) against 1.1e-7 for sums over ket primitives by a tree.
+    constexpr int NV = S::NAB * S::NCD, LV = (NV + 31) / 32;
+    constexpr bool comp = sizeof(T) == 4 && LV <= 4;
+    T lo[comp ? LV : 1];
+#pragma unroll
+    for (int k = 0; k < (comp ? LV : 1); ++k) lo[k] = T(0);
+    for (int o = lane; o < NV; o += 32) s.V[o] = T(0);
     for (int t0 = 0; t0 < nterm; t0 += 32) {
         const int tt = t0 + lane;
         bool pass = false;
@@ -244,7 +254,7 @@ __device__ __forceinline__ bool coop_quartet(const PlanDev &pl, const SpiRec &sb
                     s.W[o] = acc;
                 }
                 __syncwarp();
-                for (int o = lane; o < S::NAB * S::NCD; o += 32) {
+                const auto element = [&](int o) {
                     const int ab = o / S::NCD, cd = o - ab * S::NCD;
                     const int ax = s.eab[ab][0], ay = s.eab[ab][1], az = s.eab[ab][2];
                     const int bx = s.eab[ab][3], by = s.eab[ab][4], bz = s.eab[ab][5];
@@ -257,11 +267,29 @@ __device__ __forceinline__ bool coop_quartet(const PlanDev &pl, const SpiRec &sb
                             for (int uz = 0; uz <= az + bz; ++uz) in += e2[uz] * s.W[s.tix[(ux * NTA + uy) * NTA + uz] * S::NCD + cd];
                             acc += e0[ux] * e1[uy] * in;
                         }
-                    s.V[o] += acc;
+                    return acc;
+                };
+                if constexpr (comp) {
+#pragma unroll
+                    for (int k = 0; k < LV; ++k) {
+                        const int o = lane + 32 * k;
+                        if (o >= NV) break;
+                        const T x = element(o), h = s.V[o], t = h + x, b = t - h;
+                        s.V[o] = t;
+                        lo[k] += (h - (t - b)) + (x - b);
+                    }
+                } else {
+                    for (int o = lane; o < NV; o += 32) s.V[o] += element(o);
                 }
                 __syncwarp();
             }
         }
+    }
+    if constexpr (comp) {
+#pragma unroll
+        for (int k = 0; k < LV; ++k)
+            if (lane + 32 * k < NV) s.V[lane + 32 * k] += lo[k];
+        __syncwarp();
     }
     return some;
 }
