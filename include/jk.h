@@ -282,7 +282,7 @@ int jk_overlap(const jk_plan *plan, double *S, void *cuda_stream);
  * T and V are device pointers (nbf x nbf, row-major, FP64; either may be
  * NULL); the caller owns them.  Uses the plan's build workspace, so it is
  * ordered after earlier builds on the plan; synchronises `cuda_stream`
- * before returning.  With the electron density D, E_kin = sum D o T and
+ * before returning.  A repeated call gives the same bits.  With the electron density D, E_kin = sum D o T and
  * E_ne = sum D o V; the nuclear repulsion is jk_ewald_point_charges.
  * Errors: JK_ERR_INVALID (NULL plan, natom < 0, charges missing),
  * JK_ERR_OOM, JK_ERR_CUDA. */

@@ -252,11 +252,11 @@ void slab_gemv_t(const double *M, long long n2, int m2, const double *x, double 
     k_slab_dot_final<<<(m2 + 127) / 128, 128, 0, st>>>(m2, splits, part, rho);
 }
 
-void slab_gemv_n(const double *M, long long n2, int m2, const double *rho, double alpha, double *y, cudaStream_t st)
+void slab_gemv_n(const double *M, long long n2, int m2, const double *rho, double alpha, double *y, cudaStream_t st, bool split)
 {
     if (m2 <= 0 || n2 <= 0) return;
     const int nx = (int)((n2 + 255) / 256);
-    const int ns = std::max(1, std::min((152 * 8 + nx - 1) / nx, m2 / 64)), per = (m2 + ns - 1) / ns;
+    const int ns = split ? std::max(1, std::min((152 * 8 + nx - 1) / nx, m2 / 64)) : 1, per = (m2 + ns - 1) / ns;
     k_slab_axpy<<<dim3(nx, (m2 + per - 1) / per), 256, 0, st>>>(M, n2, m2, rho, alpha, per, y);
 }
 

@@ -22,8 +22,9 @@ struct LowRankWs {
 // m2 * kSlabSplitsMax partial sums.
 constexpr int kSlabSplitsMax = 1024;
 void slab_gemv_t(const double *M, long long n2, int m2, const double *x, double *part, double *rho, cudaStream_t st);
-// y[i] += alpha sum_b M[b][i] rho[b].
-void slab_gemv_n(const double *M, long long n2, int m2, const double *rho, double alpha, double *y, cudaStream_t st);
+// y[i] += alpha sum_b M[b][i] rho[b]; split: the slabs may be split over blocks
+// that add by atomics (in any order).
+void slab_gemv_n(const double *M, long long n2, int m2, const double *rho, double alpha, double *y, cudaStream_t st, bool split = true);
 // The same two passes over full n x n slabs of symmetric matrices, reading one
 // triangle: rho[b] = sum_ij M[b][ij] D[ij] (Ds, n x n scratch, receives the
 // symmetrised D) and y[ij] += sum_b M[b][ij] rho[b].

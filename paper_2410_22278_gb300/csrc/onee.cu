@@ -67,18 +67,38 @@ __device__ __forceinline__ void kinetic_block(const PpiRec &x, double b, double 
         }
 }
 
-// Add the block of one shell-pair image to the raw matrix: element (a, b) and,
-// unless the image is its own mirror (I = J, R = 0), the transposed one.  The
-// two triangles get the same terms; k_onee_final reads one of them.
-__device__ __forceinline__ void onee_add(double *Out, int n, int r, int c, bool mirror, double v)
+// Every kernel below leaves the block of a shell-pair image of its own (blk:
+// those of one class, NA x NB elements an image); this sums the images of each
+// shell pair in their order into the raw matrix, one element per thread, so a
+// repeated call gives the same bits (images added by atomics did not, at the
+// same time).  For I = J an image with R != 0 stands for its mirror too.
+template <int LA, int LB>
+__global__ void __launch_bounds__(128) k_onee_gather(PlanDev pl, int sp0, int sp1, int b0, const double *__restrict__ blk,
+                                                     double *__restrict__ Out)
 {
-    atomicAdd(Out + (size_t)r * n + c, v);
-    if (mirror) atomicAdd(Out + (size_t)c * n + r, v);
+    constexpr int NB = ncart(LB), NAB = ncart(LA) * NB;
+    const long long t = blockIdx.x * 128LL + threadIdx.x;
+    const int sp = sp0 + (int)(t / NAB), e = (int)(t % NAB);
+    if (sp >= sp1) return;
+    const SpairRec rec = pl.spair[sp];
+    double sum = 0.0;
+    for (int q = 0; q < rec.nspi; ++q) {
+        const int img = pl.spi_order[rec.spi0 + q];
+        const double *v = blk + (size_t)(img - b0) * NAB;
+        sum += v[e];
+        if (rec.I == rec.J) {
+            const SpiRec &si = pl.spi[img];
+            if (si.n[0] || si.n[1] || si.n[2]) sum += v[(e % NB) * NB + e / NB];
+        }
+    }
+    const size_t n = pl.nbf, r = pl.shells[rec.I].ao + e / NB, c = pl.shells[rec.J].ao + e % NB;
+    Out[r * n + c] = sum;
+    if (rec.I != rec.J) Out[c * n + r] = sum;
 }
 
 // Kinetic energy: one warp per shell-pair image, one primitive pair per lane.
 template <int LA, int LB>
-__global__ void __launch_bounds__(128) k_onee_kinetic(PlanDev pl, int b0, int b1, const double2 *__restrict__ ab, double *__restrict__ Out)
+__global__ void __launch_bounds__(128) k_onee_kinetic(PlanDev pl, int b0, int b1, const double2 *__restrict__ ab, double *__restrict__ out)
 {
     constexpr int NA = ncart(LA), NB = ncart(LB);
     const int img = b0 + blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -91,12 +111,10 @@ __global__ void __launch_bounds__(128) k_onee_kinetic(PlanDev pl, int b0, int b1
         const PpiRec x = pl.ppi[si.pp0 + q];
         kinetic_block<LA, LB>(x, ab[si.pp0 + q].y, blk);
     }
-    const bool mirror = si.I != si.J || si.n[0] || si.n[1] || si.n[2];
-    const int aoI = pl.shells[si.I].ao, aoJ = pl.shells[si.J].ao;
 #pragma unroll
     for (int k = 0; k < NA * NB; ++k) {
         const double v = warp_sum(blk[k]);
-        if (lane == (k & 31)) onee_add(Out, pl.nbf, aoI + k / NB, aoJ + k % NB, mirror, v);
+        if (lane == (k & 31)) out[(size_t)(img - b0) * (NA * NB) + k] = v;
     }
 }
 
@@ -111,7 +129,7 @@ __global__ void __launch_bounds__(128) k_onee_kinetic(PlanDev pl, int b0, int b1
 template <int LA, int LB>
 __global__ void __launch_bounds__(128) k_onee_real(PlanDev pl, int b0, int b1, int natom, const double *__restrict__ Zc,
                                                    const double *__restrict__ xyz, const double *__restrict__ cand, int ncand, int gsz,
-                                                   double *__restrict__ Out)
+                                                   double *__restrict__ out)
 {
     constexpr int NA = ncart(LA), NB = ncart(LB), NAB = NA * NB, L = LA + LB, NT = L + 1, D = L + 1;
     constexpr int NK = (NAB + 7) / 8;
@@ -216,8 +234,6 @@ __global__ void __launch_bounds__(128) k_onee_real(PlanDev pl, int b0, int b1, i
                 }
         }
     }
-    const bool mirror = si.I != si.J || si.n[0] || si.n[1] || si.n[2];
-    const int aoI = pl.shells[si.I].ao, aoJ = pl.shells[si.J].ao;
 #pragma unroll
     for (int k = 0; k < NK; ++k) {
         // lane l of each group of eight holds element 8 k + l
@@ -225,7 +241,7 @@ __global__ void __launch_bounds__(128) k_onee_real(PlanDev pl, int b0, int b1, i
         v += __shfl_xor_sync(0xffffffffu, v, 8);
         v += __shfl_xor_sync(0xffffffffu, v, 16);
         const int o = 8 * k + lane;
-        if (lane < 8 && o < NAB) onee_add(Out, pl.nbf, aoI + o / NB, aoJ + o % NB, mirror, v);
+        if (lane < 8 && o < NAB) out[(size_t)(img - b0) * NAB + o] = v;
     }
 }
 
@@ -240,7 +256,7 @@ __global__ void __launch_bounds__(128) k_onee_real(PlanDev pl, int b0, int b1, i
 //   gtab[pidx * gcur + g] = (pi / p)^{3/2} e^{-G^2 / 4p}.
 template <int LA, int LB>
 __global__ void __launch_bounds__(128) k_onee_recip(PlanDev pl, int b0, int g0, int gcur, int nmax, const double2 *__restrict__ v,
-                                                    const double *__restrict__ gtab, double *__restrict__ Out)
+                                                    const double *__restrict__ gtab, double *__restrict__ out)
 {
     constexpr int NA = ncart(LA), NB = ncart(LB), NAB = NA * NB, L = LA + LB, NT = L + 1, D = L + 1, NH = nherm(L);
     extern __shared__ double2 ph[];  // [3][2 nmax + 1]
@@ -337,16 +353,14 @@ __global__ void __launch_bounds__(128) k_onee_recip(PlanDev pl, int b0, int g0, 
                 }
         }
     }
-    const bool mirror = si.I != si.J || si.n[0] || si.n[1] || si.n[2];
-    if (threadIdx.x < NAB)
-        onee_add(Out, pl.nbf, pl.shells[si.I].ao + threadIdx.x / NB, pl.shells[si.J].ao + threadIdx.x % NB, mirror, acc);
+    if (threadIdx.x < NAB) out[(size_t)(img - b0) * NAB + threadIdx.x] += acc;  // the real part is there already
 }
 
 // one launch per class of shell-pair images (op 0 kinetic, 1 real part, 2
-// reciprocal part of the attraction)
+// reciprocal part of the attraction, 3 the images into the raw matrix)
 struct OneeArgs {
     PlanDev pl;
-    int op;
+    int op = 0;
     const double2 *ab;
     int natom;
     const double *Z, *xyz, *cand;
@@ -354,32 +368,40 @@ struct OneeArgs {
     int g0, gcur, nmax;
     const double2 *v;
     const double *gtab;
-    double *Out;
+    double *blk;   // blocks of all images, class after class
+    double *Out;   // raw matrix
     cudaStream_t st;
 };
 template <int LA, int LB>
-static void onee_go(const OneeArgs &a, int b0, int b1)
+static size_t onee_go(const OneeArgs &a, int b0, int b1, int sp0, int sp1, size_t off)
 {
-    if (b1 <= b0) return;
+    constexpr int NAB = ncart(LA) * ncart(LB);
+    if (b1 <= b0) return off;
     const unsigned nb = (unsigned)(b1 - b0);
-    if (a.op == 0) k_onee_kinetic<LA, LB><<<(nb + 3) / 4, 128, 0, a.st>>>(a.pl, b0, b1, a.ab, a.Out);
+    double *blk = a.blk + off;
+    if (a.op == 0) k_onee_kinetic<LA, LB><<<(nb + 3) / 4, 128, 0, a.st>>>(a.pl, b0, b1, a.ab, blk);
     else if (a.op == 1)
-        k_onee_real<LA, LB><<<(nb + 3) / 4, 128, 0, a.st>>>(a.pl, b0, b1, a.natom, a.Z, a.xyz, a.cand, a.ncand, a.natom > 16 ? 32 : 8, a.Out);
+        k_onee_real<LA, LB><<<(nb + 3) / 4, 128, 0, a.st>>>(a.pl, b0, b1, a.natom, a.Z, a.xyz, a.cand, a.ncand, a.natom > 16 ? 32 : 8, blk);
+    else if (a.op == 2)
+        k_onee_recip<LA, LB><<<nb, 128, 3 * (2 * a.nmax + 1) * sizeof(double2), a.st>>>(a.pl, b0, a.g0, a.gcur, a.nmax, a.v, a.gtab, blk);
     else
-        k_onee_recip<LA, LB><<<nb, 128, 3 * (2 * a.nmax + 1) * sizeof(double2), a.st>>>(a.pl, b0, a.g0, a.gcur, a.nmax, a.v, a.gtab, a.Out);
+        k_onee_gather<LA, LB><<<(unsigned)(((long long)(sp1 - sp0) * NAB + 127) / 128), 128, 0, a.st>>>(a.pl, sp0, sp1, b0, blk, a.Out);
+    return off + (size_t)nb * NAB;
 }
 
-static void launch_onee(const std::vector<ClassRange> &cls, const OneeArgs &a)
+static void launch_onee(const Plan *P, OneeArgs a, int op)
 {
+    a.op = op;
+    size_t off = 0;
     for (int c = 0; c < JK_NCLASS_MAX; ++c) {
-        const int b0 = cls[c].b0, b1 = cls[c].b1;
+        const int b0 = P->classes[c].b0, b1 = P->classes[c].b1, s0 = P->spair_class_off[c], s1 = P->spair_class_off[c + 1];
         switch (c) {
-        case 0: onee_go<0, 0>(a, b0, b1); break;
-        case 1: onee_go<1, 0>(a, b0, b1); break;
-        case 2: onee_go<1, 1>(a, b0, b1); break;
-        case 3: onee_go<2, 0>(a, b0, b1); break;
-        case 4: onee_go<2, 1>(a, b0, b1); break;
-        case 5: onee_go<2, 2>(a, b0, b1); break;
+        case 0: off = onee_go<0, 0>(a, b0, b1, s0, s1, off); break;
+        case 1: off = onee_go<1, 0>(a, b0, b1, s0, s1, off); break;
+        case 2: off = onee_go<1, 1>(a, b0, b1, s0, s1, off); break;
+        case 3: off = onee_go<2, 0>(a, b0, b1, s0, s1, off); break;
+        case 4: off = onee_go<2, 1>(a, b0, b1, s0, s1, off); break;
+        case 5: off = onee_go<2, 2>(a, b0, b1, s0, s1, off); break;
         default: break;
         }
     }
@@ -431,19 +453,37 @@ int one_electron(Plan *P, int natom, const double *Z, const double *xyz, double 
     const PlanDev pl = P->dev();
     auto ok = [](cudaError_t e) { return e == cudaSuccess; };
     const int grid = (int)std::min<size_t>((n2 + 255) / 256, 152 * 16);
+    // blocks of the images, in the build's exchange scratch (rewritten by every
+    // build before it is read) where they take at most half of it
+    size_t nblk = 0;
+    for (const ClassRange &c : P->classes) nblk += (size_t)(c.b1 - c.b0) * ncart(c.la) * ncart(c.lb);
+    nblk += nblk & 1;
+    const size_t scratch = 2 * (size_t)w.gc * n2;
+    const bool inside = nblk <= scratch / 2;
+    OneeArgs a{};
+    a.pl = pl;
+    a.st = st;
+    a.blk = w.Z;
+    if (!inside && !ok(cudaMallocAsync((void **)&a.blk, nblk * sizeof(double), st))) return fail_cuda(JK_ERR_OOM, "one-electron scratch");
+    const auto release = [&] {
+        if (!inside) cudaFreeAsync(a.blk, st);
+    };
     if (T) {
-        if (!ok(cudaMemsetAsync(w.T1, 0, n2 * sizeof(double), st))) return fail_cuda(JK_ERR_CUDA, "memset failed");
-        OneeArgs a{};
-        a.pl = pl;
-        a.op = 0;
+        bool good = ok(cudaMemsetAsync(w.T1, 0, n2 * sizeof(double), st));
         a.ab = P->d_ppi_ab;
         a.Out = w.T1;
-        a.st = st;
-        launch_onee(P->classes, a);
+        launch_onee(P, a, 0);
+        launch_onee(P, a, 3);
         k_onee_final<<<grid, 256, 0, st>>>(n, P->d_compf, w.T1, P->d_S, 0.0, T);
-        if (!ok(cudaGetLastError())) return fail(JK_ERR_CUDA, "kinetic-energy kernels failed");
+        if (!ok(cudaGetLastError()) || !good) {
+            release();
+            return fail_cuda(JK_ERR_CUDA, "kinetic-energy kernels failed");
+        }
     }
-    if (!V || natom <= 0) return ok(cudaStreamSynchronize(st)) ? JK_OK : fail_cuda(JK_ERR_CUDA, "one-electron kernels failed");
+    if (!V || natom <= 0) {
+        release();
+        return ok(cudaStreamSynchronize(st)) ? JK_OK : fail_cuda(JK_ERR_CUDA, "one-electron kernels failed");
+    }
 
     // lattice candidates for the charges' images: |R| up to the largest
     // screening radius plus the cell's circumradius (the reduced X0 is at
@@ -496,57 +536,57 @@ int one_electron(Plan *P, int natom, const double *Z, const double *xyz, double 
     const int ng = (int)(P->gvec.size() / 4);
     const size_t oX = ((size_t)natom + 1) / 2 * 2, oC = oX + (3 * (size_t)natom + 1) / 2 * 2, oN = oC + 4 * (size_t)std::max(1, ncand);
     double *dZ = nullptr;
-    if (!ok(cudaMallocAsync((void **)&dZ, sizeof(double) * (oN + 2 * (size_t)std::max(1, ng)), st))) return fail_cuda(JK_ERR_OOM, "one-electron scratch");
+    if (!ok(cudaMallocAsync((void **)&dZ, sizeof(double) * (oN + 2 * (size_t)std::max(1, ng)), st))) {
+        release();
+        return fail_cuda(JK_ERR_OOM, "one-electron scratch");
+    }
     double *dX = dZ + oX, *dC = dZ + oC;
     double2 *dn = reinterpret_cast<double2 *>(dZ + oN);
     cudaMemcpyAsync(dZ, Z, sizeof(double) * natom, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(dX, xyz, sizeof(double) * 3 * natom, cudaMemcpyHostToDevice, st);
     if (ncand) cudaMemcpyAsync(dC, cv.data(), sizeof(double) * 4 * ncand, cudaMemcpyHostToDevice, st);
     bool good = ok(cudaMemsetAsync(w.T2, 0, n2 * sizeof(double), st));
-    OneeArgs a{};
-    a.pl = pl;
-    a.op = 1;
     a.natom = natom;
     a.Z = dZ;
     a.xyz = dX;
     a.cand = dC;
     a.ncand = ncand;
     a.Out = w.T2;
-    a.st = st;
-    launch_onee(P->classes, a);
+    launch_onee(P, a, 1);
     // reciprocal part.  The phase tables of k_onee_recip hold every integer
     // coordinate of G (nmax up to 64: 6 KB); a lattice that needs more takes
     // the structure-factor slab chunk by chunk, as the build does
     if (ng > 0 && P->g_nmax <= 64) {
-        // Gaussian factors of as many G as fit the build's exchange scratch
-        // (rewritten by every build before it is read)
-        const size_t cap = 2 * (size_t)w.gc * n2, np = std::max<size_t>(1, P->pvals.size());
+        // Gaussian factors of as many G as fit what is left of that scratch
+        const size_t used = inside ? nblk : 0, cap = scratch - used, np = std::max<size_t>(1, P->pvals.size());
         const int gch = (int)std::max<size_t>(1, std::min<size_t>((size_t)ng, cap / np));
         k_nuclear_sfac<<<(ng + 3) / 4, 128, 0, st>>>(natom, dZ, dX, P->d_gvec, 0, ng, 2, -1.0, dn);
-        a.op = 2;
         a.nmax = P->g_nmax;
         const bool fits = cap >= np;
-        a.gtab = fits ? w.Z : w.gtab;  // w.gtab holds at least one G
+        a.gtab = fits ? w.Z + used : w.gtab;  // w.gtab holds at least one G
         for (int g0 = 0; g0 < ng; g0 += a.gcur) {
             a.g0 = g0;
             a.gcur = std::min(fits ? gch : w.gc, ng - g0);
             a.v = dn + g0;
             launch_gauss_table(P, g0, a.gcur, const_cast<double *>(a.gtab), st);
-            launch_onee(P->classes, a);
+            launch_onee(P, a, 2);
         }
+        launch_onee(P, a, 3);
     } else {
+        launch_onee(P, a, 3);
         for (int g0 = 0; g0 < ng; g0 += w.gc) {
             const int gcur = std::min(w.gc, ng - g0);
             launch_gauss_table(P, g0, gcur, w.gtab, st);
             for (int c = 0; c < JK_NCLASS_MAX; ++c)
                 launch_sfac(c, pl, P->spair_class_off[c], P->spair_class_off[c + 1], P->d_gvec, g0, gcur, w.gtab, w.M, st);
             k_nuclear_sfac<<<(gcur + 3) / 4, 128, 0, st>>>(natom, dZ, dX, P->d_gvec, g0, gcur, 1, 1.0, dn);
-            slab_gemv_n(w.M, (long long)n2, 2 * gcur, reinterpret_cast<const double *>(dn), -1.0, w.T2, st);
+            slab_gemv_n(w.M, (long long)n2, 2 * gcur, reinterpret_cast<const double *>(dn), -1.0, w.T2, st, false);
         }
     }
     // self term +(pi/(V w^2)) Z_tot S and the component factors
     k_onee_final<<<grid, 256, 0, st>>>(n, P->d_compf, w.T2, P->d_S, kPi / (P->volume * w2) * ztot, V);
     cudaFreeAsync(dZ, st);
+    release();
     // waited for on every path: the copies above read the caller's host arrays
     good = ok(cudaGetLastError()) && good;
     good = ok(cudaStreamSynchronize(st)) && good;
