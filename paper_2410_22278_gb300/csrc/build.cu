@@ -530,10 +530,14 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
             a.dmaxf = w.dmaxf;
             a.X = w.X;
             a.Y = K ? w.Y : nullptr;
-            const int lane = P->nside > 0 ? turn++ % P->nside : 0;
+            // the next lane whose list holds the class pair (FP64 plans have no lists)
+            const int nlane = mixed ? w.nlist : std::max(1, P->nside);
+            int lane = turn++ % nlane;
+            if (mixed)
+                while (lane > 0 && w.list_cap[lane] < std::min<long long>(w.list_cap[0], P->class_quartets(cb, ck))) lane = (lane + 1) % nlane;
             cudaStream_t ls = lane ? P->side[lane - 1] : st;
             tm.use(ls);
-            int2 *big = w.big ? w.big + (size_t)lane * w.cap : nullptr;
+            const QuartetList big{w.big ? (char *)w.big + w.list_off[lane] : nullptr, w.list_elt == 4};
             unsigned *nbig = w.nbig ? w.nbig + 2 * lane : nullptr;
             a.st = ls;
             a.DhD = w.DhD;
@@ -563,7 +567,7 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
                 a.big = big;
                 a.nbig = nbig;
                 a.ovf = nbig + 1;
-                a.cap = w.cap;
+                a.cap = w.list_cap[lane];
                 const int et = tm.start(10);
                 launch_jeng(cb, ck, a);
                 tm.stop(10, et, 1);
@@ -591,7 +595,7 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
                 a.big = big;
                 a.nbig = nbig;
                 a.ovf = nbig + 1;
-                a.cap = w.cap;
+                a.cap = w.list_cap[lane];
                 const int et = tm.start(10);
                 launch_real(cb, ck, a);
                 tm.stop(10, et, 1);
@@ -792,7 +796,7 @@ int set_schedule(Plan *P, const int *sched, int n)
 int build_counts(Plan *P, long long *counts, int n)
 {
     unsigned long long h[kCounters] = {};
-    unsigned hb[2 * (1 + Plan::kSide)] = {};
+    unsigned hb[2 * Workspace::kLists] = {};
     if (P->timer.next > 0 && cudaEventSynchronize(P->timer.pool[P->timer.next - 1]) != cudaSuccess)
         return fail_cuda(JK_ERR_CUDA, "build did not finish");
     if (cudaMemcpy(h, P->ws.cnt, sizeof h, cudaMemcpyDeviceToHost) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "count copy failed");

@@ -21,6 +21,10 @@ struct LowRankWs {
 // rho[b] = sum_i M[b][i] x[i] for b < m2 (M is [m2][n2]); part holds
 // m2 * kSlabSplitsMax partial sums.
 constexpr int kSlabSplitsMax = 1024;
+// Doubles that `part` of the passes below needs for up to m2 slabs: a pass over
+// m of them takes at most max(1, ceil(kSlabBlocks / m)) splits of each.
+constexpr int kSlabBlocks = 152 * 8;
+constexpr long long slab_part_size(int m2) { return (long long)m2 + kSlabBlocks; }
 void slab_gemv_t(const double *M, long long n2, int m2, const double *x, double *part, double *rho, cudaStream_t st);
 // y[i] += alpha sum_b M[b][i] rho[b]; split: the slabs may be split over blocks
 // that add by atomics (in any order).

@@ -88,6 +88,26 @@ struct SpairRec {    // unique shell pair (I, J) with its images [spi0, spi0 + n
     int I, J, spi0, nspi;
 };
 
+// List of image quartets (bra image, ket image): two 32-bit indices an entry,
+// or two 16-bit ones in a plan of at most 65536 images.
+struct QuartetList {
+    void *p;
+    int narrow;
+#ifdef __CUDACC__
+    __device__ __forceinline__ void put(unsigned e, int bra, int ket) const
+    {
+        if (narrow) reinterpret_cast<unsigned *>(p)[e] = (unsigned)bra << 16 | (unsigned)ket;
+        else reinterpret_cast<int2 *>(p)[e] = make_int2(bra, ket);
+    }
+    __device__ __forceinline__ int2 get(unsigned e) const
+    {
+        if (!narrow) return reinterpret_cast<const int2 *>(p)[e];
+        const unsigned v = reinterpret_cast<const unsigned *>(p)[e];
+        return make_int2((int)(v >> 16), (int)(v & 0xffffu));
+    }
+#endif
+};
+
 struct PlanDev {
     int nbf, nshell;
     int nspi, nppi, nspair;

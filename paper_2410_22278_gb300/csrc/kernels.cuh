@@ -432,7 +432,7 @@ template <int LA, int LB, int LC, int LD, typename T>
 __global__ void __launch_bounds__(kRealThreads) k_real(PlanDev pl, int b0, int b1, int k0, int k1, int same, int kchunk, int mode,
                                                         double tau, const T *__restrict__ Dp, const T *__restrict__ dmax,
                                                         double *__restrict__ X, double *__restrict__ Y,
-                                                        unsigned long long *__restrict__ cnt, int2 *__restrict__ big,
+                                                        unsigned long long *__restrict__ cnt, QuartetList big,
                                                         unsigned *__restrict__ nbig, unsigned cap, unsigned *__restrict__ ovf)
 {
     constexpr int NA = ncart(LA), NB = ncart(LB), NC = ncart(LC), ND = ncart(LD);
@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(kRealThreads) k_real(PlanDev pl, int b0, int b
             if (est >= tauf || ipq > 0.7225f * (ipq + pl.inv_omega2f)) {
                 const unsigned slot = atomicAdd(nbig, 1u);
                 if (slot < cap) {
-                    big[slot] = make_int2(bra, kt);
+                    big.put(slot, bra, kt);
                     valid = false;
                 } else {
                     atomicAdd(ovf, 1u);

@@ -30,7 +30,7 @@ struct RealLaunch {
     const float *Dpf, *dmaxf;     // FP32 kernels
     double *X, *Y;
     unsigned long long *cnt;
-    int2 *big;           // compact list of large quartets (mixed precision)
+    QuartetList big;     // compact list of large quartets (mixed precision)
     unsigned *nbig, *ovf;
     unsigned cap;
     bool list_pass;      // launch the FP64 list kernel instead of the tile kernel

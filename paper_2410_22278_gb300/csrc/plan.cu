@@ -413,6 +413,42 @@ static int upload(const std::vector<T> &h, T **d, size_t &bytes)
     return JK_OK;
 }
 
+// Lists of large quartets of a mixed plan.  The FP64 share is a small fraction:
+// a list holds up to 2% of all image quartets of the plan (at least 1 Mi, at
+// most 64 Mi), and never more than its class pair has.  A class pair's list is
+// in use from its tile kernel to its list pass, so each lane of the real-space
+// phase needs one; the l-th lane's holds the l-th largest class pair, and a
+// class pair only goes to a lane that can hold it (run_build).  As many lanes as
+// fit the bytes that one list of 8-byte entries and partial sums for the
+// largest split of every slab took: a plan with side streams asks for no more
+// than one without (a server admits plans by their workspace).
+static void quartet_lists(Plan *P, size_t &bytes)
+{
+    Workspace &w = P->ws;
+    const long long cap = std::min<long long>(std::max<long long>(P->n_quartets / 50, 1 << 20), 64ll << 20);
+    std::vector<long long> need;
+    for (int i = 0; i < JK_NCLASS_MAX; ++i)
+        for (int j = i; j < JK_NCLASS_MAX; ++j) need.push_back(std::min(cap, P->class_quartets(i, j)));
+    std::sort(need.rbegin(), need.rend());
+    const bool narrow = P->spi.size() <= 65536;
+    w.list_elt = narrow ? sizeof(unsigned) : sizeof(int2);
+    const long long slab = 2LL * w.gc * kSlabSplitsMax - slab_part_size(2 * w.gc) - 8;  // doubles
+    const long long fit = cap * (long long)sizeof(int2) + slab * (long long)sizeof(double);
+    static_assert(Workspace::kLists >= Plan::kSide, "a list per lane");
+    w.nlist = std::max(1, P->nside);
+    const auto total = [&] { return std::accumulate(need.begin(), need.begin() + w.nlist, 0LL) * (long long)w.list_elt; };
+    while (w.nlist > 1 && total() > fit) --w.nlist;
+    // what is left of those bytes lets the largest class pairs into more lanes
+    for (int l = 1; l < w.nlist; ++l) need[l] += std::min(need[0] - need[l], std::max(0LL, fit - total()) / (long long)w.list_elt);
+    bytes = 0;
+    for (int l = 0; l < w.nlist; ++l) {
+        w.list_cap[l] = (unsigned)need[l];
+        w.list_off[l] = bytes;
+        bytes += (size_t)need[l] * w.list_elt;
+    }
+    bytes = std::max<size_t>(bytes, 8);
+}
+
 static int alloc_ws(Plan *P)
 {
     Workspace &w = P->ws;
@@ -459,7 +495,7 @@ static int alloc_ws(Plan *P)
         return true;
     };
     bool ok = al(&w.gtab, std::max<size_t>(1, P->pvals.size()) * (size_t)gc) && al(&w.Dp, n2) && al(&w.X, n2) && al(&w.Y, n2) && al(&w.JLR, n2) && al(&w.KLR, n2) && al(&w.T1, n2) &&
-              al(&w.T2, n2) && al(&w.M, 2 * (size_t)gc * n2) && al(&w.Z, 2 * (size_t)gc * n2) && al(&w.rho, 2 * (size_t)gc) && al(&w.rho_part, 2 * (size_t)gc * kSlabSplitsMax) &&
+              al(&w.T2, n2) && al(&w.M, 2 * (size_t)gc * n2) && al(&w.Z, 2 * (size_t)gc * n2) && al(&w.rho, 2 * (size_t)gc) && al(&w.rho_part, slab_part_size(2 * (int)gc)) &&
               al(&w.dmax, (size_t)P->nshell * P->nshell) && al(&w.scal, 16) && (!mixed || al((double **)&w.Dpf, (n2 + 1) / 2)) &&
               (!mixed || al((double **)&w.dmaxf, ((size_t)P->nshell * P->nshell + 2) / 2));
     {
@@ -509,13 +545,11 @@ static int alloc_ws(Plan *P)
     if (cudaMalloc((void **)&w.err, sizeof(unsigned)) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed");
     if (cudaMalloc((void **)&w.cnt, kCounters * sizeof(unsigned long long)) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed");
     if (P->precision == JK_MIXED) {
-        // the FP64 share is a small fraction; the list holds up to 2% of all image quartets (at most 64 Mi entries)
-        const long long want = std::min<long long>(std::max<long long>(P->n_quartets / 50, 1 << 20), 64ll << 20);
-        w.cap = (unsigned)want;
-        w.nlist = std::max(1, P->nside);  // the caller's stream and all but the last side stream
-        if (cudaMalloc((void **)&w.big, sizeof(int2) * w.cap * w.nlist) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed for quartet list");
+        size_t lb = 0;
+        quartet_lists(P, lb);
+        if (cudaMalloc((void **)&w.big, lb) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed for quartet list");
         if (cudaMalloc((void **)&w.nbig, 2 * sizeof(unsigned) * w.nlist) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed");
-        bytes += (sizeof(int2) * w.cap + 2 * sizeof(unsigned)) * w.nlist;
+        bytes += lb + 2 * sizeof(unsigned) * w.nlist;
     }
     cudaMemset(w.err, 0, sizeof(unsigned));
     w.bytes = bytes + sizeof(unsigned) + kCounters * sizeof(unsigned long long);

@@ -44,7 +44,7 @@ struct Workspace {
     double *M = nullptr;      // structure-factor chunk [2*gc][n][n]
     double *Z = nullptr;      // D * M chunk, stacked
     double *rho = nullptr;    // [2*gc] density structure factors
-    double *rho_part = nullptr;  // [2*gc][kSlabSplitsMax] their partial sums
+    double *rho_part = nullptr;  // [slab_part_size(2*gc)] their partial sums
     double *dmax = nullptr;   // [nshell*nshell] max |D'| per shell block
     float *Dpf = nullptr;     // single-precision copies for the FP32 kernels (mixed precision)
     float *dmaxf = nullptr;   // [nshell*nshell + 1] of dmax, then its largest value
@@ -56,10 +56,14 @@ struct Workspace {
     float *DhF = nullptr;
     unsigned *err = nullptr;  // device check word
     unsigned long long *cnt = nullptr;  // kCounters build counters (see above)
-    int2 *big = nullptr;                // compact list of quartets sent to FP64 (mixed precision)
-    unsigned *nbig = nullptr;           // [0] list length, [1] overflow count (accumulated over a build)
-    unsigned cap = 0;
-    int nlist = 1;                      // lists (big: nlist * cap entries, nbig: nlist pairs), one per lane of the real-space phase
+    // quartets sent to FP64 (mixed precision): one list per lane of the
+    // real-space phase, list_cap[l] entries of list_elt bytes from list_off[l] on
+    static constexpr int kLists = 4;
+    void *big = nullptr;
+    unsigned *nbig = nullptr;           // per list: [0] length, [1] overflow count (accumulated over a build)
+    int nlist = 0;                      // 0: FP64 plans
+    size_t list_elt = 8, list_off[kLists] = {};
+    unsigned list_cap[kLists] = {};
     int gc = 0;               // G vectors per chunk
     double *gtab = nullptr;   // [distinct p][gc]: (pi/p)^{3/2} e^{-G^2/4p} of the current G chunk
     float2 *gtab2 = nullptr;  // the same as double-floats (mixed-precision structure factors)
@@ -207,6 +211,12 @@ struct Plan {
     std::vector<EnergySlot> energy_free;  // not in use by a call
     std::vector<EnergySlot> energy_lost;  // left by a failed call
     PlanDev dev() const;
+    // unique image quartets of a pair of classes
+    long long class_quartets(int cb, int ck) const
+    {
+        const long long nb = classes[cb].b1 - classes[cb].b0, nk = classes[ck].b1 - classes[ck].b0;
+        return cb == ck ? nb * (nb + 1) / 2 : nb * nk;
+    }
 };
 
 int build_plan(const jk_cell *cell, const jk_shell *shells, int nshell, double omega, const jk_cutoffs *cut,

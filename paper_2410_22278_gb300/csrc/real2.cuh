@@ -448,7 +448,7 @@ __device__ __forceinline__ bool pair_reaches(const PlanDev &pl, const float4 &bq
 // Mixed precision: true if the image quartet (bra, kt) goes to the FP64 list,
 // decided as in k_real; called for the few that may (pair_reaches).
 template <typename T>
-__device__ __noinline__ bool list_quartet(const PlanDev &pl, int bra, int kt, float tauf, const T *__restrict__ dmax, int2 *__restrict__ big,
+__device__ __noinline__ bool list_quartet(const PlanDev &pl, int bra, int kt, float tauf, const T *__restrict__ dmax, QuartetList big,
                                           unsigned *__restrict__ nbig, unsigned cap, unsigned *__restrict__ ovf)
 {
     const SpiRec sb = pl.spi[bra], sk = pl.spi[kt];
@@ -458,7 +458,7 @@ __device__ __noinline__ bool list_quartet(const PlanDev &pl, int bra, int kt, fl
     if (!(est >= tauf || ipq > 0.7225f * (ipq + pl.inv_omega2f))) return false;
     const unsigned slot = atomicAdd(nbig, 1u);
     if (slot < cap) {
-        big[slot] = make_int2(bra, kt);
+        big.put(slot, bra, kt);
         return true;
     }
     atomicAdd(ovf, 1u);
@@ -788,7 +788,7 @@ template <int LA, int LB, int LC, int LD, typename T>
 __global__ void __launch_bounds__(32 * kWarpsPerBlock, tile_blocks<T>(LA + LB + LC + LD)) k_real_w(PlanDev pl, TileMap map, int k0, int k1, int same, int mode, double tau,
                                                                 const T *__restrict__ Dp, const T *__restrict__ dmax,
                                                                 double *__restrict__ X, double *__restrict__ Y,
-                                                                unsigned long long *__restrict__ cnt, int2 *__restrict__ big,
+                                                                unsigned long long *__restrict__ cnt, QuartetList big,
                                                                 unsigned *__restrict__ nbig, unsigned cap, unsigned *__restrict__ ovf)
 {
     constexpr int NA = ncart(LA), NB = ncart(LB), NC = ncart(LC), ND = ncart(LD), NV = NA * NB * NC * ND;
@@ -1026,7 +1026,7 @@ template <int LA, int LB, int LC, int LD, typename T>
 __global__ void __launch_bounds__(kRealThreads) k_real_q(PlanDev pl, int b0, int b1, int k0, int k1, int same, int kchunk, int mode,
                                                           double tau, const T *__restrict__ Dp, const T *__restrict__ dmax,
                                                           double *__restrict__ X, double *__restrict__ Y,
-                                                          unsigned long long *__restrict__ cnt, int2 *__restrict__ big,
+                                                          unsigned long long *__restrict__ cnt, QuartetList big,
                                                           unsigned *__restrict__ nbig, unsigned cap, unsigned *__restrict__ ovf)
 {
     constexpr int NA = ncart(LA), NB = ncart(LB), NC = ncart(LC), ND = ncart(LD), NV = NA * NB * NC * ND;
@@ -1180,7 +1180,7 @@ __global__ void __launch_bounds__(kRealThreads) k_real_q(PlanDev pl, int b0, int
             if (est >= tauf || ipq > 0.7225f * (ipq + pl.inv_omega2f)) {
                 const unsigned slot = atomicAdd(nbig, 1u);
                 if (slot < cap) {
-                    big[slot] = make_int2(bra, kt);
+                    big.put(slot, bra, kt);
                     valid = false;
                 } else {
                     atomicAdd(ovf, 1u);
@@ -1232,7 +1232,7 @@ __global__ void __launch_bounds__(kRealThreads) k_real_q(PlanDev pl, int b0, int
 // (ss|pp) of the 64-water box: two batches) and one lane digested alone.
 // Counters as k_real_w (cnt points at the FP64 slots).
 template <int LA, int LB, int LC, int LD>
-__global__ void __launch_bounds__(32 * kWarpsPerBlock, LA + LB + LC + LD <= 3 ? 3 : 2) k_real_list_w(PlanDev pl, const int2 *__restrict__ big,
+__global__ void __launch_bounds__(32 * kWarpsPerBlock, LA + LB + LC + LD <= 3 ? 3 : 2) k_real_list_w(PlanDev pl, QuartetList big,
                                                                         const unsigned *__restrict__ nbig, unsigned cap, int same,
                                                                         const double *__restrict__ Dp, double *__restrict__ X,
                                                                         double *__restrict__ Y, unsigned long long *__restrict__ cnt)
@@ -1260,7 +1260,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, LA + LB + LC + LD <= 3 ? 
         const int cnt_e = (int)min(per, total - base);
         int nk = 1, nterm = 0;
         if (lane < cnt_e) {
-            const int2 pr = big[base + lane];
+            const int2 pr = big.get(base + lane);
             const int b0 = __float_as_int(__ldg(&pl.spr[pr.x].w)), k0 = __float_as_int(__ldg(&pl.spr[pr.y].w));
             nk = __float_as_int(__ldg(&pl.spr[pr.y + 1].w)) - k0;
             nterm = (__float_as_int(__ldg(&pl.spr[pr.x + 1].w)) - b0) * nk;
@@ -1313,7 +1313,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, LA + LB + LC + LD <= 3 ? 
         }
         __syncwarp();
         if (lane < cnt_e) {
-            const int2 pr = big[base + lane];
+            const int2 pr = big.get(base + lane);
             const int4 b4 = __ldg(pl.spd + pr.x), k4 = __ldg(pl.spd + pr.y);
             double V[NV], Dij[NA * NB];
             Acc<double> jb[NA * NB];

@@ -372,7 +372,7 @@ __device__ __forceinline__ void coop_counts(const Tally &tl, unsigned nq, unsign
 template <int LA, int LB, int LC, int LD, typename T>
 __global__ void __launch_bounds__(32) k_real_c(PlanDev pl, TileMap map, int k0, int k1, int same, int mode, double tau,
                                                const T *__restrict__ Dp, const T *__restrict__ dmax, double *__restrict__ X,
-                                               double *__restrict__ Y, unsigned long long *__restrict__ cnt, int2 *__restrict__ big,
+                                               double *__restrict__ Y, unsigned long long *__restrict__ cnt, QuartetList big,
                                                unsigned *__restrict__ nbig, unsigned cap, unsigned *__restrict__ ovf)
 {
     constexpr int L = LA + LB + LC + LD;
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(32) k_real_c(PlanDev pl, TileMap map, int k0, 
 
 // FP64 pass over the listed large quartets: one warp per list entry.
 template <int LA, int LB, int LC, int LD>
-__global__ void __launch_bounds__(32) k_real_list_c(PlanDev pl, const int2 *__restrict__ big, const unsigned *__restrict__ nbig,
+__global__ void __launch_bounds__(32) k_real_list_c(PlanDev pl, QuartetList big, const unsigned *__restrict__ nbig,
                                                     unsigned cap, int same, const double *__restrict__ Dp, double *__restrict__ X,
                                                     double *__restrict__ Y, unsigned long long *__restrict__ cnt)
 {
@@ -431,7 +431,7 @@ __global__ void __launch_bounds__(32) k_real_list_c(PlanDev pl, const int2 *__re
     unsigned nq = 0;
     coop_init(s);
     for (unsigned q = blockIdx.x; q < total; q += gridDim.x) {
-        const int2 pr = big[q];
+        const int2 pr = big.get(q);
         const SpiRec sb = pl.spi[pr.x], sk = pl.spi[pr.y];
         ++nq;
         tl.quart += (threadIdx.x & 31) == 0;
