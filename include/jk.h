@@ -208,17 +208,22 @@ int jk_energy_noalloc(const jk_plan *plan, const double *D, const double *J, con
                       double *e_exch, void *cuda_stream);
 
 /* Device time of each phase of the most recent jk_build on this plan, in
- * milliseconds, from CUDA events recorded on the build's stream around the
- * phase's kernels (waits for that build to finish).  ms[0] prologue (D scaling, zeroing, density slices and
- * factorisation), ms[1] real space (fork to the last list pass), ms[2]
- * reciprocal structure factors, ms[3] reciprocal Coulomb contraction, ms[4]
- * reciprocal exchange contraction, ms[5] background and assembly, ms[6]
- * whole build, ms[7] the tensor-core GEMM launches inside ms[4] (mixed
- * precision), ms[8] their operand slicing, ms[9] the FP64 list passes inside
- * ms[1] (mixed precision), ms[10] the FP32 (mixed) or FP64 tile kernels
- * inside ms[1], ms[11] (not a time) the BF16 MMA flops the GEMMs issued;
- * launches[i] the kernel launches per phase.  n = number of slots the
- * caller provides (<= 12 used). */
+ * milliseconds, from CUDA events recorded around the phase's kernels on the
+ * streams they run on (waits for that build to finish).  ms[0] prologue (D
+ * scaling, zeroing, density slices and factorisation), ms[1] real space (fork
+ * to the last list pass), ms[2] reciprocal structure factors, ms[3] reciprocal
+ * Coulomb contraction, ms[4] reciprocal exchange contraction, ms[5] background
+ * and assembly, ms[6] whole build, ms[7] the tensor-core GEMM launches inside
+ * ms[4] (mixed precision), ms[8] their operand slicing, ms[9] the FP64 list
+ * passes inside ms[1] (mixed precision), ms[10] the FP32 (mixed) or FP64 tile
+ * kernels inside ms[1], ms[11] (not a time) the BF16 MMA flops the GEMMs
+ * issued; launches[i] the kernel launches per phase.
+ * Plans of at most 2e8 image quartets deal their class pairs out over several
+ * streams and run the reciprocal phase beside them: there ms[9] and ms[10] are
+ * the times during which at least one of their kernels was running, ms[2] to
+ * ms[4] overlap ms[1], and so the phases can add up to more than ms[6] (none is
+ * longer than it by itself).
+ * n = number of slots the caller provides (<= 12 used). */
 int jk_build_times(jk_plan *plan, double *ms, int *launches, int n);
 
 /* Autotuner (no counterpart in the paper): choose the tile shape of every

@@ -327,7 +327,7 @@ void PhaseTimer::destroy()
 
 // Reciprocal (erf) part of the build on stream st: structure factors (or
 // the cache), the Coulomb slab passes and the exchange contraction, chunk
-// by chunk of G.  Enqueued on its own stream, concurrent with real space.
+// by chunk of G.  Small plans enqueue it on a side stream, beside real space.
 static int reciprocal_phase(Plan *P, double *J, double *K, cudaStream_t st)
 {
     const int n = P->nbf;
@@ -493,9 +493,9 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
         cudaEventRecord(P->side_fork, st);
         for (int i = 0; i < P->nside; ++i) cudaStreamWaitEvent(P->side[i], P->side_fork, 0);
     }
-    const auto join = [&] {
+    const auto join = [&](int i0, int i1) {
         tm.use(st);
-        for (int i = 0; i < P->nside; ++i) {
+        for (int i = i0; i < i1; ++i) {
             cudaEventRecord(P->side_join[i], P->side[i]);
             cudaStreamWaitEvent(st, P->side_join[i], 0);
         }
@@ -503,7 +503,7 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
     if (P->nside > 0) {
         tm.use(P->side[P->nside - 1]);
         if ((rc = reciprocal_phase(P, J, K, P->side[P->nside - 1]))) {
-            join();
+            join(0, P->nside);
             return rc;
         }
         tm.use(st);
@@ -608,11 +608,11 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
                 nreal += 2;
             }
             if ((rc = cuda_check("real-space kernel"))) {
-                join();
+                join(0, P->nside);
                 return rc;
             }
         }
-    join();
+    join(0, P->nside - 1);
     if (jeng) {
         // Hermite J of every primitive pair back to Cartesian, into X
         for (int c = kJengClass; c < JK_NCLASS_MAX; ++c)
@@ -622,7 +622,8 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
     tm.stop(1, ev, nreal);
 
     // ---- reciprocal space
-    if (P->nside == 0 && (rc = reciprocal_phase(P, J, K, st))) return rc;
+    if (P->nside > 0) join(P->nside - 1, P->nside);
+    else if ((rc = reciprocal_phase(P, J, K, st))) return rc;
 
     ev = tm.start(5);
 
@@ -826,10 +827,23 @@ int build_times(Plan *P, double *ms, int *launches, int n)
     }
     if (tm.marks.empty()) return JK_OK;
     if (cudaEventSynchronize(tm.pool[tm.next - 1]) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "build did not finish");
+    // a phase's intervals add up, unless they lie on several streams: then the
+    // time during which at least one of them ran (from the build's first event)
+    std::vector<std::pair<float, float>> iv[PhaseTimer::kPhases];
     for (auto &m : tm.marks) {
-        float t = 0;
+        float t0 = 0, t = 0;
         cudaEventElapsedTime(&t, tm.pool[m.second.first], tm.pool[m.second.second]);
-        if (m.first < n && ms) ms[m.first] += t;
+        if (P->nside > 0) cudaEventElapsedTime(&t0, tm.pool[0], tm.pool[m.second.first]);
+        if (P->nside > 0) iv[m.first].push_back({t0, t0 + t});
+        else if (m.first < n && ms) ms[m.first] += t;
+    }
+    for (int p = 0; p < PhaseTimer::kPhases && p < n && ms; ++p) {
+        std::sort(iv[p].begin(), iv[p].end());
+        float end = -1.0f;
+        for (auto &x : iv[p]) {
+            ms[p] += std::max(0.0f, x.second - std::max(x.first, end));
+            end = std::max(end, x.second);
+        }
     }
     for (int i = 0; i < n && i < PhaseTimer::kPhases; ++i)
         if (launches) launches[i] = tm.launches[i];
