@@ -228,14 +228,15 @@ int jk_build_times(jk_plan *plan, double *ms, int *launches, int n);
 
 /* Autotuner (no counterpart in the paper): choose the tile shape of every
  * real-space class-pair kernel -- for class pairs of s and p shells the
- * family (0 lane-per-bra, 8 .. 128 kets per tile; 1 warp-per-bra, 128 ..
- * 2048 kets per warp on average; 2 pair queue, 32 .. 512 kets per tile),
- * for class pairs with a d shell, which have one kernel (family 0, a bra or
- * a quartet per warp), 1 .. 2048 kets per warp -- by timing the candidates on two sub-ranges of bras with CUDA
- * events, on
- * `cuda_stream`, using density D (device, as in jk_build) for realistic
- * work.  If cache_path is not NULL, choices are read from and written to
- * that text file, keyed by GPU name, precision, class pair and size
+ * family (0 lane-per-bra, 8 .. 128 kets per tile; 1 warp-per-bra, 8 .. 2048
+ * kets per warp on average, 1 .. 256 for (pp|pp), whose warps take one image
+ * quartet each; 2 pair queue, 32 .. 512 kets per tile), for class pairs with a
+ * d shell, which have one kernel (family 0, a bra or a quartet per warp), 1 ..
+ * 2048 kets per warp -- by timing the candidates and the plan's untuned
+ * schedule with CUDA events on `cuda_stream`, using density D (device, as in
+ * jk_build) for realistic work.  The untuned schedule stays unless a candidate
+ * is faster by 2%.  If cache_path is not NULL, choices are read from and
+ * written to that text file, keyed by GPU name, precision, class pair and size
  * bucket.  chosen (may be NULL) receives 42 ints: (family, kets) for each
  * of the 21 class pairs (bra class <= ket class, classes ss, ps, pp, ds,
  * dp, dd).  Overwrites the
@@ -245,7 +246,8 @@ int jk_autotune(jk_plan *plan, const double *D, void *cuda_stream, const char *c
 /* Set the real-space schedule directly (what jk_autotune chooses): sched
  * holds (family, kets) for the first n class pairs in jk_autotune's order;
  * families 1 and 2 only for class pairs of s and p shells, kets in
- * 1..65535.  Results do not depend on the schedule beyond rounding.
+ * 1..65535: kets per tile in families 0 and 2 of the s and p class pairs, else
+ * the mean number of kets per warp.  Results do not depend on the schedule beyond rounding.
  * Errors: JK_ERR_INVALID (nothing is changed). */
 int jk_plan_set_schedule(jk_plan *plan, const int *sched, int n);
 

@@ -244,12 +244,13 @@ static void launch_hermite(int cls, bool back, const PlanDev &pl, int b0, int b1
 }
 
 // The warps of a warp-per-bra launch over the bras [b0, b1) and kets [k0, k1)
-// (TileMap).  kchunk is the mean number of kets of a warp: a warp gets the
-// work of kchunk kets of the mean primitive count with a bra of the mean one.
+// (TileMap) of the bra class B.  kchunk is the mean number of kets of a warp: a
+// warp gets the work of kchunk kets of the mean primitive count with a bra of
+// the class's mean one (also where only a part of its bras is launched).
 // Images are in descending order of primitive count inside a class, so a
 // range of bras of similar count is contiguous; a new range starts where the
 // count has fallen by a quarter.
-static TileMap tile_map(const Plan *P, int b0, int b1, int k0, int k1, int kchunk)
+static TileMap tile_map(const Plan *P, const ClassRange &B, int b0, int b1, int k0, int k1, int kchunk)
 {
     TileMap m{};
     if (b1 <= b0 || k1 <= k0) return m;
@@ -257,7 +258,7 @@ static TileMap tile_map(const Plan *P, int b0, int b1, int k0, int k1, int kchun
         return (double)(P->spi[i1 - 1].pp0 + P->spi[i1 - 1].npp - P->spi[i0].pp0);
     };
     const double pk = prims(k0, k1);
-    double work = (double)kchunk * (prims(b0, b1) / (b1 - b0)) * (pk / (k1 - k0));
+    double work = (double)kchunk * (prims(B.b0, B.b1) / (B.b1 - B.b0)) * (pk / (k1 - k0));
     // at most 2^28 warps (blockIdx.x); only a hand-set schedule gets there
     work = std::max(work, prims(b0, b1) * pk / (double)(1 << 28));
     for (int b = b0; b < b1;) {
@@ -521,7 +522,7 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
             a.k1 = Kc.b1;
             a.same = cb == ck;
             a.kchunk = P->kchunk[cb][ck];
-            a.map = tile_map(P, a.b0, a.b1, a.k0, a.k1, a.kchunk);
+            a.map = tile_map(P, B, a.b0, a.b1, a.k0, a.k1, a.kchunk);
             a.variant = P->kvariant[cb][ck];
             a.tau = P->mixed_tau;
             a.Dp = w.Dp;
@@ -641,11 +642,15 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
     return cuda_check("epilogue");
 }
 
-// Autotuner: for every class pair with work, time the real-space tile
-// kernel of the plan's precision over a sub-range of at most 4096 bras
-// against all kets, for ket-chunk sizes {8, 16, 32, 64, 128}, and keep the
-// fastest.  Results are cached in a text file (one line per GPU name,
-// precision, class pair and size bucket) when cache_path is given.
+// Autotuner: for every class pair with work, time the real-space tile kernel of
+// the plan's precision with each candidate over two sub-ranges of at most 2048
+// bras against all kets, and the two fastest, with the plan's untuned schedule,
+// over the whole class where that takes less than about a second.  A candidate
+// replaces the untuned schedule only if it is faster by 2%: the sub-ranges alone
+// preferred few kets per warp, and the 64-water tiles so tuned took 389 ms
+// against 350 untuned.  Results are cached in a text file (one line per GPU
+// name, precision, class pair and size bucket: family * 65536 + kets, or 0
+// where the untuned schedule stays) when cache_path is given.
 int autotune(Plan *P, const double *D, cudaStream_t st, const char *cache_path, int *chosen)
 {
     if (cudaSetDevice(P->device) != cudaSuccess) return fail_cuda(JK_ERR_CUDA, "cudaSetDevice failed");
@@ -673,15 +678,48 @@ int autotune(Plan *P, const double *D, cudaStream_t st, const char *cache_path, 
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    float part_ms = 0;
-    // candidates (family, kets per tile): for s and p class pairs the
-    // lane-per-bra kernels with 8 .. 128 kets per tile, the warp kernels with
-    // 128 .. 2048 kets per warp and the pair-queue kernels with 32 .. 512
-    // kets per tile; for class pairs with a d shell the warp kernels with 1
-    // .. 2048 kets per warp; a choice is stored as family * 65536 + kets
-    std::vector<int> cands_t = {8, 16, 32, 64, 128}, cands_w, cands_d = {1, 4, 16, 64, 128, 512, 2048};
-    for (int c : {128, 256, 512, 1024, 2048}) cands_w.push_back(65536 + c);   // warp kernels
-    for (int c : {32, 64, 128, 256, 512}) cands_w.push_back(2 * 65536 + c);   // pair-queue kernels
+    // device time of choice c over the bras [b0, b1) of a class pair, the
+    // shortest of reps launches; negative if a launch failed
+    const auto timed = [&](int cb, int ck, int b0, int b1, int c, int reps) -> float {
+        const ClassRange &B = P->classes[cb], &Kc = P->classes[ck];
+        float best = 1e30f;
+        for (int r = 0; r < reps; ++r) {
+            RealLaunch a{};
+            a.pl = pl;
+            a.b0 = b0;
+            a.b1 = b1;
+            a.k0 = Kc.b0;
+            a.k1 = Kc.b1;
+            a.same = cb == ck;
+            a.kchunk = c & 65535;
+            a.map = tile_map(P, B, a.b0, a.b1, a.k0, a.k1, a.kchunk);
+            a.variant = c >> 16;
+            a.mode = 0;
+            a.fp32 = mixed;
+            a.Dp = w.Dp;
+            a.dmax = w.dmax;
+            a.Dpf = w.Dpf;
+            a.dmaxf = w.dmaxf;
+            a.X = w.X;
+            a.Y = w.Y;
+            a.cnt = w.cnt;
+            a.st = st;
+            cudaEventRecord(e0, st);
+            launch_real(cb, ck, a);
+            cudaEventRecord(e1, st);
+            float ms = 0;
+            if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) return -1.0f;
+            best = std::min(best, ms);
+            if (ms > (b1 - b0 < B.b1 - B.b0 ? 2.0f : 20.0f)) break;  // long enough not to need another
+        }
+        return best;
+    };
+    // candidates: for s and p class pairs the lane-per-bra kernels with 8 .. 128
+    // kets per tile, the warp kernels with 8 .. 2048 kets per warp (1 .. 256
+    // where a warp takes one image quartet) and the pair-queue kernels with 32
+    // .. 512 kets per tile; for class pairs with a d shell their one kernel with
+    // 1 .. 2048 kets per warp
+    constexpr float kMargin = 0.98f;
     int k = 0;
     bool dirty = false;
     for (int cb = 0; cb < JK_NCLASS_MAX; ++cb)
@@ -693,66 +731,69 @@ int autotune(Plan *P, const double *D, cudaStream_t st, const char *cache_path, 
             }
             if (B.b1 <= B.b0 || Kc.b1 <= Kc.b0) continue;
             char key[512];
-            snprintf(key, sizeof key, "%s|%s|v4|%d%d|%d|%d", prop.name, mixed ? "mixed" : "fp64", cb, ck, bucket(B.b1 - B.b0),
+            snprintf(key, sizeof key, "%s|%s|v5|%d%d|%d|%d", prop.name, mixed ? "mixed" : "fp64", cb, ck, bucket(B.b1 - B.b0),
                      bucket(Kc.b1 - Kc.b0));
             for (char *q = key; *q; ++q)
                 if (*q == ' ') *q = '_';
-            int best = -1;
+            int family, kets;
+            P->default_schedule(cb, ck, family, kets);
+            const int own = family << 16 | kets;
+            int best = 0;
             auto it = cache.find(key);
             if (it != cache.end()) {
                 best = it->second;
             } else {
-                float best_ms = 1e30f;
-                std::vector<int> cands = real_has_warp_kernel(cb, ck) ? cands_t : cands_d;
-                if (real_has_warp_kernel(cb, ck)) cands.insert(cands.end(), cands_w.begin(), cands_w.end());
-                // two sub-ranges of at most 2048 bras (the class is sorted by
-                // primitive count, so the start and the middle differ)
-                const int nbc = B.b1 - B.b0, mid = B.b0 + nbc / 2;
-                for (int c : cands)
-                    for (int part = 0; part < 2; ++part) {
-                        RealLaunch a{};
-                        a.pl = pl;
-                        a.b0 = part == 0 ? B.b0 : std::max(B.b0 + std::min(nbc, 2048), mid);
-                        a.b1 = std::min(B.b1, a.b0 + 2048);
-                        if (a.b1 <= a.b0) continue;
-                        a.k0 = Kc.b0;
-                        a.k1 = Kc.b1;
-                        a.same = cb == ck;
-                        a.kchunk = c & 65535;
-                        a.map = tile_map(P, a.b0, a.b1, a.k0, a.k1, a.kchunk);
-                        a.variant = c >> 16;
-                        a.mode = 0;
-                        a.fp32 = mixed;
-                        a.Dp = w.Dp;
-                        a.dmax = w.dmax;
-                        a.Dpf = w.Dpf;
-                        a.dmaxf = w.dmaxf;
-                        a.X = w.X;
-                        a.Y = w.Y;
-                        a.cnt = w.cnt;
-                        a.st = st;
-                        cudaEventRecord(e0, st);
-                        launch_real(cb, ck, a);
-                        cudaEventRecord(e1, st);
-                        if (cudaEventSynchronize(e1) != cudaSuccess) {
-                            cudaEventDestroy(e0);
-                            cudaEventDestroy(e1);
-                            return fail_cuda(JK_ERR_CUDA, "autotune launch failed");
-                    }
-                        float ms = 0;
-                        cudaEventElapsedTime(&ms, e0, e1);
-                        if (part == 0) part_ms = ms;
-                        else part_ms += ms;
-                        if (part == 1 || nbc <= 2048) {
-                            if (part_ms < best_ms) {
-                                best_ms = part_ms;
-                                best = c;
-                            }
+                std::vector<int> cands;
+                if (real_has_warp_kernel(cb, ck)) {
+                    for (int c : {8, 16, 32, 64, 128}) cands.push_back(c);
+                    if (P->warp_per_quartet(cb, ck))
+                        for (int c : {1, 4, 16, 64, 256}) cands.push_back(65536 + c);
+                    else
+                        for (int c : {8, 32, 128, 256, 512, 1024, 2048}) cands.push_back(65536 + c);
+                    for (int c : {32, 64, 128, 256, 512}) cands.push_back(2 * 65536 + c);
+                } else {
+                    for (int c : {1, 4, 16, 64, 128, 512, 2048}) cands.push_back(c);
+                }
+                cands.erase(std::remove(cands.begin(), cands.end(), own), cands.end());
+                // the class is sorted by primitive count, so the start and the middle differ
+                const int nbc = B.b1 - B.b0, m0 = std::max(B.b0 + std::min(nbc, 2048), B.b0 + nbc / 2), m1 = std::min(B.b1, m0 + 2048);
+                const auto sample = [&](int c) -> float {
+                    const float t0 = timed(cb, ck, B.b0, std::min(B.b1, B.b0 + 2048), c, 3);
+                    const float t1 = m1 > m0 ? timed(cb, ck, m0, m1, c, 3) : 0.0f;
+                    return t0 < 0 || t1 < 0 ? -1.0f : t0 + t1;
+                };
+                float t_own = sample(own);
+                bool failed = t_own < 0;
+                std::vector<std::pair<float, int>> t;
+                for (int c : cands) {
+                    t.push_back({sample(c), c});
+                    failed = failed || t.back().first < 0;
+                }
+                std::sort(t.begin(), t.end());
+                if (nbc > 2048) {
+                    const auto prims = [&](int i0, int i1) { return i1 > i0 ? P->spi[i1 - 1].pp0 + P->spi[i1 - 1].npp - P->spi[i0].pp0 : 0; };
+                    const double part = (double)prims(B.b0, B.b0 + 2048) + prims(m0, m1);
+                    if (t_own * prims(B.b0, B.b1) / part < 1000.0) {
+                        t_own = timed(cb, ck, B.b0, B.b1, own, 2);
+                        failed = failed || t_own < 0;
+                        t.resize(std::min<size_t>(t.size(), 2));
+                        for (auto &x : t) {
+                            x.first = timed(cb, ck, B.b0, B.b1, x.second, 2);
+                            failed = failed || x.first < 0;
+                        }
+                        std::sort(t.begin(), t.end());
                     }
                 }
+                if (failed) {
+                    cudaEventDestroy(e0);
+                    cudaEventDestroy(e1);
+                    return fail_cuda(JK_ERR_CUDA, "autotune launch failed");
+                }
+                if (!t.empty() && t[0].first < kMargin * t_own) best = t[0].second;
                 cache[key] = best;
                 dirty = true;
             }
+            if (best >> 16 > 2 || (best >> 16 > 0 && !real_has_warp_kernel(cb, ck)) || best <= 0 || (best & 65535) == 0) best = own;
             P->kchunk[cb][ck] = best & 65535;
             P->kvariant[cb][ck] = best >> 16;
             if (chosen) {

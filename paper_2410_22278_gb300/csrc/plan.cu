@@ -557,6 +557,28 @@ static int alloc_ws(Plan *P)
     return JK_OK;
 }
 
+// Untuned schedule: the warp kernels, with kets per warp for about 256 warps
+// per SM (half of them empty for a class with itself) up to 512 kets, then for a
+// thousand warps per SM up to 2048 -- few enough that a small cell still fills
+// the chip and the last warps do not hold up a launch, enough to fill the
+// batches of a warp; the kernels that give an image quartet a whole warp
+// (real3.cuh) have no batches and take 1 to 64.
+void Plan::default_schedule(int cb, int ck, int &family, int &kets) const
+{
+    const ClassRange &B = classes[cb], &K = classes[ck];
+    const long long few = (long long)(B.b1 - B.b0) * (K.b1 - K.b0) / (152 * 1024);
+    family = cb <= 2 && ck <= 2 ? 1 : 0;
+    kets = (int)(warp_per_quartet(cb, ck) ? std::min(64LL, std::max(1LL, few))
+                                          : std::max(std::min(512LL, std::max(8LL, 4 * few)), std::min(2048LL, few)));
+}
+
+// Class pairs whose blocks are too large for a lane (more than 36 elements).
+bool Plan::warp_per_quartet(int cb, int ck) const
+{
+    const auto nc = [](int l) { return (l + 1) * (l + 2) / 2; };
+    return nc(classes[cb].la) * nc(classes[cb].lb) * nc(classes[ck].la) * nc(classes[ck].lb) > 36;
+}
+
 int build_plan(const jk_cell *cell, const jk_shell *shells, int nshell, double omega, const jk_cutoffs *cut,
                jk_precision precision, int device, Plan **out)
 {
@@ -581,7 +603,7 @@ int build_plan(const jk_cell *cell, const jk_shell *shells, int nshell, double o
     Plan *P = new Plan();
     for (int i = 0; i < JK_NCLASS_MAX; ++i)
         for (int j = 0; j < JK_NCLASS_MAX; ++j) {
-            P->kvariant[i][j] = (i <= 2 && j <= 2) ? 1 : 0;
+            P->kvariant[i][j] = 0;
             P->kchunk[i][j] = 32;
         }
     P->device = device;
@@ -823,22 +845,8 @@ int build_plan(const jk_cell *cell, const jk_shell *shells, int nshell, double o
         if (cr.b1 <= cr.b0) cr.b0 = cr.b1 = 0;
         P->classes.push_back(cr);
     }
-    // untuned schedule: kets per warp for about 256 warps per SM (half of them
-    // empty for a class with itself) up to 512 kets, then for a thousand warps
-    // per SM up to 2048 -- few enough that a small cell still fills the chip
-    // and the last warps do not hold up a launch, enough to fill the batches of
-    // a warp; the kernels that give an image quartet a whole warp (real3.cuh)
-    // have no batches and take 1 to 64
     for (int i = 0; i < JK_NCLASS_MAX; ++i)
-        for (int j = i; j < JK_NCLASS_MAX; ++j) {
-            const ClassRange &B = P->classes[i], &K = P->classes[j];
-            const long long nb = B.b1 - B.b0, nk = K.b1 - K.b0;
-            const auto nc = [](int l) { return (l + 1) * (l + 2) / 2; };
-            const bool coop = nc(B.la) * nc(B.lb) * nc(K.la) * nc(K.lb) > 36;
-            const long long few = nb * nk / (152 * 1024);
-            P->kchunk[i][j] = (int)(coop ? std::min(64LL, std::max(1LL, few))
-                                         : std::max(std::min(512LL, std::max(8LL, 4 * few)), std::min(2048LL, few)));
-        }
+        for (int j = i; j < JK_NCLASS_MAX; ++j) P->default_schedule(i, j, P->kvariant[i][j], P->kchunk[i][j]);
     // ---- unique shell pairs with their images (reciprocal-space build), grouped by class
     {
         std::map<std::pair<int, int>, std::vector<int>> byp;

@@ -211,6 +211,8 @@ struct Plan {
     std::vector<EnergySlot> energy_free;  // not in use by a call
     std::vector<EnergySlot> energy_lost;  // left by a failed call
     PlanDev dev() const;
+    void default_schedule(int cb, int ck, int &family, int &kets) const;
+    bool warp_per_quartet(int cb, int ck) const;
     // unique image quartets of a pair of classes
     long long class_quartets(int cb, int ck) const
     {
