@@ -19,7 +19,8 @@
 #define JK_NCLASS_MAX 6          // (la, lb) with la >= lb, la <= 2
 
 // Boys table: F_m(T_k) for T_k = k / JK_BOYS_INV_STEP, k = 0 .. JK_BOYS_NPTS-1,
-// m = 0 .. JK_BOYS_MCOL-1.  Above JK_BOYS_TMAX the asymptotic branch is used.
+// m = 0 .. JK_BOYS_MCOL-1, in single precision.  The FP32 seeds read it below
+// T = L + 1.5 and take erfc and the upward recursion above.
 #define JK_BOYS_INV_STEP 32
 #define JK_BOYS_TMAX 36.0
 #define JK_BOYS_NPTS (36 * 32 + 2)
@@ -121,8 +122,7 @@ struct PlanDev {
     const PpiRec *ppi;
     const SpairRec *spair;
     const int *spi_order;        // spi indices grouped by shell pair (for the reciprocal build)
-    const double *boys;          // [JK_BOYS_NPTS][JK_BOYS_MCOL]
-    const float *boys_f;
+    const float *boys_f;         // [JK_BOYS_NPTS][JK_BOYS_MCOL]
     const double *boys_t;        // [JK_MAXLQ + 2][JK_TPTS][JK_TROW] Taylor rows of F_L and H_0
     const PpiF *ppf;
     const float *ppB;            // B = |K| p^{-5/4} of each primitive pair (descending inside an image)

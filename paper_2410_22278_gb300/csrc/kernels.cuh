@@ -82,9 +82,6 @@ __device__ __forceinline__ void seeds(double x2, double alpha, double aw, double
         f *= -2.0 * alpha;
     }
 }
-// Single precision unless c_w is close to 1 (the integration interval
-// [c_w, 1] is short and the table branch would lose bits), where the seed is
-// formed in double and rounded once.
 // Single precision throughout.  The mixed path sends every quartet whose
 // largest c_w exceeds 0.85 (the integration interval [c_w, 1] is short and
 // the table branch would lose bits) to the FP64 list instead (k_real, mode

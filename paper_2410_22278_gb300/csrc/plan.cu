@@ -343,7 +343,6 @@ PlanDev Plan::dev() const
     d.ppi = d_ppi;
     d.spair = d_spair;
     d.spi_order = d_spi_order;
-    d.boys = d_boys;
     d.boys_f = d_boys_f;
     d.boys_t = d_boys_t;
     d.r1 = d_r1;
@@ -1120,7 +1119,7 @@ int finish_plan_device(Plan *P)
     std::vector<double> tab;
     boys_table(JK_BOYS_MCOL, JK_BOYS_NPTS, JK_BOYS_INV_STEP, tab);
     std::vector<float> tabf(tab.begin(), tab.end());
-    if ((rc = upload(tab, &P->d_boys, b)) || (rc = upload(tabf, &P->d_boys_f, b))) return rc;
+    if ((rc = upload(tabf, &P->d_boys_f, b))) return rc;
     if ((rc = upload(taylor_rows(), &P->d_boys_t, b))) return rc;
     std::vector<double> g0 = {0.0, 0.0, 0.0, 1.0};
     if ((rc = upload(g0, &P->d_g0, b))) return rc;
@@ -1241,7 +1240,7 @@ void destroy_plan(Plan *P)
         if (P->side_join[i]) cudaEventDestroy(P->side_join[i]);
     }
     if (P->side_fork) cudaEventDestroy(P->side_fork);
-    void *ptrs[] = {P->d_shells, P->d_spi, P->d_ppi, P->d_ppf, P->d_ppB, P->d_pps, P->d_pplb, P->d_r1f, P->d_spair, P->d_spi_order, P->d_boys, P->d_boys_f, P->d_boys_t, P->d_r1, P->d_gvec,
+    void *ptrs[] = {P->d_shells, P->d_spi, P->d_ppi, P->d_ppf, P->d_ppB, P->d_pps, P->d_pplb, P->d_r1f, P->d_spair, P->d_spi_order, P->d_boys_f, P->d_boys_t, P->d_r1, P->d_gvec,
                     P->d_g0, P->d_compf, P->d_ppi_ab, P->d_kblk, P->d_kblk2, P->d_spq, P->d_spr, P->d_spd, P->d_pvals, P->d_gtab0, P->d_ppi_pidx, P->d_phase, P->d_ppdf, P->d_gdf, P->d_phasef, P->ws.gtab, P->ws.gtab2, P->d_S, P->ws.Dp, P->ws.X, P->ws.Y, P->ws.JLR, P->ws.KLR, P->ws.T1, P->ws.T2,
                     P->ws.M, P->ws.Z, P->ws.rho, P->ws.rho_part, P->ws.DhD, P->ws.JH, P->ws.DhF, P->ws.dmax, P->ws.scal, P->ws.err, P->ws.cnt, P->ws.big, P->ws.nbig,
                     P->ws.Ms, P->ws.Zs, P->ws.Ds, P->ws.Mex, P->ws.Zex, P->ws.Dex, P->ws.Dpf, P->ws.dmaxf, P->ws.Cs, P->ws.Cex, P->ws.Kpart,

@@ -171,7 +171,6 @@ struct Plan {
     float *d_r1f = nullptr;
     SpairRec *d_spair = nullptr;
     int *d_spi_order = nullptr;
-    double *d_boys = nullptr;
     float *d_boys_f = nullptr;
     double *d_boys_t = nullptr;  // Taylor rows of the FP64 seeds
     double *d_r1 = nullptr;
