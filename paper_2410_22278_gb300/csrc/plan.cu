@@ -418,10 +418,10 @@ static int upload(const std::vector<T> &h, T **d, size_t &bytes)
 // in use from its tile kernel to its list pass, so each lane of the real-space
 // phase needs one; the l-th lane's holds the l-th largest class pair, and a
 // class pair only goes to a lane that can hold it (run_build).  As many lanes as
-// fit the bytes that one list of 8-byte entries and partial sums for the
-// largest split of every slab took: a plan with side streams asks for no more
-// than one without (a server admits plans by their workspace).
-static void quartet_lists(Plan *P, size_t &bytes)
+// fit the bytes of one list of 8-byte entries and `spare` more, what the rest of
+// the workspace does without: a plan with side streams asks for no more than one
+// without did (a server admits plans by their workspace).
+static void quartet_lists(Plan *P, long long spare, size_t &bytes)
 {
     Workspace &w = P->ws;
     const long long cap = std::min<long long>(std::max<long long>(P->n_quartets / 50, 1 << 20), 64ll << 20);
@@ -431,8 +431,7 @@ static void quartet_lists(Plan *P, size_t &bytes)
     std::sort(need.rbegin(), need.rend());
     const bool narrow = P->spi.size() <= 65536;
     w.list_elt = narrow ? sizeof(unsigned) : sizeof(int2);
-    const long long slab = 2LL * w.gc * kSlabSplitsMax - slab_part_size(2 * w.gc) - 8;  // doubles
-    const long long fit = cap * (long long)sizeof(int2) + slab * (long long)sizeof(double);
+    const long long fit = cap * (long long)sizeof(int2) + spare;
     static_assert(Workspace::kLists >= Plan::kSide, "a list per lane");
     w.nlist = std::max(1, P->nside);
     const auto total = [&] { return std::accumulate(need.begin(), need.begin() + w.nlist, 0LL) * (long long)w.list_elt; };
@@ -493,17 +492,25 @@ static int alloc_ws(Plan *P)
         bytes += std::max<size_t>(count, 1) * sizeof(double);
         return true;
     };
+    // What the plan takes less of than one with partial sums for the largest
+    // split of every slab, J-engine arrays without a use and a second Gaussian
+    // table (less a few words for the counters of the lists).
+    long long spare = (2LL * gc * kSlabSplitsMax - slab_part_size(2 * (int)gc) - 8) * (long long)sizeof(double);
     bool ok = al(&w.gtab, std::max<size_t>(1, P->pvals.size()) * (size_t)gc) && al(&w.Dp, n2) && al(&w.X, n2) && al(&w.Y, n2) && al(&w.JLR, n2) && al(&w.KLR, n2) && al(&w.T1, n2) &&
               al(&w.T2, n2) && al(&w.M, 2 * (size_t)gc * n2) && al(&w.Z, 2 * (size_t)gc * n2) && al(&w.rho, 2 * (size_t)gc) && al(&w.rho_part, slab_part_size(2 * (int)gc)) &&
               al(&w.dmax, (size_t)P->nshell * P->nshell) && al(&w.scal, 16) && (!mixed || al((double **)&w.Dpf, (n2 + 1) / 2)) &&
               (!mixed || al((double **)&w.dmaxf, ((size_t)P->nshell * P->nshell + 2) / 2));
     {
-        // J-engine arrays: stride N_H(2 lmax)
+        // J-engine arrays: stride N_H(2 lmax); only plans with d shells use them
         int lmax = 0;
         for (auto &sh : P->shells) lmax = std::max(lmax, sh.l);
         const int L2 = 2 * lmax;
         w.hs = (L2 + 1) * (L2 + 2) * (L2 + 3) / 6;
-        const size_t nh = std::max<size_t>(1, P->ppi.size()) * w.hs;
+        size_t nh = std::max<size_t>(1, P->ppi.size()) * w.hs;
+        if (lmax < 2) {
+            spare += (long long)(nh - 1) * 20;
+            nh = 1;
+        }
         ok = ok && al(&w.DhD, nh) && al(&w.JH, nh) && al((double **)&w.DhF, (nh + 1) / 2);
     }
     if (!ok) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed for build workspace");
@@ -524,9 +531,8 @@ static int alloc_ws(Plan *P)
             bytes += count * sizeof(int);
             return true;
         };
-        if (cudaMalloc((void **)&w.gtab2, std::max<size_t>(1, P->pvals.size()) * (size_t)gc * sizeof(float2)) != cudaSuccess)
-            return fail_cuda(JK_ERR_OOM, "cudaMalloc failed for the double-float Gaussian table");
-        bytes += std::max<size_t>(1, P->pvals.size()) * (size_t)gc * sizeof(float2);
+        w.gtab2 = reinterpret_cast<float2 *>(w.gtab);
+        spare += (long long)std::max<size_t>(1, P->pvals.size()) * gc * (long long)sizeof(float2);
         if (!alb(&w.Ms, 2 * (size_t)gc * sl) || !alb(&w.Zs, 2 * (size_t)gc * sl) || !alb(&w.Ds, sl) || !alb(&w.Cs, sl) ||
             !ali(&w.Mex, 2 * (size_t)gc * w.npad) || !ali(&w.Zex, 2 * (size_t)gc * w.npad) || !ali(&w.Dex, w.npad) ||
             !ali(&w.Cex, w.npad))
@@ -545,7 +551,7 @@ static int alloc_ws(Plan *P)
     if (cudaMalloc((void **)&w.cnt, kCounters * sizeof(unsigned long long)) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed");
     if (P->precision == JK_MIXED) {
         size_t lb = 0;
-        quartet_lists(P, lb);
+        quartet_lists(P, spare, lb);
         if (cudaMalloc((void **)&w.big, lb) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed for quartet list");
         if (cudaMalloc((void **)&w.nbig, 2 * sizeof(unsigned) * w.nlist) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed");
         bytes += lb + 2 * sizeof(unsigned) * w.nlist;
@@ -632,8 +638,9 @@ int build_plan(const jk_cell *cell, const jk_shell *shells, int nshell, double o
     if (!(c.ewald_K > 0)) c.ewald_K = 1e-14;
     // 3e-3 by default, 300 times the paper's switch-over value (Section
     // 3.5): this GPU's FP64 rate is 1/74 of its measured FP32 rate (about 1/2
-    // on the paper's GPU); on the 64-water box mixed stays within 7e-9 of FP64
-    // in J and K and 3e-9 Ha in E, and within 2.3e-9 of the oracle's rows
+    // on the paper's GPU); on 64-water boxes mixed stays within 7e-9 of FP64 in
+    // J and K and 6e-8 Ha in E (1.1e-8 on the benchmark's), and within 2e-9 of
+    // the oracle's rows
     P->mixed_tau = c.mixed_switch > 0 ? c.mixed_switch : 3e-3;
     P->cut = c;
 
@@ -1241,7 +1248,7 @@ void destroy_plan(Plan *P)
     }
     if (P->side_fork) cudaEventDestroy(P->side_fork);
     void *ptrs[] = {P->d_shells, P->d_spi, P->d_ppi, P->d_ppf, P->d_ppB, P->d_pps, P->d_pplb, P->d_r1f, P->d_spair, P->d_spi_order, P->d_boys_f, P->d_boys_t, P->d_r1, P->d_gvec,
-                    P->d_g0, P->d_compf, P->d_ppi_ab, P->d_kblk, P->d_kblk2, P->d_spq, P->d_spr, P->d_spd, P->d_pvals, P->d_gtab0, P->d_ppi_pidx, P->d_phase, P->d_ppdf, P->d_gdf, P->d_phasef, P->ws.gtab, P->ws.gtab2, P->d_S, P->ws.Dp, P->ws.X, P->ws.Y, P->ws.JLR, P->ws.KLR, P->ws.T1, P->ws.T2,
+                    P->d_g0, P->d_compf, P->d_ppi_ab, P->d_kblk, P->d_kblk2, P->d_spq, P->d_spr, P->d_spd, P->d_pvals, P->d_gtab0, P->d_ppi_pidx, P->d_phase, P->d_ppdf, P->d_gdf, P->d_phasef, P->ws.gtab, P->d_S, P->ws.Dp, P->ws.X, P->ws.Y, P->ws.JLR, P->ws.KLR, P->ws.T1, P->ws.T2,
                     P->ws.M, P->ws.Z, P->ws.rho, P->ws.rho_part, P->ws.DhD, P->ws.JH, P->ws.DhF, P->ws.dmax, P->ws.scal, P->ws.err, P->ws.cnt, P->ws.big, P->ws.nbig,
                     P->ws.Ms, P->ws.Zs, P->ws.Ds, P->ws.Mex, P->ws.Zex, P->ws.Dex, P->ws.Dpf, P->ws.dmaxf, P->ws.Cs, P->ws.Cex, P->ws.Kpart,
                     P->ws.lr.Vt, P->ws.lr.diag, P->ws.lr.done_row, P->ws.lr.sgn, P->ws.lr.rowmap, P->ws.lr.dyn, P->ws.lr.bar, P->ws.lr.Ct};

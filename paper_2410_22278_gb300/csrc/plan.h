@@ -66,7 +66,7 @@ struct Workspace {
     unsigned list_cap[kLists] = {};
     int gc = 0;               // G vectors per chunk
     double *gtab = nullptr;   // [distinct p][gc]: (pi/p)^{3/2} e^{-G^2/4p} of the current G chunk
-    float2 *gtab2 = nullptr;  // the same as double-floats (mixed-precision structure factors)
+    float2 *gtab2 = nullptr;  // the same as double-floats (mixed-precision structure factors), in its place
     size_t bytes = 0;
     // split-precision tensor-core exchange (mixed precision)
     int npad = 0, oz_slices = 0;

@@ -767,9 +767,10 @@ __device__ __forceinline__ void eval_terms(const PlanDev &pl, const unsigned *ri
 // The work of a warp is bounded by its primitive quartets, not its kets: cut
 // by kets alone, the (ss|ss) launch of a 5-molecule box waited for one warp
 // (36 x 36 primitive quartets, up to 20 images each) for 80% of its 63 ms.
-// Against one ket's primitives per step and kets alone: mixed J+K build of 5
-// water molecules 77 -> 29 ms, of 31 (reciprocal cache) 223 -> 193 ms, of 64
-// 962 -> 801 ms; FP64 build of 6 molecules 325 -> 131 ms.  Bound by
+// Against one ket's primitives per step and kets alone, when this split came
+// in: mixed J+K build of 5 water molecules 77 -> 29 ms, of 31 (reciprocal cache)
+// 223 -> 193 ms, of 64 962 -> 801 ms; FP64 build of 6 molecules 325 -> 131 ms
+// (with what followed 22.9, 176, 713 and 85.6 ms).  Bound by
 // instruction issue (0.53 a clock and scheduler, 17 of 32 lanes active).
 // The stages have very different pass rates (water box, (ss|ss): 17% of the
 // pairs, then 1.3 terms out of 6.7 screened primitive quartets per pair), so

@@ -17,9 +17,11 @@
 // quartet (the lane-per-bra kernel this replaces here) the whole chain ran in
 // one lane with its arrays in local memory, and a class pair with a few
 // thousand quartets kept a few warps busy for tens of milliseconds.  With the
-// split of real2.cuh for the smaller classes: FP64 build of a 20-function
-// s/p/d cell 321 -> 7.2 ms, mixed build of one diamond cell 386 -> 26 ms, of
-// 2 x 2 x 2 cells 745 -> 340 ms.
+// split of real2.cuh for the smaller classes, when they came in: FP64 build of
+// a 20-function s/p/d cell 321 -> 7.2 ms, mixed build of one diamond cell 386 ->
+// 26 ms, of 2 x 2 x 2 cells 745 -> 340 ms (with what followed 1.93, 16.3 and 299
+// ms).  (pp|pp) of 16 water molecules: 0.20 ms, issue slots 15% busy, waiting
+// on global and shared memory in turn; its FP64 list 1.4 ms.
 #pragma once
 #include "real2.cuh"
 
