@@ -67,33 +67,53 @@ __device__ __forceinline__ void kinetic_block(const PpiRec &x, double b, double 
         }
 }
 
+// Where the images of a class start, where their blocks do, its first shell
+// pair and its first element among all (first[JK_NCLASS_MAX]: their number).
+struct ImageBlocks {
+    int b0[JK_NCLASS_MAX], sp0[JK_NCLASS_MAX];
+    size_t off[JK_NCLASS_MAX];
+    long long first[JK_NCLASS_MAX + 1];
+};
+
 // Every kernel below leaves the block of a shell-pair image of its own (blk:
 // those of one class, NA x NB elements an image); this sums the images of each
-// shell pair in their order into the raw matrix, one element per thread, so a
-// repeated call gives the same bits (images added by atomics did not, at the
-// same time).  For I = J an image with R != 0 stands for its mirror too.
-template <int LA, int LB>
-__global__ void __launch_bounds__(128) k_onee_gather(PlanDev pl, int sp0, int sp1, int b0, const double *__restrict__ blk,
-                                                     double *__restrict__ Out)
+// shell pair into the raw matrix, gsz lanes an element and in a fixed order, so
+// a repeated call gives the same bits (images added by atomics did not).  For
+// I = J an image with R != 0 stands for its mirror too.  Bound by latency: all
+// classes in one launch, eight chains an element, or 32 in small cells, whose
+// shell pairs have ten and more images (launched class by class with one chain
+// an element, a call on the 8-function cell took 0.90 ms instead of 0.87, on one
+// water molecule 4.26 instead of 4.07; those are the times with atomics).
+__global__ void __launch_bounds__(128) k_onee_gather(PlanDev pl, ImageBlocks ib, int gsz, const double *__restrict__ blk, double *__restrict__ Out)
 {
-    constexpr int NB = ncart(LB), NAB = ncart(LA) * NB;
-    const long long t = blockIdx.x * 128LL + threadIdx.x;
-    const int sp = sp0 + (int)(t / NAB), e = (int)(t % NAB);
-    if (sp >= sp1) return;
-    const SpairRec rec = pl.spair[sp];
+    const long long x = (blockIdx.x * 128LL + threadIdx.x) / gsz;
+    const int part = threadIdx.x & (gsz - 1);
+    const bool on = x < ib.first[JK_NCLASS_MAX];
+    int c = 0;
+    while (c + 1 < JK_NCLASS_MAX && x >= ib.first[c + 1]) ++c;
+    const int la = c == 0 ? 0 : c <= 2 ? 1 : 2, lb = c - la * (la + 1) / 2, NB = ncart(lb), NAB = ncart(la) * NB;
     double sum = 0.0;
-    for (int q = 0; q < rec.nspi; ++q) {
-        const int img = pl.spi_order[rec.spi0 + q];
-        const double *v = blk + (size_t)(img - b0) * NAB;
-        sum += v[e];
-        if (rec.I == rec.J) {
-            const SpiRec &si = pl.spi[img];
-            if (si.n[0] || si.n[1] || si.n[2]) sum += v[(e % NB) * NB + e / NB];
+    SpairRec rec{};
+    int e = 0;
+    if (on) {
+        rec = pl.spair[ib.sp0[c] + (int)((x - ib.first[c]) / NAB)];
+        e = (int)((x - ib.first[c]) % NAB);
+        for (int q = part; q < rec.nspi; q += gsz) {
+            const int img = pl.spi_order[rec.spi0 + q];
+            const double *v = blk + ib.off[c] + (size_t)(img - ib.b0[c]) * NAB;
+            sum += v[e];
+            if (rec.I == rec.J) {
+                const SpiRec &si = pl.spi[img];
+                if (si.n[0] || si.n[1] || si.n[2]) sum += v[(e % NB) * NB + e / NB];
+            }
         }
     }
-    const size_t n = pl.nbf, r = pl.shells[rec.I].ao + e / NB, c = pl.shells[rec.J].ao + e % NB;
-    Out[r * n + c] = sum;
-    if (rec.I != rec.J) Out[c * n + r] = sum;
+    __syncwarp();
+    for (int o = gsz >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (!on || part != 0) return;
+    const size_t n = pl.nbf, r = pl.shells[rec.I].ao + e / NB, k = pl.shells[rec.J].ao + e % NB;
+    Out[r * n + k] = sum;
+    if (rec.I != rec.J) Out[k * n + r] = sum;
 }
 
 // Kinetic energy: one warp per shell-pair image, one primitive pair per lane.
@@ -357,7 +377,7 @@ __global__ void __launch_bounds__(128) k_onee_recip(PlanDev pl, int b0, int g0, 
 }
 
 // one launch per class of shell-pair images (op 0 kinetic, 1 real part, 2
-// reciprocal part of the attraction, 3 the images into the raw matrix)
+// reciprocal part of the attraction)
 struct OneeArgs {
     PlanDev pl;
     int op = 0;
@@ -373,7 +393,7 @@ struct OneeArgs {
     cudaStream_t st;
 };
 template <int LA, int LB>
-static size_t onee_go(const OneeArgs &a, int b0, int b1, int sp0, int sp1, size_t off)
+static size_t onee_go(const OneeArgs &a, int b0, int b1, size_t off)
 {
     constexpr int NAB = ncart(LA) * ncart(LB);
     if (b1 <= b0) return off;
@@ -382,10 +402,8 @@ static size_t onee_go(const OneeArgs &a, int b0, int b1, int sp0, int sp1, size_
     if (a.op == 0) k_onee_kinetic<LA, LB><<<(nb + 3) / 4, 128, 0, a.st>>>(a.pl, b0, b1, a.ab, blk);
     else if (a.op == 1)
         k_onee_real<LA, LB><<<(nb + 3) / 4, 128, 0, a.st>>>(a.pl, b0, b1, a.natom, a.Z, a.xyz, a.cand, a.ncand, a.natom > 16 ? 32 : 8, blk);
-    else if (a.op == 2)
-        k_onee_recip<LA, LB><<<nb, 128, 3 * (2 * a.nmax + 1) * sizeof(double2), a.st>>>(a.pl, b0, a.g0, a.gcur, a.nmax, a.v, a.gtab, blk);
     else
-        k_onee_gather<LA, LB><<<(unsigned)(((long long)(sp1 - sp0) * NAB + 127) / 128), 128, 0, a.st>>>(a.pl, sp0, sp1, b0, blk, a.Out);
+        k_onee_recip<LA, LB><<<nb, 128, 3 * (2 * a.nmax + 1) * sizeof(double2), a.st>>>(a.pl, b0, a.g0, a.gcur, a.nmax, a.v, a.gtab, blk);
     return off + (size_t)nb * NAB;
 }
 
@@ -394,17 +412,33 @@ static void launch_onee(const Plan *P, OneeArgs a, int op)
     a.op = op;
     size_t off = 0;
     for (int c = 0; c < JK_NCLASS_MAX; ++c) {
-        const int b0 = P->classes[c].b0, b1 = P->classes[c].b1, s0 = P->spair_class_off[c], s1 = P->spair_class_off[c + 1];
+        const int b0 = P->classes[c].b0, b1 = P->classes[c].b1;
         switch (c) {
-        case 0: off = onee_go<0, 0>(a, b0, b1, s0, s1, off); break;
-        case 1: off = onee_go<1, 0>(a, b0, b1, s0, s1, off); break;
-        case 2: off = onee_go<1, 1>(a, b0, b1, s0, s1, off); break;
-        case 3: off = onee_go<2, 0>(a, b0, b1, s0, s1, off); break;
-        case 4: off = onee_go<2, 1>(a, b0, b1, s0, s1, off); break;
-        case 5: off = onee_go<2, 2>(a, b0, b1, s0, s1, off); break;
+        case 0: off = onee_go<0, 0>(a, b0, b1, off); break;
+        case 1: off = onee_go<1, 0>(a, b0, b1, off); break;
+        case 2: off = onee_go<1, 1>(a, b0, b1, off); break;
+        case 3: off = onee_go<2, 0>(a, b0, b1, off); break;
+        case 4: off = onee_go<2, 1>(a, b0, b1, off); break;
+        case 5: off = onee_go<2, 2>(a, b0, b1, off); break;
         default: break;
         }
     }
+}
+
+static void launch_gather(const Plan *P, const OneeArgs &a)
+{
+    ImageBlocks ib{};
+    for (int c = 0; c < JK_NCLASS_MAX; ++c) {
+        const ClassRange &r = P->classes[c];
+        const long long nab = ncart(r.la) * ncart(r.lb);
+        ib.b0[c] = r.b0;
+        ib.sp0[c] = P->spair_class_off[c];
+        if (c + 1 < JK_NCLASS_MAX) ib.off[c + 1] = ib.off[c] + (size_t)((r.b1 - r.b0) * nab);
+        ib.first[c + 1] = ib.first[c] + (P->spair_class_off[c + 1] - P->spair_class_off[c]) * nab;
+    }
+    const int gsz = P->spi.size() > 8 * P->spair.size() ? 32 : 8;
+    const long long threads = gsz * ib.first[JK_NCLASS_MAX];
+    if (threads > 0) k_onee_gather<<<(unsigned)((threads + 127) / 128), 128, 0, a.st>>>(a.pl, ib, gsz, a.blk, a.Out);
 }
 
 // sign (8 pi w(G) / V)^{pw/2} (Re, Im) of rho_N(G) = sum_C Z_C e^{-iG.C}, one
@@ -473,7 +507,7 @@ int one_electron(Plan *P, int natom, const double *Z, const double *xyz, double 
         a.ab = P->d_ppi_ab;
         a.Out = w.T1;
         launch_onee(P, a, 0);
-        launch_onee(P, a, 3);
+        launch_gather(P, a);
         k_onee_final<<<grid, 256, 0, st>>>(n, P->d_compf, w.T1, P->d_S, 0.0, T);
         if (!ok(cudaGetLastError()) || !good) {
             release();
@@ -571,9 +605,9 @@ int one_electron(Plan *P, int natom, const double *Z, const double *xyz, double 
             launch_gauss_table(P, g0, a.gcur, const_cast<double *>(a.gtab), st);
             launch_onee(P, a, 2);
         }
-        launch_onee(P, a, 3);
+        launch_gather(P, a);
     } else {
-        launch_onee(P, a, 3);
+        launch_gather(P, a);
         for (int g0 = 0; g0 < ng; g0 += w.gc) {
             const int gcur = std::min(w.gc, ng - g0);
             launch_gauss_table(P, g0, gcur, w.gtab, st);
