@@ -648,7 +648,7 @@ int run_build(Plan *P, const double *D, double *J, double *K, cudaStream_t st)
 // over the whole class where that takes less than about a second.  A candidate
 // replaces the untuned schedule only if it is faster by 2%: the sub-ranges alone
 // preferred few kets per warp, and the 64-water tiles so tuned took 389 ms
-// against 350 untuned.  Results are cached in a text file (one line per GPU
+// against 354 untuned.  Results are cached in a text file (one line per GPU
 // name, precision, class pair and size bucket: family * 65536 + kets, or 0
 // where the untuned schedule stays) when cache_path is given.
 int autotune(Plan *P, const double *D, cudaStream_t st, const char *cache_path, int *chosen)

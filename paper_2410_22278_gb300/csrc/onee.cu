@@ -499,8 +499,10 @@ int one_electron(Plan *P, int natom, const double *Z, const double *xyz, double 
     a.st = st;
     a.blk = w.Z;
     if (!inside && !ok(cudaMallocAsync((void **)&a.blk, nblk * sizeof(double), st))) return fail_cuda(JK_ERR_OOM, "one-electron scratch");
-    const auto release = [&] {
+    // end of the call on any path: the scratch goes back and the stream is waited for
+    const auto finish = [&] {
         if (!inside) cudaFreeAsync(a.blk, st);
+        return ok(cudaStreamSynchronize(st));
     };
     if (T) {
         bool good = ok(cudaMemsetAsync(w.T1, 0, n2 * sizeof(double), st));
@@ -510,14 +512,11 @@ int one_electron(Plan *P, int natom, const double *Z, const double *xyz, double 
         launch_gather(P, a);
         k_onee_final<<<grid, 256, 0, st>>>(n, P->d_compf, w.T1, P->d_S, 0.0, T);
         if (!ok(cudaGetLastError()) || !good) {
-            release();
+            finish();
             return fail_cuda(JK_ERR_CUDA, "kinetic-energy kernels failed");
         }
     }
-    if (!V || natom <= 0) {
-        release();
-        return ok(cudaStreamSynchronize(st)) ? JK_OK : fail_cuda(JK_ERR_CUDA, "one-electron kernels failed");
-    }
+    if (!V || natom <= 0) return finish() ? JK_OK : fail_cuda(JK_ERR_CUDA, "one-electron kernels failed");
 
     // lattice candidates for the charges' images: |R| up to the largest
     // screening radius plus the cell's circumradius (the reduced X0 is at
@@ -571,7 +570,7 @@ int one_electron(Plan *P, int natom, const double *Z, const double *xyz, double 
     const size_t oX = ((size_t)natom + 1) / 2 * 2, oC = oX + (3 * (size_t)natom + 1) / 2 * 2, oN = oC + 4 * (size_t)std::max(1, ncand);
     double *dZ = nullptr;
     if (!ok(cudaMallocAsync((void **)&dZ, sizeof(double) * (oN + 2 * (size_t)std::max(1, ng)), st))) {
-        release();
+        finish();
         return fail_cuda(JK_ERR_OOM, "one-electron scratch");
     }
     double *dX = dZ + oX, *dC = dZ + oC;
@@ -620,10 +619,8 @@ int one_electron(Plan *P, int natom, const double *Z, const double *xyz, double 
     // self term +(pi/(V w^2)) Z_tot S and the component factors
     k_onee_final<<<grid, 256, 0, st>>>(n, P->d_compf, w.T2, P->d_S, kPi / (P->volume * w2) * ztot, V);
     cudaFreeAsync(dZ, st);
-    release();
-    // waited for on every path: the copies above read the caller's host arrays
     good = ok(cudaGetLastError()) && good;
-    good = ok(cudaStreamSynchronize(st)) && good;
+    good = finish() && good;  // also where a launch failed: the copies above read the caller's host arrays
     return good ? JK_OK : fail_cuda(JK_ERR_CUDA, "nuclear-attraction kernels failed");
 }
 

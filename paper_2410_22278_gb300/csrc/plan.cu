@@ -412,26 +412,26 @@ static int upload(const std::vector<T> &h, T **d, size_t &bytes)
     return JK_OK;
 }
 
-// Lists of large quartets of a mixed plan.  The FP64 share is a small fraction:
-// a list holds up to 2% of all image quartets of the plan (at least 1 Mi, at
-// most 64 Mi), and never more than its class pair has.  A class pair's list is
-// in use from its tile kernel to its list pass, so each lane of the real-space
-// phase needs one; the l-th lane's holds the l-th largest class pair, and a
-// class pair only goes to a lane that can hold it (run_build).  As many lanes as
-// fit the bytes of one list of 8-byte entries and `spare` more, what the rest of
-// the workspace does without: a plan with side streams asks for no more than one
-// without did (a server admits plans by their workspace).
-static void quartet_lists(Plan *P, long long spare, size_t &bytes)
+// Capacities that the lists of large quartets of a mixed plan have to have,
+// largest first.  The FP64 share is a small fraction: a list holds up to 2% of
+// all image quartets of the plan (at least 1 Mi, at most 64 Mi: cap), and never
+// more than its class pair has.
+static std::vector<long long> list_needs(const Plan *P, long long cap)
 {
-    Workspace &w = P->ws;
-    const long long cap = std::min<long long>(std::max<long long>(P->n_quartets / 50, 1 << 20), 64ll << 20);
     std::vector<long long> need;
     for (int i = 0; i < JK_NCLASS_MAX; ++i)
         for (int j = i; j < JK_NCLASS_MAX; ++j) need.push_back(std::min(cap, P->class_quartets(i, j)));
     std::sort(need.rbegin(), need.rend());
-    const bool narrow = P->spi.size() <= 65536;
-    w.list_elt = narrow ? sizeof(unsigned) : sizeof(int2);
-    const long long fit = cap * (long long)sizeof(int2) + spare;
+    return need;
+}
+
+// The lists, of `fit` bytes at most if there are several.  A class pair's list
+// is in use from its tile kernel to its list pass, so each lane of the
+// real-space phase needs one; the l-th lane's holds the l-th largest class pair,
+// and a class pair only goes to a lane that can hold it (run_build).
+static void quartet_lists(Plan *P, std::vector<long long> need, long long fit, size_t &bytes)
+{
+    Workspace &w = P->ws;
     static_assert(Workspace::kLists >= Plan::kSide, "a list per lane");
     w.nlist = std::max(1, P->nside);
     const auto total = [&] { return std::accumulate(need.begin(), need.begin() + w.nlist, 0LL) * (long long)w.list_elt; };
@@ -464,6 +464,35 @@ static int alloc_ws(Plan *P)
     long long gc = (long long)(budget / per_g);
     gc = std::max<long long>(1, std::min<long long>(gc, std::max(ng, 1)));
     gc = std::min<long long>(gc, 4096);
+    // J-engine arrays: stride N_H(2 lmax); only plans with d shells use them
+    int lmax = 0;
+    for (auto &sh : P->shells) lmax = std::max(lmax, sh.l);
+    w.hs = (2 * lmax + 1) * (2 * lmax + 2) * (2 * lmax + 3) / 6;
+    size_t nh = std::max<size_t>(1, P->ppi.size()) * w.hs;
+    // Bytes of the lists of large quartets: a plan with a list for each lane
+    // takes no more workspace than one with a single list of 8-byte entries did
+    // (a server admits plans by it).  What that one had besides were partial sums
+    // for the largest split of every slab, J-engine arrays without a use and a
+    // second Gaussian table (less a few words for the counters of the lists);
+    // if that is not enough for lanes that hold any class pair, the G chunk
+    // gives up a few of its vectors (one diamond cell at omega 0.4: four of 293;
+    // with three lanes its builds took 20% longer).
+    long long fit = 0;
+    std::vector<long long> need;
+    if (mixed) {
+        const long long cap = std::min<long long>(std::max<long long>(P->n_quartets / 50, 1 << 20), 64ll << 20);
+        need = list_needs(P, cap);
+        w.list_elt = P->spi.size() <= 65536 ? sizeof(unsigned) : sizeof(int2);
+        fit = cap * (long long)sizeof(int2) + (2 * gc * kSlabSplitsMax - slab_part_size(2 * (int)gc) - 16) * (long long)sizeof(double) +
+              (long long)std::max<size_t>(1, P->pvals.size()) * gc * (long long)sizeof(float2) + (lmax < 2 ? (long long)(nh - 1) * 20 : 0);
+        const double lacking = (double)(P->nside * need[0]) * w.list_elt - (double)fit;
+        const long long cut = lacking > 0 ? (long long)(lacking / per_g) + 1 : 0;
+        if (cut <= gc / 16) {
+            gc -= cut;
+            fit += (long long)(cut * per_g);
+        }
+    }
+    if (lmax < 2) nh = 1;
     w.gc = (int)gc;
     if (mixed && ng > 0) {
         // Slices per G chunk.  With balanced 8-bit digits the split-precision
@@ -492,27 +521,11 @@ static int alloc_ws(Plan *P)
         bytes += std::max<size_t>(count, 1) * sizeof(double);
         return true;
     };
-    // What the plan takes less of than one with partial sums for the largest
-    // split of every slab, J-engine arrays without a use and a second Gaussian
-    // table (less a few words for the counters of the lists).
-    long long spare = (2LL * gc * kSlabSplitsMax - slab_part_size(2 * (int)gc) - 8) * (long long)sizeof(double);
     bool ok = al(&w.gtab, std::max<size_t>(1, P->pvals.size()) * (size_t)gc) && al(&w.Dp, n2) && al(&w.X, n2) && al(&w.Y, n2) && al(&w.JLR, n2) && al(&w.KLR, n2) && al(&w.T1, n2) &&
               al(&w.T2, n2) && al(&w.M, 2 * (size_t)gc * n2) && al(&w.Z, 2 * (size_t)gc * n2) && al(&w.rho, 2 * (size_t)gc) && al(&w.rho_part, slab_part_size(2 * (int)gc)) &&
               al(&w.dmax, (size_t)P->nshell * P->nshell) && al(&w.scal, 16) && (!mixed || al((double **)&w.Dpf, (n2 + 1) / 2)) &&
               (!mixed || al((double **)&w.dmaxf, ((size_t)P->nshell * P->nshell + 2) / 2));
-    {
-        // J-engine arrays: stride N_H(2 lmax); only plans with d shells use them
-        int lmax = 0;
-        for (auto &sh : P->shells) lmax = std::max(lmax, sh.l);
-        const int L2 = 2 * lmax;
-        w.hs = (L2 + 1) * (L2 + 2) * (L2 + 3) / 6;
-        size_t nh = std::max<size_t>(1, P->ppi.size()) * w.hs;
-        if (lmax < 2) {
-            spare += (long long)(nh - 1) * 20;
-            nh = 1;
-        }
-        ok = ok && al(&w.DhD, nh) && al(&w.JH, nh) && al((double **)&w.DhF, (nh + 1) / 2);
-    }
+    ok = ok && al(&w.DhD, nh) && al(&w.JH, nh) && al((double **)&w.DhF, (nh + 1) / 2);
     if (!ok) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed for build workspace");
     // the structure-factor kernels write only the entries of shell pairs with
     // images, the same ones for every G; the others must read as zero
@@ -532,7 +545,6 @@ static int alloc_ws(Plan *P)
             return true;
         };
         w.gtab2 = reinterpret_cast<float2 *>(w.gtab);
-        spare += (long long)std::max<size_t>(1, P->pvals.size()) * gc * (long long)sizeof(float2);
         if (!alb(&w.Ms, 2 * (size_t)gc * sl) || !alb(&w.Zs, 2 * (size_t)gc * sl) || !alb(&w.Ds, sl) || !alb(&w.Cs, sl) ||
             !ali(&w.Mex, 2 * (size_t)gc * w.npad) || !ali(&w.Zex, 2 * (size_t)gc * w.npad) || !ali(&w.Dex, w.npad) ||
             !ali(&w.Cex, w.npad))
@@ -551,7 +563,7 @@ static int alloc_ws(Plan *P)
     if (cudaMalloc((void **)&w.cnt, kCounters * sizeof(unsigned long long)) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed");
     if (P->precision == JK_MIXED) {
         size_t lb = 0;
-        quartet_lists(P, spare, lb);
+        quartet_lists(P, need, fit, lb);
         if (cudaMalloc((void **)&w.big, lb) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed for quartet list");
         if (cudaMalloc((void **)&w.nbig, 2 * sizeof(unsigned) * w.nlist) != cudaSuccess) return fail_cuda(JK_ERR_OOM, "cudaMalloc failed");
         bytes += lb + 2 * sizeof(unsigned) * w.nlist;

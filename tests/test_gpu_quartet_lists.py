@@ -19,6 +19,7 @@ CELLS = {
     "skewed_spd": (lambda: sc.small_random_cell(1, natom=2, lmax=2, skew=True), 382144468),
     "water5": (lambda: sc.water_cell(5, (29.94 * 5) ** (1.0 / 3.0), n_occ=20), 627094200),
     "diamond1": (lambda: sc.diamond_cell(1), 499547580),
+    "diamond1_soft": (lambda: sc.diamond_cell(1, omega=0.4), 288255684),  # the G chunk gives up four vectors
 }
 
 
