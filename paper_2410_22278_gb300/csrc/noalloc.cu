@@ -126,13 +126,22 @@ int energy_noalloc(const Plan *P, const double *D, const double *J, const double
     if (rc) return rc;
     const long long per_block = std::max(kEnergyMinPerBlock, (n2 + kEnergyBlocks - 1) / kEnergyBlocks);
     const int nblk = (int)std::max(1LL, (n2 + per_block - 1) / per_block);  // <= kEnergyBlocks
-    k_energy_partials<<<nblk, kEnergyThreads, 0, st>>>(n2, per_block, D, J, K, scratch);
-    k_energy_final<<<1, kEnergyThreads, 0, st>>>(nblk, scratch);
-    if (cudaGetLastError() != cudaSuccess) return fail(JK_ERR_CUDA, "jk_energy_noalloc: launch failed");
+    // judged by the status of these launches, not by an error that an earlier
+    // call left in this thread; the stream is waited for on every path, since
+    // the kernels read the caller's matrices and write the shared scratch
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(nblk);
+    cfg.blockDim = dim3(kEnergyThreads);
+    cfg.stream = st;
+    bool launched = cudaLaunchKernelEx(&cfg, k_energy_partials, n2, per_block, D, J, K, scratch) == cudaSuccess;
+    cfg.gridDim = dim3(1);
+    launched = launched && cudaLaunchKernelEx(&cfg, k_energy_final, nblk, scratch) == cudaSuccess;
     double h[2] = {0, 0};
-    if (cudaMemcpyAsync(h, scratch + 2 * kEnergyBlocks, sizeof h, cudaMemcpyDeviceToHost, st) != cudaSuccess)
-        return fail(JK_ERR_CUDA, "jk_energy_noalloc: copy of the result failed");
-    if (cudaStreamSynchronize(st) != cudaSuccess) return fail(JK_ERR_CUDA, "jk_energy_noalloc: reduction failed");
+    const bool copied = launched && cudaMemcpyAsync(h, scratch + 2 * kEnergyBlocks, sizeof h, cudaMemcpyDeviceToHost, st) == cudaSuccess;
+    const bool done = cudaStreamSynchronize(st) == cudaSuccess;
+    if (!launched) return fail_cuda(JK_ERR_CUDA, "jk_energy_noalloc: launch failed");
+    if (!copied) return fail_cuda(JK_ERR_CUDA, "jk_energy_noalloc: copy of the result failed");
+    if (!done) return fail_cuda(JK_ERR_CUDA, "jk_energy_noalloc: reduction failed");
     *e_coul = h[0];
     *e_exch = h[1];
     return JK_OK;

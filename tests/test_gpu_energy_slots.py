@@ -69,6 +69,19 @@ def test_error_of_an_earlier_call(jk, plan):
     assert max(abs(got[0] - want[0]), abs(got[1] - want[1])) < TOL
 
 
+def test_error_of_an_earlier_call_without_allocation(jk, plan):
+    D, J, K = matrices(plan.nbf, 2)
+    want = expected(D, J, K)
+    st = torch.cuda.current_stream().cuda_stream
+    torch.cuda.synchronize()
+    leave_error()
+    try:
+        got = plan.energy_noalloc(D.data_ptr(), J.data_ptr(), K.data_ptr(), st)
+    finally:
+        clear_error()
+    assert max(abs(got[0] - want[0]), abs(got[1] - want[1])) < TOL
+
+
 def test_threads_with_and_without_one(jk, plan):
     data = [matrices(plan.nbf, 10 + s) for s in range(6)]
     want = [expected(*d) for d in data]
